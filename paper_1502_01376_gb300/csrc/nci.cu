@@ -4,7 +4,7 @@
 // [k]E1 = [k]B1 = k1 (plus the Sec. 4 bump), [k]E2 = [k]B2 =
 // sin(k2 dx2/2)/(dx2/2), and the cubic Eq. asym1 about the beam resonance).
 //
-// One thread per (sample, alias).  The roots sought are all zeros of
+// The roots sought for a (sample, alias) are all zeros of
 //   G(w) = [w] D(w) (w' - k1' v0)
 // (the relation times the factors that remove its poles: G is entire) in the
 // disk |w - w_res| < rho about the beam resonance w' = k1' v0, with
@@ -23,6 +23,17 @@
 //     into four pieces whose zeros are counted by their boundary's winding,
 //     recursively, and Newton's method is run inside each piece that holds
 //     one zero (complete by construction).
+//
+// A warp takes a group of up to 32 (sample, alias) pairs.  The FP64 pipe bounds
+// it (a warp-wide FP64 instruction occupies it for the same time with one live
+// lane or with 32), so the work is laid out to keep lanes live: the windings
+// with the contour's points across the lanes, one pair after the other; the
+// cubic's and the resonance's seeds with one pair per lane; the ring seeds and
+// the subdivision, which few pairs need but each for a long time, again one pair
+// at a time with seeds and contour points across the lanes.  With one thread per
+// pair doing all of it (before), the few hard pairs ran alone for tens of
+// milliseconds, 3.6 of 32 lanes live: 69 ms for 32256 samples x 3 aliases, 7.1 ms now, of which
+// the counts take a third and the cubic's seeds most of the rest.
 //
 // Readings (the printed forms are garbled here): s_{l,i} = sinc(k'_i dx_i/2)^(l+1)
 // with k' aliased; S_B3 = S'_B3 cos(w dt/2), B's time centring, whose
@@ -56,9 +67,26 @@ __device__ __forceinline__ double dsinc(double x) { return x == 0.0 ? 1.0 : sin(
 
 // The symbols of one (sample, alias).
 struct NciMode {
-    double h, v0, a, b, wg, k1a, kE1, kE2, k2, SE1, SE2, SB3s, Sj1, Sj2;
-    int mu;
+    double h, rh, v0, b, muwg, res, kE1, kE2, k2, SE1, SE2, SB3s, Sj1, Sj2;
+    double K2, as, sb, sk, c1, c2, c3, c4;      // the products G uses (see nci_G)
+    double c, sc, cc;                           // the resonance, sin(c h), cos(c h)
 };
+
+// SIGN = -1: sin x and cos x, SIGN = 1: sinh x and cosh x, by Taylor series for |x| <= 1/2
+template <int SIGN>
+__device__ __forceinline__ void taylor_trig(double x, double* s, double* c) {
+    const double z = SIGN * x * x;
+    double a = 1.0 / 1307674368000.0, b = 1.0 / 20922789888000.0;      // 1/15!, 1/16!
+    a = fma(a, z, 1.0 / 6227020800.0);  b = fma(b, z, 1.0 / 87178291200.0);
+    a = fma(a, z, 1.0 / 39916800.0);    b = fma(b, z, 1.0 / 479001600.0);
+    a = fma(a, z, 1.0 / 362880.0);      b = fma(b, z, 1.0 / 3628800.0);
+    a = fma(a, z, 1.0 / 5040.0);        b = fma(b, z, 1.0 / 40320.0);
+    a = fma(a, z, 1.0 / 120.0);         b = fma(b, z, 1.0 / 720.0);
+    a = fma(a, z, 1.0 / 6.0);           b = fma(b, z, 1.0 / 24.0);
+    b = fma(b, z, 0.5);
+    *s = fma(a * z, x, x);
+    *c = fma(b, z, 1.0);
+}
 
 // G(w) and G'(w).  With u = w h (h = dt/2): [w] = sin(u)/h, c = cos(u) (B's time
 // centring), d[w]/dw = c, dc/dw = -h sin(u) = -h^2 [w].
@@ -67,74 +95,119 @@ struct NciMode {
 //   C = b (Sj1 SE1 w' kE2^2 (v0^2 - 1) + Sj2 SE2 kE2^2 Delta
 //          + Sj1 kE2 k2 (SE2 kE1 v0 - SB3 v0^2 [w]))                  ([w] x coupling term)
 //   G = A S + C Delta,  SB3 = SB3s c.
-__device__ void nci_G(const NciMode& m, Z w, Z* g, Z* dg) {
-    double su, cu;
-    sincos(w.re * m.h, &su, &cu);
-    const double ch = cosh(w.im * m.h), sh = sinh(w.im * m.h);
+template <bool DERIV>
+__device__ __forceinline__ void nci_G(const NciMode& m, Z w, Z* g, Z* dg) {
+    // sin and cos of Re w h = c h + d and sinh and cosh of y = Im w h.  Near the resonance (|d|, |y| <=
+    // 1/2: the disk, as long as rho h <= 1/2) from their Taylor series (to x^15 and x^16: the first
+    // term left out is below 1e-18) and the addition theorem, about a third of the FP64 instructions of
+    // the calls elsewhere
+    double su, cu, sh, ch;
+    const double d = (w.re - m.c) * m.h, y = w.im * m.h;
+    if (fabs(d) <= 0.5 && fabs(y) <= 0.5) {
+        double sd, cd;
+        taylor_trig<-1>(d, &sd, &cd);
+        taylor_trig<1>(y, &sh, &ch);
+        su = m.sc * cd + m.cc * sd;
+        cu = m.cc * cd - m.sc * sd;
+    } else {
+        sincos(w.re * m.h, &su, &cu);
+        sh = sinh(y);
+        ch = cosh(y);
+    }
     const Z sn = zc(su * ch, cu * sh);                  // sin(w h)
     const Z cs = zc(cu * ch, -su * sh);                 // cos(w h)
-    const Z wb = zsc(sn, 1.0 / m.h);
-    const Z dwb = cs;
-    const Z dcs = zsc(sn, -m.h);
-    const Z wp = zc(w.re + m.mu * m.wg, w.im);
-    const Z D = zc(wp.re - m.k1a * m.v0, wp.im);        // Delta; dDelta/dw = 1, dw'/dw = 1
-    const double K2 = m.kE1 * m.kE1 + m.kE2 * m.kE2, kE2s = m.kE2 * m.kE2;
+    const Z wb = zsc(sn, m.rh);
+    const Z wp = zc(w.re + m.muwg, w.im);
+    const Z D = zc(wp.re - m.res, wp.im);               // Delta; dDelta/dw = 1, dw'/dw = 1
     const Z D2 = zmul(D, D);
-    // A and A'
-    const Z A = zsub(zmul(wb, D2), zsc(wp, m.a * m.Sj1 * m.SE1));
-    const Z dA = zsub(zadd(zmul(dwb, D2), zsc(zmul(wb, D), 2.0)), zc(m.a * m.Sj1 * m.SE1, 0.0));
-    // S and S'
-    const Z wb2K = zsub(zmul(wb, wb), zc(K2, 0.0));
-    const double sb = m.b * m.Sj2;
-    const Z S = zsub(zmul(wb2K, D), zsc(zsub(zsc(wb, m.SE2), zsc(cs, m.SB3s * m.kE1 * m.v0)), sb));
-    const Z dS = zsub(zadd(zsc(zmul(zmul(wb, dwb), D), 2.0), wb2K),
-                      zsc(zsub(zsc(dwb, m.SE2), zsc(dcs, m.SB3s * m.kE1 * m.v0)), sb));
-    // C and C'
-    const double c1 = m.b * m.Sj1 * m.SE1 * kE2s * (m.v0 * m.v0 - 1.0);
-    const double c2 = m.b * m.Sj2 * m.SE2 * kE2s;
-    const double c3 = m.b * m.Sj1 * m.kE2 * m.k2 * m.SE2 * m.kE1 * m.v0;
-    const double c4 = m.b * m.Sj1 * m.kE2 * m.k2 * m.SB3s * m.v0 * m.v0;
-    const Z C = zsub(zadd(zadd(zsc(wp, c1), zsc(D, c2)), zc(c3, 0.0)), zsc(zmul(cs, wb), c4));
-    const Z dC = zsub(zc(c1 + c2, 0.0), zsc(zadd(zmul(dcs, wb), zmul(cs, dwb)), c4));
+    const Z A = zsub(zmul(wb, D2), zsc(wp, m.as));
+    const Z wb2K = zsub(zmul(wb, wb), zc(m.K2, 0.0));
+    const Z S = zsub(zmul(wb2K, D), zsc(zsub(zsc(wb, m.SE2), zsc(cs, m.sk)), m.sb));
+    const Z C = zsub(zadd(zadd(zsc(wp, m.c1), zsc(D, m.c2)), zc(m.c3, 0.0)), zsc(zmul(cs, wb), m.c4));
     *g = zadd(zmul(A, S), zmul(C, D));
-    if (dg) *dg = zadd(zadd(zadd(zmul(dA, S), zmul(A, dS)), zmul(dC, D)), C);
+    if (DERIV) {
+        const Z dcs = zsc(sn, -m.h);
+        const Z dA = zsub(zadd(zmul(cs, D2), zsc(zmul(wb, D), 2.0)), zc(m.as, 0.0));
+        const Z dS = zsub(zadd(zsc(zmul(zmul(wb, cs), D), 2.0), wb2K), zsc(zsub(zsc(cs, m.SE2), zsc(dcs, m.sk)), m.sb));
+        const Z dC = zsub(zc(m.c1 + m.c2, 0.0), zsc(zadd(zmul(dcs, wb), zmul(cs, cs)), m.c4));
+        *dg = zadd(zadd(zadd(zmul(dA, S), zmul(A, dS)), zmul(dC, D)), C);
+    }
 }
 
 // Winding number of G along a closed polyline given by point(i), i = 0..n (point(n) =
 // point(0)), with the number of points raised until no phase step exceeds 0.5 rad.
 // Returns -1 if no sampling up to kMaxWind points resolves it (a zero on the path).
+// Called by the whole warp with one mode: the lanes take consecutive points, 32 at a time.
+// A step from g0 to g1 is below 0.5 rad when Re(g1 conj g0) > 0 and |Im| <= tan(0.5) Re; the
+// steps' sum over 2 pi is the signed number of crossings of the negative real axis, which such a
+// step makes exactly when Im g changes sign at Re g < 0 (no arc tangent needed).
 constexpr int kMaxWind = 1 << 13;
 template <typename Path>
 __device__ int winding(const NciMode& m, Path path, int n0) {
+    constexpr double kTan = 0.54630248984379051326;      // tan(0.5)
+    const int lane = threadIdx.x & 31;
     for (int n = n0; n <= kMaxWind; n *= 4) {
-        Z g0;
-        nci_G(m, path(0, n), &g0, nullptr);
-        const Z gs = g0;
-        double tot = 0.0;
-        bool ok = true;
-        for (int i = 1; i <= n && ok; i++) {
-            Z g1;
-            if (i == n) g1 = gs;
-            else nci_G(m, path(i, n), &g1, nullptr);
-            // arg(g1 / g0) = atan2(Im(g1 conj g0), Re(g1 conj g0))
-            const double re = g1.re * g0.re + g1.im * g0.im, im = g1.im * g0.re - g1.re * g0.im;
-            if (re == 0.0 && im == 0.0) { ok = false; break; }
-            const double d = atan2(im, re);
-            if (fabs(d) > 0.5) ok = false;
-            tot += d;
-            g0 = g1;
+        Z first = zc(0.0, 0.0), last = zc(0.0, 0.0);
+        int cross = 0;
+        bool ok = true, undefined = false;
+        for (int i0 = 0; i0 <= n && ok; i0 += 32) {
+            const int i = i0 + lane;
+            Z g = first;                                  // point n is point 0
+            if (i0 < n) nci_G<false>(m, path(i, n), &g, nullptr);
+            Z p = zc(__shfl_up_sync(0xffffffffu, g.re, 1), __shfl_up_sync(0xffffffffu, g.im, 1));
+            if (lane == 0) p = last;
+            bool bad = false, nan = false;
+            if (i0 + lane > 0 && i0 + lane <= n) {
+                const double re = g.re * p.re + g.im * p.im, im = g.im * p.re - g.re * p.im;
+                nan = isnan(re) || isnan(im);
+                bad = !nan && !(re > 0.0 && fabs(im) <= kTan * re);
+                if (p.re < 0.0) cross += (p.im >= 0.0 && g.im < 0.0) ? 1 : (p.im < 0.0 && g.im >= 0.0) ? -1 : 0;
+            }
+            ok = !__any_sync(0xffffffffu, bad);
+            undefined = undefined || __any_sync(0xffffffffu, nan);
+            if (i0 == 0) first = zc(__shfl_sync(0xffffffffu, g.re, 0), __shfl_sync(0xffffffffu, g.im, 0));
+            last = zc(__shfl_sync(0xffffffffu, g.re, 31), __shfl_sync(0xffffffffu, g.im, 31));
         }
-        if (ok) return (int)llround(tot / (2.0 * 3.14159265358979323846));
+        if (ok) return undefined ? 0 : __reduce_add_sync(0xffffffffu, cross);
     }
     return -1;
 }
 
-__device__ int winding_circle(const NciMode& m, Z c, double r) {
-    return winding(m, [&](int i, int n) {
-        double s, co;
-        sincospi(2.0 * (double)i / (double)n, &s, &co);
-        return zc(c.re + r * co, c.im + r * s);
-    }, 64);
+// The same along a circle about a point c of the real axis.  G is real there (its coefficients are
+// real), so G(conj w) = conj G(w) and only the points i = 0..n/2 of the upper half are evaluated;
+// each step counts with its mirror step.  (zx, zy): cos and sin of the lane's point for n = 64;
+// end: G(c - r), the point n/2.
+__device__ int winding_circle(const NciMode& m, double c, double r, double zx, double zy, Z end) {
+    constexpr double kTan = 0.54630248984379051326;
+    const int lane = threadIdx.x & 31;
+    for (int n = 64; n <= kMaxWind; n *= 4) {
+        Z last = zc(0.0, 0.0);
+        int cross = 0;
+        bool ok = true, undefined = false;
+        for (int i0 = 0; i0 < n / 2 && ok; i0 += 32) {
+            if (n > 64) sincospi(2.0 * (i0 + lane) / (double)n, &zy, &zx);
+            Z g;
+            nci_G<false>(m, zc(c + r * zx, r * zy), &g, nullptr);
+            bool bad = false, nan = false;
+            auto step = [&](Z a, Z b) {                               // from a to b, and from conj b to conj a
+                const double re = b.re * a.re + b.im * a.im, im = b.im * a.re - b.re * a.im;
+                const bool undef = isnan(re) || isnan(im);
+                nan |= undef;
+                bad |= !undef && !(re > 0.0 && fabs(im) <= kTan * re);
+                if (a.re < 0.0) cross += (a.im >= 0.0 && b.im < 0.0) ? 1 : (a.im < 0.0 && b.im >= 0.0) ? -1 : 0;
+                if (b.re < 0.0) cross += (-b.im >= 0.0 && -a.im < 0.0) ? 1 : (-b.im < 0.0 && -a.im >= 0.0) ? -1 : 0;
+            };
+            Z p = zc(__shfl_up_sync(0xffffffffu, g.re, 1), __shfl_up_sync(0xffffffffu, g.im, 1));
+            if (lane == 0) p = last;
+            if (i0 + lane > 0) step(p, g);
+            if (i0 + 32 == n / 2 && lane == 31) step(g, end);
+            ok = !__any_sync(0xffffffffu, bad);
+            undefined = undefined || __any_sync(0xffffffffu, nan);
+            last = zc(__shfl_sync(0xffffffffu, g.re, 31), __shfl_sync(0xffffffffu, g.im, 31));
+        }
+        if (ok) return undefined ? 0 : __reduce_add_sync(0xffffffffu, cross);
+    }
+    return -1;
 }
 __device__ int winding_rect(const NciMode& m, double x0, double x1, double y0, double y1) {
     return winding(m, [&](int i, int n) {
@@ -144,26 +217,45 @@ __device__ int winding_rect(const NciMode& m, double x0, double x1, double y0, d
         if (e == 0) return zc(x0 + (x1 - x0) * t, y0);
         if (e == 1) return zc(x1, y0 + (y1 - y0) * t);
         if (e == 2) return zc(x1 - (x1 - x0) * t, y1);
-        if (e == 3) return zc(x0, y1 - (y1 - y0) * t);
-        return zc(x0, y0);
+        return zc(x0, y1 - (y1 - y0) * t);
     }, 128);
 }
 
-// Newton's method on G deflated by the nf zeros in r[]; true if it converges to w.
-__device__ bool newton_deflated(const NciMode& m, Z w, const Z* r, int nf, Z* out) {
-    for (int it = 0; it < 80; it++) {
-        Z g, dg;
-        nci_G(m, w, &g, &dg);
-        if (g.re == 0.0 && g.im == 0.0) { *out = w; return true; }
-        Z q = zdiv(dg, g);                               // G'/G
-        for (int j = 0; j < nf; j++) q = zsub(q, zdiv(zc(1.0, 0.0), zsub(w, r[j])));
-        if (q.re == 0.0 && q.im == 0.0) return false;
-        const Z step = zdiv(zc(1.0, 0.0), q);
-        w = zsub(w, step);
-        if (!(isfinite(w.re) && isfinite(w.im))) return false;
-        if (zabs(step) <= 1e-14 * fmax(1.0, zabs(w))) { *out = w; return true; }
+// One attempt of Newton's method on G deflated by the nf zeros in r[], advanced one step per call:
+// 0 = go on, 1 = converged to w, -1 = failed.  An attempt has kNewtonMax steps.  Each step is a
+// function of w alone, so an attempt that meets a w it has seen (kept at steps 1, 2, 4, 8, ...:
+// a limit cycle at rounding level) can never converge and fails at once.
+constexpr int kNewtonMax = 80;
+struct Newton { Z w, seen; int it; };
+__device__ __forceinline__ Newton newton_start(Z w) { return Newton{w, zc(nan(""), 0.0), 0}; }
+__device__ __forceinline__ int newton_step(const NciMode& m, Newton& s, const Z* r, int nf) {
+    Z g, dg;
+    nci_G<true>(m, s.w, &g, &dg);
+    if (g.re == 0.0 && g.im == 0.0) return 1;
+    // step = 1 / (G'/G - sum 1/(w - r_j)) = G / (G' - G sum)
+    Z sum = zc(0.0, 0.0);
+    for (int j = 0; j < nf; j++) {
+        const Z d = zsub(s.w, r[j]);
+        const double q = 1.0 / (d.re * d.re + d.im * d.im);
+        sum = zc(sum.re + d.re * q, sum.im - d.im * q);
     }
-    return false;
+    const Z den = zsub(dg, zmul(g, sum));
+    if (den.re == 0.0 && den.im == 0.0) return -1;
+    const Z step = zdiv(g, den);
+    s.w = zsub(s.w, step);
+    if (!(isfinite(s.w.re) && isfinite(s.w.im))) return -1;
+    // |step| <= 1e-14 max(1, |w|)
+    if (step.re * step.re + step.im * step.im <= 1e-28 * fmax(1.0, s.w.re * s.w.re + s.w.im * s.w.im)) return 1;
+    if (++s.it == kNewtonMax || (s.w.re == s.seen.re && s.w.im == s.seen.im)) return -1;
+    if ((s.it & (s.it - 1)) == 0) s.seen = s.w;
+    return 0;
+}
+__device__ bool newton_deflated(const NciMode& m, Z w, const Z* r, int nf, Z* out) {
+    Newton s = newton_start(w);
+    int st;
+    while ((st = newton_step(m, s, r, nf)) == 0) {}
+    *out = s.w;
+    return st > 0;
 }
 
 // Plain Newton's method for one zero inside a rectangle.
@@ -229,27 +321,21 @@ __device__ double k_eff(const NciSample& s) {
 // error bits of k_nci (the kernel's *err)
 enum : int { NCI_ETOOMANY = 1, NCI_EUNRESOLVED = 2 };
 
-__global__ void k_nci(const NciSample* __restrict__ smp, int64_t n, int order, int correct_j1,
-                      const int* __restrict__ alias, int n_alias, double* __restrict__ growth, double2* __restrict__ root,
-                      int max_out, double2* __restrict__ roots_out, int* __restrict__ count_out, int* __restrict__ err) {
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (tid >= n * n_alias) return;
-    const int64_t i = tid / n_alias;
-    const int ai = (int)(tid % n_alias);
-    const NciSample s = smp[i];
+// the symbols of a pair, its resonance c (real) and the disk's radius
+__device__ void nci_symbols(const NciSample& s, int mu, int nu1, int order, int correct_j1, NciMode& m, double* c, double* rho,
+                            double* k1a_out) {
     const double pi = 3.14159265358979323846;
-    NciMode m;
     m.h = 0.5 * s.dt;
+    m.rh = 1.0 / m.h;
     m.v0 = sqrt(1.0 - 1.0 / (s.gamma * s.gamma));
-    m.mu = alias[2 * ai];
-    const int nu1 = alias[2 * ai + 1];
-    m.wg = 2.0 * pi / s.dt;
-    const double sgnmu = (m.mu & 1) ? -1.0 : 1.0;
-    m.a = s.wp2 / (s.gamma * s.gamma * s.gamma) * sgnmu;
+    const double wg = 2.0 * pi / s.dt;
+    m.muwg = mu * wg;
+    const double sgnmu = (mu & 1) ? -1.0 : 1.0;
+    const double a = s.wp2 / (s.gamma * s.gamma * s.gamma) * sgnmu;
     m.b = s.wp2 / s.gamma * sgnmu;
     m.k2 = s.k2;
-    m.k1a = s.k1 + nu1 * 2.0 * pi / s.dx1;
-    const double s1 = dsinc(0.5 * m.k1a * s.dx1), s2 = dsinc(0.5 * s.k2 * s.dx2);
+    const double k1a = s.k1 + nu1 * 2.0 * pi / s.dx1;
+    const double s1 = dsinc(0.5 * k1a * s.dx1), s2 = dsinc(0.5 * s.k2 * s.dx2);
     double sl1 = s1, sl2 = s2, sm1 = 1.0, sm2 = 1.0;                 // orders l + 1 and l
     for (int q = 0; q < order; q++) { sl1 *= s1; sl2 *= s2; sm1 *= s1; sm2 *= s2; }
     const double sgn = (nu1 & 1) ? -1.0 : 1.0;
@@ -262,110 +348,217 @@ __global__ void k_nci(const NciSample* __restrict__ smp, int64_t n, int order, i
     const double corr = (correct_j1 && s.k1 != 0.0) ? dsinc(0.5 * s.k1 * s.dx1) * s.k1 / m.kE1 : 1.0;
     m.Sj1 = sm1 * sl2 * sgn * F * corr;
     m.Sj2 = sl1 * sm2 * F;
+    m.res = k1a * m.v0;
+    const double kE2s = m.kE2 * m.kE2;
+    m.K2 = m.kE1 * m.kE1 + kE2s;
+    m.as = a * m.Sj1 * m.SE1;
+    m.sb = m.b * m.Sj2;
+    m.sk = m.SB3s * m.kE1 * m.v0;
+    m.c1 = m.b * m.Sj1 * m.SE1 * kE2s * (m.v0 * m.v0 - 1.0);
+    m.c2 = m.b * m.Sj2 * m.SE2 * kE2s;
+    m.c3 = m.b * m.Sj1 * m.kE2 * m.k2 * m.SE2 * m.kE1 * m.v0;
+    m.c4 = m.b * m.Sj1 * m.kE2 * m.k2 * m.SB3s * m.v0 * m.v0;
+    m.c = *c = m.res - m.muwg;
+    sincos(m.c * m.h, &m.sc, &m.cc);
+    *rho = cbrt(s.wp2 / s.gamma);
+    *k1a_out = k1a;
+}
 
-    const Z c = zc(m.k1a * m.v0 - m.mu * m.wg, 0.0);                // the resonance
-    const double rho = cbrt(s.wp2 / s.gamma);
-    Z r[kMaxRoots];
-    int nf = 0, N = 0, e = 0;
-    if (rho > 0.0) {
-        N = winding_circle(m, c, rho);
-        if (N < 0 || N > kMaxRoots) { e |= (N < 0) ? NCI_EUNRESOLVED : NCI_ETOOMANY; N = 0; }
-    }
-    // ---- seeds: the cubic's roots (Eq. asym1, v0 -> 1 in k~1), the resonance, rings in the disk
-    if (N > 0) {
-        const double kt = m.k1a - m.mu * m.wg, hh = m.h;
-        const double xi0 = sin(kt * hh) / hh, xi1 = cos(kt * hh), ze0 = cos(kt * hh), ze1 = -sin(kt * hh) * hh;
-        const double kE1 = m.kE1, kE2 = m.kE2, SB = m.SB3s;
-        const double A2 = 2.0 * xi0 * xi0 * xi0 * xi1;
-        const double B2 = xi0 * xi0 * (xi0 * xi0 - kE1 * kE1 - kE2 * kE2 - m.b * m.Sj2 * (m.SE2 * xi1 - ze1 * SB * kE1));
-        const double C2 = m.b * (xi0 * xi0 * m.Sj2 * (ze0 * SB * kE1 - m.SE2 * xi0) - xi1 * m.Sj1 * kE2 * m.k2 * m.SE2 * kE1
-                                 + xi0 * kE2 * (m.Sj2 * m.SE2 * kE2 - m.Sj1 * m.k2 * ze1 * SB * xi0));
-        const double D2 = m.b * xi0 * kE2 * m.k2 * m.Sj1 * (m.SE2 * kE1 - ze0 * SB * xi0);
-        constexpr int kRing = 8;
-        const int nseed = 4 + 3 * kRing;
-        Z cub[3];
-        const bool have_cubic = A2 != 0.0;
-        if (have_cubic) cubic_roots(A2, B2, C2, D2, cub);
-        for (int q = 0; q < nseed && nf < N; q++) {
-            Z w0;
-            if (q < 3) {
-                if (!have_cubic) continue;
-                w0 = zc(c.re + cub[q].re, cub[q].im);
-                if (zabs(zsub(w0, c)) >= rho) continue;
-            } else if (q == 3) {
-                w0 = zc(c.re + 1e-6 * rho, 1e-7 * rho);
-            } else {
-                const int ring = (q - 4) / kRing, k = (q - 4) % kRing;
-                const double rr = rho * (0.15 + 0.3 * ring);
-                double sn, cs;
-                sincospi((2.0 * k + 0.5 * ring) / kRing, &sn, &cs);
-                w0 = zc(c.re + rr * cs, c.im + rr * sn);
-            }
-            Z w;
-            if (!newton_deflated(m, w0, r, nf, &w)) continue;
-            if (zabs(zsub(w, c)) >= rho) continue;
-            r[nf++] = w;
+// the cubic of Eq. asym1 (v0 -> 1 in k~1) about the resonance; false if it has no leading term
+__device__ bool nci_cubic(const NciMode& m, double k1a, Z cub[3]) {
+    const double kt = k1a - m.muwg, hh = m.h;
+    const double xi0 = sin(kt * hh) / hh, xi1 = cos(kt * hh), ze0 = cos(kt * hh), ze1 = -sin(kt * hh) * hh;
+    const double kE1 = m.kE1, kE2 = m.kE2, SB = m.SB3s;
+    const double A2 = 2.0 * xi0 * xi0 * xi0 * xi1;
+    const double B2 = xi0 * xi0 * (xi0 * xi0 - kE1 * kE1 - kE2 * kE2 - m.b * m.Sj2 * (m.SE2 * xi1 - ze1 * SB * kE1));
+    const double C2 = m.b * (xi0 * xi0 * m.Sj2 * (ze0 * SB * kE1 - m.SE2 * xi0) - xi1 * m.Sj1 * kE2 * m.k2 * m.SE2 * kE1
+                             + xi0 * kE2 * (m.Sj2 * m.SE2 * kE2 - m.Sj1 * m.k2 * ze1 * SB * xi0));
+    const double D2 = m.b * xi0 * kE2 * m.k2 * m.Sj1 * (m.SE2 * kE1 - ze0 * SB * xi0);
+    if (A2 == 0.0) return false;
+    cubic_roots(A2, B2, C2, D2, cub);
+    return true;
+}
+
+// a zero this far from the real axis (in units of rho) and its conjugate are two: nearer ones could be
+// one real zero's rounding
+constexpr double kPairIm = 1e-4;
+constexpr int kRing = 8, kRingSeeds = 3 * kRing;      // three rings of seeds inside the disk
+
+// Step 3 for one pair, by the whole warp (every lane with the same values; the windings' points
+// across the lanes): the zeros of the disk by subdivision of a rectangle around it.
+__device__ int nci_subdivide(const NciMode& m, Z c, double rho, Z* r, int* e) {
+    int nf = 0;
+    const double fr[4][2] = {{0.4871, 0.5317}, {0.4413, 0.5689}, {0.5593, 0.4231}, {0.3917, 0.6143}};
+    const double hmin = fmax(1e-12 * rho, 1e-9 * fmax(1.0, zabs(c)));
+    const double x0 = c.re - rho, x1 = c.re + 1.0007 * rho, y0 = c.im - 1.0003 * rho, y1 = c.im + 1.0011 * rho;
+    const int Nr = winding_rect(m, x0, x1, y0, y1);
+    if (Nr < 0) *e |= NCI_EUNRESOLVED;
+    struct Rect { double x0, x1, y0, y1; int N; };
+    Rect st[kStack];
+    int sp = 0;
+    if (Nr > 0) st[sp++] = Rect{x0, x1, y0, y1, Nr};
+    auto keep = [&](Z w) {
+        if (nf < kMaxRoots) {
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) r[nf] = w;
+            nf++;
+        } else {
+            *e |= NCI_ETOOMANY;
         }
-    }
-    // ---- the rest by argument-principle subdivision of a rectangle enclosing the disk
-    if (nf < N) {
-        nf = 0;
-        const double fr[4][2] = {{0.4871, 0.5317}, {0.4413, 0.5689}, {0.5593, 0.4231}, {0.3917, 0.6143}};
-        const double hmin = fmax(1e-12 * rho, 1e-9 * fmax(1.0, zabs(c)));
-        double x0 = c.re - rho, x1 = c.re + 1.0007 * rho, y0 = c.im - 1.0003 * rho, y1 = c.im + 1.0011 * rho;
-        const int Nr = winding_rect(m, x0, x1, y0, y1);
-        if (Nr < 0) e |= NCI_EUNRESOLVED;
-        struct Rect { double x0, x1, y0, y1; int N; };
-        Rect st[kStack];
-        int sp = 0;
-        if (Nr > 0) st[sp++] = Rect{x0, x1, y0, y1, Nr};
-        while (sp > 0) {
-            const Rect q = st[--sp];
-            if (q.N == 1) {
-                Z w;
-                if (newton_in(m, zc(q.x0 + fr[0][0] * (q.x1 - q.x0), q.y0 + fr[0][1] * (q.y1 - q.y0)), q.x0, q.x1, q.y0, q.y1, &w)) {
-                    if (zabs(zsub(w, c)) < rho) {
-                        if (nf < kMaxRoots) r[nf++] = w;
-                        else e |= NCI_ETOOMANY;
-                    }
-                    continue;
-                }
-            }
-            if (fmax(q.x1 - q.x0, q.y1 - q.y0) < hmin) {          // a cluster below resolution
-                const Z w = zc(0.5 * (q.x0 + q.x1), 0.5 * (q.y0 + q.y1));
-                if (zabs(zsub(w, c)) < rho)
-                    for (int k = 0; k < q.N; k++) {
-                        if (nf < kMaxRoots) r[nf++] = w;
-                        else e |= NCI_ETOOMANY;
-                    }
+    };
+    while (sp > 0) {
+        const Rect q = st[--sp];
+        if (q.N == 1) {
+            Z w;
+            if (newton_in(m, zc(q.x0 + fr[0][0] * (q.x1 - q.x0), q.y0 + fr[0][1] * (q.y1 - q.y0)), q.x0, q.x1, q.y0, q.y1, &w)) {
+                if (zabs(zsub(w, c)) < rho) keep(w);
                 continue;
             }
-            bool split = false;
-            for (int f = 0; f < 4 && !split; f++) {
-                const double xm = q.x0 + fr[f][0] * (q.x1 - q.x0), ym = q.y0 + fr[f][1] * (q.y1 - q.y0);
-                const Rect kid[4] = {{q.x0, xm, q.y0, ym, 0}, {xm, q.x1, q.y0, ym, 0}, {q.x0, xm, ym, q.y1, 0}, {xm, q.x1, ym, q.y1, 0}};
-                int ns[4], tot = 0;
-                bool ok = true;
-                for (int k = 0; k < 4 && ok; k++) {
-                    ns[k] = winding_rect(m, kid[k].x0, kid[k].x1, kid[k].y0, kid[k].y1);
-                    ok = ns[k] >= 0;
-                    tot += ns[k];
-                }
-                if (!ok || tot != q.N) continue;
-                split = true;
-                for (int k = 0; k < 4; k++) {
-                    if (ns[k] == 0) continue;
-                    if (sp >= kStack) { e |= NCI_EUNRESOLVED; break; }
-                    st[sp] = kid[k];
-                    st[sp].N = ns[k];
-                    sp++;
-                }
+        }
+        if (fmax(q.x1 - q.x0, q.y1 - q.y0) < hmin) {          // a cluster below resolution
+            const Z w = zc(0.5 * (q.x0 + q.x1), 0.5 * (q.y0 + q.y1));
+            if (zabs(zsub(w, c)) < rho)
+                for (int k = 0; k < q.N; k++) keep(w);
+            continue;
+        }
+        bool split = false;
+        for (int f = 0; f < 4 && !split; f++) {
+            const double xm = q.x0 + fr[f][0] * (q.x1 - q.x0), ym = q.y0 + fr[f][1] * (q.y1 - q.y0);
+            const Rect kid[4] = {{q.x0, xm, q.y0, ym, 0}, {xm, q.x1, q.y0, ym, 0}, {q.x0, xm, ym, q.y1, 0}, {xm, q.x1, ym, q.y1, 0}};
+            int ns[4], tot = 0;
+            bool ok = true;
+            for (int k = 0; k < 4 && ok; k++) {
+                ns[k] = winding_rect(m, kid[k].x0, kid[k].x1, kid[k].y0, kid[k].y1);
+                ok = ns[k] >= 0;
+                tot += ns[k];
             }
-            if (!split) e |= NCI_EUNRESOLVED;
+            if (!ok || tot != q.N) continue;
+            split = true;
+            for (int k = 0; k < 4; k++) {
+                if (ns[k] == 0) continue;
+                if (sp >= kStack) { *e |= NCI_EUNRESOLVED; break; }
+                st[sp] = kid[k];
+                st[sp].N = ns[k];
+                sp++;
+            }
+        }
+        if (!split) *e |= NCI_EUNRESOLVED;
+    }
+    __syncwarp();
+    return nf;
+}
+
+// A warp (block of kNciThreads / 32 of them) per `group` consecutive pairs (group <= 32, a lane each).
+constexpr int kNciThreads = 64;
+__global__ void __launch_bounds__(kNciThreads) k_nci(const NciSample* __restrict__ smp, int64_t n, int order, int correct_j1,
+                                                     const int* __restrict__ alias, int n_alias, int group,
+                                                     double* __restrict__ growth, double2* __restrict__ root, int max_out,
+                                                     double2* __restrict__ roots_out, int* __restrict__ count_out,
+                                                     int* __restrict__ err) {
+    __shared__ NciMode modes[kNciThreads / 32][32];
+    __shared__ Z roots[kNciThreads / 32][32][kMaxRoots];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t first = ((int64_t)blockIdx.x * (kNciThreads / 32) + warp) * group;
+    const int64_t tid = first + lane, total = n * n_alias;
+    const bool live = lane < group && tid < total;
+    if (first >= total) return;                                     // the whole warp
+    NciMode& m = modes[warp][lane];
+    Z* const r = roots[warp][lane];
+    double c = 0.0, rho = 0.0, k1a = 0.0;
+    int nf = 0, N = 0, e = 0;
+    if (live) {
+        const int ai = (int)(tid % n_alias);
+        nci_symbols(smp[tid / n_alias], alias[2 * ai], alias[2 * ai + 1], order, correct_j1, m, &c, &rho, &k1a);
+    }
+    __syncwarp();
+    // ---- 1. the count, one pair after the other
+    double zx, zy;
+    sincospi(2.0 * lane / 64.0, &zy, &zx);
+    Z end = zc(0.0, 0.0);
+    if (live && rho > 0.0) nci_G<false>(m, zc(c - rho, 0.0), &end, nullptr);
+    for (unsigned todo = __ballot_sync(0xffffffffu, live && rho > 0.0); todo; todo &= todo - 1) {
+        const int j = __ffs(todo) - 1;
+        const int w = winding_circle(modes[warp][j], __shfl_sync(0xffffffffu, c, j), __shfl_sync(0xffffffffu, rho, j), zx, zy,
+                                     zc(__shfl_sync(0xffffffffu, end.re, j), __shfl_sync(0xffffffffu, end.im, j)));
+        if (lane == j) N = w;
+    }
+    if (N < 0 || N > kMaxRoots) { e |= (N < 0) ? NCI_EUNRESOLVED : NCI_ETOOMANY; N = 0; }
+    // ---- 2a. the cubic's roots inside the disk and the resonance as seeds, a pair per lane; one
+    // Newton step of every lane's current attempt per turn
+    {
+        Z cub[3];
+        bool have = false;
+        if (N > 0) have = nci_cubic(m, k1a, cub);
+        int q = -1;
+        bool skip = false;                                          // the next seed is the last one's conjugate, done
+        Newton s = newton_start(zc(0.0, 0.0));
+        auto next = [&]() {                                         // the next seed, or q = 4 when done
+            if (nf >= N) { q = 4; return; }
+            for (q += skip ? 2 : 1, skip = false; q < 4; q++) {
+                if (q == 3) { s = newton_start(zc(c + 1e-6 * rho, 1e-7 * rho)); return; }
+                const Z w0 = q == 0 ? cub[0] : q == 1 ? cub[1] : cub[2];
+                if (have && zabs(zsub(zc(c + w0.re, w0.im), zc(c, 0.0))) < rho) { s = newton_start(zc(c + w0.re, w0.im)); return; }
+            }
+        };
+        next();
+        while (__any_sync(0xffffffffu, q < 4)) {
+            if (q < 4) {
+                const int st = newton_step(m, s, r, nf);
+                if (st > 0 && zabs(zsub(s.w, zc(c, 0.0))) < rho) {
+                    r[nf++] = s.w;
+                    // G's coefficients are real: the conjugate of a zero well off the real axis is another
+                    if (nf < N && fabs(s.w.im) > kPairIm * rho) {
+                        r[nf++] = zc(s.w.re, -s.w.im);
+                        skip = q == 1;
+                    }
+                }
+                if (st != 0) next();
+            }
+            __syncwarp();
         }
     }
+    // ---- 2b. the rings, one pair after the other, a seed per lane: an attempt that finds nothing
+    // leaves the others' deflation as it was, so all run at once; the first that succeeds is kept
+    // and those after it run again, deflated by it too
+    for (unsigned todo = __ballot_sync(0xffffffffu, nf < N); todo; todo &= todo - 1) {
+        const int j = __ffs(todo) - 1;
+        const NciMode& mj = modes[warp][j];
+        Z* const rj = roots[warp][j];
+        const Z cj = zc(__shfl_sync(0xffffffffu, c, j), 0.0);
+        const double rhoj = __shfl_sync(0xffffffffu, rho, j);
+        const int Nj = __shfl_sync(0xffffffffu, N, j);
+        int nj = __shfl_sync(0xffffffffu, nf, j), from = 0;
+        while (nj < Nj && from < kRingSeeds) {
+            bool found = false;
+            Z w = zc(0.0, 0.0);
+            if (lane >= from && lane < kRingSeeds) {
+                const int ring = lane / kRing, k = lane % kRing;
+                const double rr = rhoj * (0.15 + 0.3 * ring);
+                double sn, cs;
+                sincospi((2.0 * k + 0.5 * ring) / kRing, &sn, &cs);
+                found = newton_deflated(mj, zc(cj.re + rr * cs, cj.im + rr * sn), rj, nj, &w) && zabs(zsub(w, cj)) < rhoj;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, found);
+            if (!hit) break;
+            const int win = __ffs(hit) - 1;
+            const bool pair = __shfl_sync(0xffffffffu, fabs(w.im) > kPairIm * rhoj, win) && nj + 1 < Nj;
+            if (lane == win) {
+                rj[nj] = w;
+                if (pair) rj[nj + 1] = zc(w.re, -w.im);
+            }
+            __syncwarp();
+            nj += pair ? 2 : 1;
+            from = win + 1;
+        }
+        // ---- 3. what the seeds left
+        int ej = 0;
+        if (nj < Nj) nj = nci_subdivide(mj, cj, rhoj, rj, &ej);
+        if (lane == j) { nf = nj; e |= ej; }
+    }
+    __syncwarp();
+    if (!live) return;
     double best = 0.0;
-    Z broot = c;
+    Z broot = zc(c, 0.0);
     for (int k = 0; k < nf; k++)
         if (r[k].im > best) { best = r[k].im; broot = r[k]; }
     growth[tid] = best;
@@ -385,9 +578,12 @@ static hyb_status nci_launch(const double* samples, int64_t n, int order, int co
     }
     if (n == 0) return HYB_OK;
     const int64_t total = n * n_alias;
-    const int thr = 64;
-    k_nci<<<(unsigned)((total + thr - 1) / thr), thr, 0, (cudaStream_t)stream>>>(
-        reinterpret_cast<const NciSample*>(samples), n, order, correct_j1, alias, n_alias, growth,
+    // 32 pairs per warp where that still gives every SM eight warps, fewer on small calls
+    const int64_t spread = total / (152 * 8);
+    const int group = spread >= 32 ? 32 : spread < 1 ? 1 : (int)spread;
+    const int64_t per_block = (int64_t)group * (kNciThreads / 32);
+    k_nci<<<(unsigned)((total + per_block - 1) / per_block), kNciThreads, 0, (cudaStream_t)stream>>>(
+        reinterpret_cast<const NciSample*>(samples), n, order, correct_j1, alias, n_alias, group, growth,
         reinterpret_cast<double2*>(root), max_out, reinterpret_cast<double2*>(roots_out), count_out, err);
     HYB_CUDA_TRY(cudaGetLastError());
     return HYB_OK;
