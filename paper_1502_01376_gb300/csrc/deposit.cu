@@ -9,7 +9,11 @@
 //   3D: W1 = dS1 (S2^0 S3^0 + dS2 S3^0/2 + S2^0 dS3/2 + dS2 dS3/3), cyclic for W2, W3,
 //       j_a = -q/(dt dV/dx_a) cumulative sum of W_a along axis a.
 // S are B-spline shape factors of order 1, 2 or 3 (grid points at integers).
-// One thread per particle; contributions are added with atomics.
+// FP32 2D: a lane adds up a run of particles of one cell in registers (k_deposit2d_runs);
+// otherwise one thread per particle adds its contributions with atomics.
+#include <algorithm>
+#include <type_traits>
+
 #include "hyb_internal.cuh"
 
 namespace hyb {
@@ -32,89 +36,345 @@ template <int ORDER> struct Win { static constexpr int lo = (ORDER == 1) ? -1 : 
 
 __device__ __forceinline__ int wrapi(int i, int n) { i %= n; return i < 0 ? i + n : i; }
 
-// 2D: lanes take particles 8 apart within each chunk of 256, so that for a sorted chunk the
-// lanes of a warp sit in different (mostly consecutive) cells and their atomic adds at the same
-// window offset go to different, neighbouring addresses.  (A variant that accumulated each block's
-// currents in a shared tile first and added each tile point once ran slower: 6.4 against 5.6 ms
-// for the 67 M particles of the drifting plasma.)
 constexpr int kDepThreads = 256;
 
+// One particle's moves and 1D shapes: WN = ORDER + 2 consecutive points per axis from gx, gy (relative to
+// the cell), outside which the shapes at x^n and at x^{n+1} (|x^{n+1} - x^n| < 1 cell) are zero and the
+// cumulative sums are back to 0; the start is clamped into the full window LO .. LO + W - 1, which
+// at a rounding edge only drops a point of weight 0.
 template <typename T, int ORDER>
-__global__ void __launch_bounds__(kDepThreads) k_deposit2d(T* __restrict__ J1, T* __restrict__ J2, T* __restrict__ J3,
-                                                          int n1, int n2, const int32_t* __restrict__ cell,
-                                                          const T* __restrict__ off0, const T* __restrict__ off1,
-                                                          const T* __restrict__ v3, const T* __restrict__ q, int64_t np,
-                                                          T c1s, T c2s, T c3s, int* __restrict__ flag) {
-    constexpr int W = Win<ORDER>::n, LO = Win<ORDER>::lo;
-    T* const Jc[3] = {J1, J2, J3};
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t base = blockIdx.x * (int64_t)kDepThreads; base < np; base += (int64_t)gridDim.x * kDepThreads) {
-        const int64_t p = base + lane * (kDepThreads / 32) + warp;
-        if (p >= np) continue;
-        const int cx = cell[2 * p], cy = cell[2 * p + 1];
-        const T x0 = off0[2 * p], y0 = off0[2 * p + 1], x1 = off1[2 * p], y1 = off1[2 * p + 1];
-        const T dx = x1 - x0, dy = y1 - y0;
-        if (!(x0 >= (T)0 && x0 < (T)1 && y0 >= (T)0 && y0 < (T)1 && dx > (T)-1 && dx < (T)1 && dy > (T)-1 && dy < (T)1) ||
-            cx < 0 || cx >= n1 || cy < 0 || cy >= n2) {
-            atomicOr(flag, 1);
-            continue;
-        }
-        // along each axis only the points where the shape at x^n or at x^{n+1} is non-zero: at most
-        // ORDER + 2 consecutive points (|x^{n+1} - x^n| < 1 cell), starting at gx, gy (relative to the
-        // cell, clamped into the full window LO .. LO + W - 1, which at a rounding edge only drops a
-        // point of weight 0); beyond them the cumulative sums are back to 0
-        constexpr int WN = ORDER + 2;
-        const int gx = min(max((int)floor((x0 < x1 ? x0 : x1) - (T)0.5 * (T)(ORDER + 1)) + 1, LO), LO + W - WN);
-        const int gy = min(max((int)floor((y0 < y1 ? y0 : y1) - (T)0.5 * (T)(ORDER + 1)) + 1, LO), LO + W - WN);
-        T Sx0[WN], Sx1[WN], Sy0[WN], Sy1[WN];
+struct Move2d {
+    static constexpr int WN = ORDER + 2;
+    int gx, gy;
+    T Sx0[WN], Sx1[WN], Sy0[WN], Sy1[WN];
+    __device__ __forceinline__ void set(T x0, T x1, T y0, T y1) {
+        constexpr int W = Win<ORDER>::n, LO = Win<ORDER>::lo;
+        gx = min(max((int)floor((x0 < x1 ? x0 : x1) - (T)0.5 * (T)(ORDER + 1)) + 1, LO), LO + W - WN);
+        gy = min(max((int)floor((y0 < y1 ? y0 : y1) - (T)0.5 * (T)(ORDER + 1)) + 1, LO), LO + W - WN);
 #pragma unroll
         for (int w = 0; w < WN; w++) {
             const T px = (T)(gx + w), py = (T)(gy + w);
             Sx0[w] = bspline<ORDER>(x0 - px); Sx1[w] = bspline<ORDER>(x1 - px);
             Sy0[w] = bspline<ORDER>(y0 - py); Sy1[w] = bspline<ORDER>(y1 - py);
         }
-        const T qp = q[p];
-        const T c1 = c1s * qp, c2 = c2s * qp;
-        const T c3 = v3 ? c3s * qp * v3[p] : (T)0;
-        int col[WN];
-        int64_t row[WN];
+    }
+};
+// the conditions on a particle (NaN offsets fail them); a particle that breaks them is skipped and flagged
+template <typename T>
+__device__ __forceinline__ bool move_ok(int cx, int cy, T x0, T x1, T y0, T y1, int n1, int n2) {
+    const T dx = x1 - x0, dy = y1 - y0;
+    return x0 >= (T)0 && x0 < (T)1 && y0 >= (T)0 && y0 < (T)1 && dx > (T)-1 && dx < (T)1 && dy > (T)-1 && dy < (T)1 &&
+           cx >= 0 && cx < n1 && cy >= 0 && cy < n2;
+}
+
+// one particle, each contribution added with its own atomic
+template <typename T, int ORDER>
+__device__ __forceinline__ void deposit_one(T* J1, T* J2, T* J3, int n1, int n2, int cx, int cy, const Move2d<T, ORDER>& m, T c1, T c2,
+                                            T c3) {
+    constexpr int WN = ORDER + 2;
+    T* const Jc[3] = {J1, J2, J3};
+    int col[WN];
+    int64_t row[WN];
 #pragma unroll
-        for (int w = 0; w < WN; w++) { col[w] = wrapi(cx + gx + w, n1); row[w] = (int64_t)wrapi(cy + gy + w, n2) * n1; }
-        auto add = [&](int c, int i, int j, T v) { atomicAdd(Jc[c] + row[j] + col[i], v); };
+    for (int w = 0; w < WN; w++) { col[w] = wrapi(cx + m.gx + w, n1); row[w] = (int64_t)wrapi(cy + m.gy + w, n2) * n1; }
+    auto add = [&](int c, int i, int j, T v) { atomicAdd(Jc[c] + row[j] + col[i], v); };
 #pragma unroll
-        for (int j = 0; j < WN; j++) {
-            const T sy = (T)0.5 * (Sy0[j] + Sy1[j]);
-            if (sy == (T)0) continue;
-            T acc = (T)0;
-#pragma unroll
-            for (int i = 0; i < WN; i++) {
-                acc += (Sx1[i] - Sx0[i]) * sy;
-                if (acc != (T)0) add(0, i, j, c1 * acc);
-            }
-        }
+    for (int j = 0; j < WN; j++) {
+        const T sy = (T)0.5 * (m.Sy0[j] + m.Sy1[j]);
+        if (sy == (T)0) continue;
+        T acc = (T)0;
 #pragma unroll
         for (int i = 0; i < WN; i++) {
-            const T sx = (T)0.5 * (Sx0[i] + Sx1[i]);
-            if (sx == (T)0) continue;
-            T acc = (T)0;
+            acc += (m.Sx1[i] - m.Sx0[i]) * sy;
+            if (acc != (T)0) add(0, i, j, c1 * acc);
+        }
+    }
 #pragma unroll
-            for (int j = 0; j < WN; j++) {
-                acc += (Sy1[j] - Sy0[j]) * sx;
-                if (acc != (T)0) add(1, i, j, c2 * acc);
+    for (int i = 0; i < WN; i++) {
+        const T sx = (T)0.5 * (m.Sx0[i] + m.Sx1[i]);
+        if (sx == (T)0) continue;
+        T acc = (T)0;
+#pragma unroll
+        for (int j = 0; j < WN; j++) {
+            acc += (m.Sy1[j] - m.Sy0[j]) * sx;
+            if (acc != (T)0) add(1, i, j, c2 * acc);
+        }
+    }
+    if (c3 != (T)0) {
+        // S1^0 S2^0/3 + S1^1 S2^0/6 + S1^0 S2^1/6 + S1^1 S2^1/3 = S1^0 a_j + S1^1 b_j
+#pragma unroll
+        for (int j = 0; j < WN; j++) {
+            const T aj = (m.Sy0[j] + m.Sy0[j] + m.Sy1[j]) * ((T)1 / (T)6), bj = (m.Sy0[j] + m.Sy1[j] + m.Sy1[j]) * ((T)1 / (T)6);
+#pragma unroll
+            for (int i = 0; i < WN; i++) {
+                const T w3 = m.Sx0[i] * aj + m.Sx1[i] * bj;
+                if (w3 != (T)0) add(2, i, j, c3 * w3);
             }
         }
-        if (c3 != (T)0) {
-            // S1^0 S2^0/3 + S1^1 S2^0/6 + S1^0 S2^1/6 + S1^1 S2^1/3 = S1^0 a_j + S1^1 b_j
+    }
+}
+
+// 2D, one thread per particle (FP64): lanes take particles BS / 32 apart within each chunk of BS, so
+// that for a sorted chunk the lanes of a warp sit in different (mostly consecutive) cells and their
+// atomic adds at the same window offset go to different, neighbouring addresses.
+template <typename T, int ORDER>
+__global__ void __launch_bounds__(kDepThreads) k_deposit2d(T* __restrict__ J1, T* __restrict__ J2, T* __restrict__ J3,
+                                                          int n1, int n2, const int32_t* __restrict__ cell,
+                                                          const T* __restrict__ off0, const T* __restrict__ off1,
+                                                          const T* __restrict__ v3, const T* __restrict__ q, int64_t np,
+                                                          T c1s, T c2s, T c3s, int* __restrict__ flag) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < np; base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = base + lane * (int)(blockDim.x >> 5) + warp;
+        if (p >= np) continue;
+        const int cx = cell[2 * p], cy = cell[2 * p + 1];
+        const T x0 = off0[2 * p], y0 = off0[2 * p + 1], x1 = off1[2 * p], y1 = off1[2 * p + 1];
+        if (!move_ok(cx, cy, x0, x1, y0, y1, n1, n2)) {
+            atomicOr(flag, 1);
+            continue;
+        }
+        Move2d<T, ORDER> m;
+        m.set(x0, x1, y0, y1);
+        const T qp = q[p];
+        deposit_one<T, ORDER>(J1, J2, J3, n1, n2, cx, cy, m, c1s * qp, c2s * qp, v3 ? c3s * qp * v3[p] : (T)0);
+    }
+}
+
+// FP32 2D.  Bound before: one atomic per particle, point and component, 48 at order 2, at the L2's rate of
+// about 155 G sectors/s when they scatter and 110 G when a warp's are consecutive (measured): 5.1 ms for
+// the 67 M particles of the drifting plasma, 1.5 ms now.  Every current is a sum of products of a function of x1 and one of x2,
+//   j1 = c1 P1(i) sy(j), j2 = sx(i) c2 P2(j), j3 = S1^0(i) c3 a(j) + S1^1(i) c3 b(j)
+// (P the cumulative sum of dS, s = (S^0 + S^1)/2), and particles stored in cell order come in runs of one
+// cell, whose functions all fit the same N x N window, N = ORDER + 3 points.  A warp therefore cuts
+// its particles into runs and gives each lane one: the lane adds its run's particles in registers and
+// only then touches memory.  When the 32 cells are consecutive, each row of the window is first
+// summed across the lanes (shuffles), so that a row of 32 + N - 1 points takes two atomics of the warp;
+// otherwise each lane adds its window, one atomic per point, neighbouring lanes to neighbouring addresses.
+// Where that would touch more sectors than the particles one by one (runs too short and
+// scattered), each lane adds one particle's points on its own.
+// (Also tried: the particles' functions in shared memory and a lane per window point, for any order of
+// particles: 3.7 ms, bound by the shared-memory reads, 10 wavefronts per particle; scattered
+// particles' rows as aligned quads with red.v4: 0.24 against 0.20 ms for 1 M particles.)
+// The shapes S^0 (x0 in [0, 1)) and S^1 (x1) at the N points of a window from B0, for a particle whose own
+// points lie in it: bspline()'s values, bit for bit (the last product of a piece is rounded on its own: the
+// differences dS of a cold plasma's moves are a few units of it), with only the pieces that each point can need.
+template <int ORDER>
+__device__ __forceinline__ float spline_in(float a) {       // |d| = a below the first knot
+    if (ORDER == 1) return 1.f - a;
+    if (ORDER == 2) return 0.75f - a * a;
+    return __fmul_rn(4.f - 6.f * a * a + 3.f * a * a * a, 1.f / 6.f);
+}
+template <int ORDER>
+__device__ __forceinline__ float spline_out(float a) {      // above it
+    if (ORDER == 1) return 0.f;
+    if (ORDER == 2) { const float t = fmaxf(1.5f - a, 0.f); return __fmul_rn(0.5f * t, t); }
+    const float t = fmaxf(2.f - a, 0.f);
+    return __fmul_rn(t * t * t, 1.f / 6.f);
+}
+template <int ORDER>
+__device__ __forceinline__ float spline_any(float d) {
+    const float a = fabsf(d);
+    if (ORDER == 1) return fmaxf(1.f - a, 0.f);
+    return a <= (ORDER == 2 ? 0.5f : 1.f) ? spline_in<ORDER>(a) : spline_out<ORDER>(a);
+}
+template <int ORDER>
+__device__ __forceinline__ void window_shapes(float x0, float x1, float (&S0)[ORDER + 3], float (&S1)[ORDER + 3]) {
+    if constexpr (ORDER == 1) {                              // points -1 .. 2, x1 in (-1, 2)
+        S0[0] = 0.f; S0[1] = spline_in<1>(x0); S0[2] = spline_in<1>(fabsf(x0 - 1.f)); S0[3] = 0.f;
 #pragma unroll
-            for (int j = 0; j < WN; j++) {
-                const T aj = (Sy0[j] + Sy0[j] + Sy1[j]) * ((T)1 / (T)6), bj = (Sy0[j] + Sy1[j] + Sy1[j]) * ((T)1 / (T)6);
+        for (int e = 0; e < 4; e++) S1[e] = spline_any<1>(x1 - (float)(e - 1));
+    } else if constexpr (ORDER == 2) {                       // points -1 .. 3, x1 in [-1/2, 2)
+        S0[0] = spline_out<2>(x0 + 1.f); S0[1] = spline_any<2>(x0); S0[2] = spline_any<2>(x0 - 1.f); S0[3] = spline_out<2>(2.f - x0); S0[4] = 0.f;
+        S1[0] = spline_out<2>(x1 + 1.f);
 #pragma unroll
-                for (int i = 0; i < WN; i++) {
-                    const T w3 = Sx0[i] * aj + Sx1[i] * bj;
-                    if (w3 != (T)0) add(2, i, j, c3 * w3);
+        for (int e = 1; e < 4; e++) S1[e] = spline_any<2>(x1 - (float)(e - 1));
+        S1[4] = spline_out<2>(3.f - x1);
+    } else {                                                 // points -2 .. 3, x1 in (-1, 2)
+        S0[0] = 0.f; S0[1] = spline_out<3>(x0 + 1.f); S0[2] = spline_in<3>(x0); S0[3] = spline_in<3>(fabsf(x0 - 1.f));
+        S0[4] = spline_out<3>(2.f - x0); S0[5] = 0.f;
+        S1[0] = spline_out<3>(x1 + 2.f);
+#pragma unroll
+        for (int e = 1; e < 5; e++) S1[e] = spline_any<3>(x1 - (float)(e - 2));
+        S1[5] = spline_out<3>(3.f - x1);
+    }
+}
+
+// one particle on its own (kept out of line: rare in the run kernel)
+template <int ORDER>
+__device__ __noinline__ void deposit_alone(float* J1, float* J2, float* J3, int n1, int n2, int2 cc, float2 o0, float2 o1, float c1,
+                                           float c2, float c3) {
+    Move2d<float, ORDER> m;
+    m.set(o0.x, o1.x, o0.y, o1.y);
+    deposit_one<float, ORDER>(J1, J2, J3, n1, n2, cc.x, cc.y, m, c1, c2, c3);
+}
+
+constexpr int kRunWarps = 4, kRunScan = 512;      // warps per block; particles looked at for 32 runs
+constexpr int kRunMax = 32;                       // a longer run is cut (at multiples of this many particles)
+
+template <int ORDER>
+__global__ void __launch_bounds__(32 * kRunWarps, ORDER == 3 ? 3 : 4)
+k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restrict__ J3, int n1, int n2,
+                 const int2* __restrict__ cell, const float2* __restrict__ off0, const float2* __restrict__ off1,
+                 const float* __restrict__ v3, const float* __restrict__ q, int64_t np, int64_t per_warp, float c1s, float c2s,
+                 float c3s, int* __restrict__ flag) {
+    constexpr int WN = ORDER + 2, N = ORDER + 3, B0 = ORDER == 3 ? -2 : -1;
+    __shared__ int s_start[kRunWarps][64];       // at most 32 + 32 heads
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int* const start = s_start[warp];
+    const int64_t first = ((int64_t)blockIdx.x * kRunWarps + warp) * per_warp;
+    const int64_t last = first + per_warp < np ? first + per_warp : np;
+    int64_t base = first;
+    while (base < last) {
+        // ---- the next runs: places (from base) where the cell changes or a multiple of kRunMax begins
+        int nr = 0, seen = 0;
+        const int avail = (int)(last - base < kRunScan ? last - base : kRunScan);
+        int2 carry = make_int2(0, 0);
+        while (seen < avail && nr <= 32) {
+            const int i = seen + lane;
+            const int2 c = i < avail ? cell[base + i] : make_int2(0, 0);
+            {   // the rest of these particles into L2: two 128-byte lines of either offset array, one of q and v3
+                const int64_t g = base + seen + (lane & 1) * 16;
+                const void* line = lane < 2 ? (const void*)(off0 + g) : lane < 4 ? (const void*)(off1 + g)
+                                   : lane == 4 ? (const void*)(q + g) : (const void*)(v3 + g);
+                if (g < last && lane < (v3 ? 7 : 5) && lane != 5) asm volatile("prefetch.global.L2 [%0];" :: "l"(line));
+            }
+            int2 pc = make_int2(__shfl_up_sync(0xffffffffu, c.x, 1), __shfl_up_sync(0xffffffffu, c.y, 1));
+            if (lane == 0) pc = carry;
+            const bool head = i < avail && (i == 0 || c.x != pc.x || c.y != pc.y || ((base + i) & (kRunMax - 1)) == 0);
+            const unsigned h = __ballot_sync(0xffffffffu, head);
+            if (head) start[nr + __popc(h & ((1u << lane) - 1u))] = i;
+            nr += __popc(h);
+            carry = make_int2(__shfl_sync(0xffffffffu, c.x, 31), __shfl_sync(0xffffffffu, c.y, 31));
+            seen += 32;
+        }
+        __syncwarp();
+        const int runs = min(nr, 32);
+        int end = nr > 32 ? start[32] : min(seen, avail);                   // particles of these runs
+        const int s0 = lane < runs ? start[lane] : end, s1 = lane + 1 < runs ? start[lane + 1] : end;
+        const int2 cc = lane < runs ? cell[base + s0] : make_int2(-1, -1);
+        const bool inside = cc.x >= 0 && cc.x < n1 && cc.y >= 0 && cc.y < n2;
+        __syncwarp();
+        // ---- which way: consecutive cells of a row; else by the sectors touched
+        const int2 c0 = make_int2(__shfl_sync(0xffffffffu, cc.x, 0), __shfl_sync(0xffffffffu, cc.y, 0));
+        const bool row = __all_sync(0xffffffffu, inside && cc.y == c0.y && cc.x == c0.x + lane);
+        const int2 left = make_int2(__shfl_up_sync(0xffffffffu, cc.x, 1), __shfl_up_sync(0xffffffffu, cc.y, 1));
+        const int sectors = __popc(__ballot_sync(0xffffffffu, lane < runs && (lane == 0 || left.y != cc.y || (left.x >> 3) != (cc.x >> 3))));
+        if (row || N * N * sectors <= WN * WN * end) {
+            float a1[N][N], a2[N][N], a3[N][N];
+#pragma unroll
+            for (int j = 0; j < N; j++)
+#pragma unroll
+                for (int i = 0; i < N; i++) a1[j][i] = a2[j][i] = a3[j][i] = 0.f;
+            float2 n0 = make_float2(0.f, 0.f), nw = n0;
+            float nq = 0.f, nv = 0.f;
+            auto fetch = [&](int i) {
+                if (i < s1) {
+                    n0 = off0[base + i];
+                    nw = off1[base + i];
+                    nq = q[base + i];
+                    nv = v3 ? v3[base + i] : 0.f;
+                }
+            };
+            fetch(s0);
+            const int longest = __reduce_max_sync(0xffffffffu, s1 - s0);
+            for (int t = 0; t < longest; t++) {
+                const bool here = s0 + t < s1;
+                const float2 o0 = n0, o1 = nw;
+                const float qp = nq, vp = nv;
+                fetch(s0 + t + 1);
+                if (!here) continue;
+                if (!move_ok(cc.x, cc.y, o0.x, o1.x, o0.y, o1.y, n1, n2)) {
+                    atomicOr(flag, 1);
+                    continue;
+                }
+                const float c1 = c1s * qp, c2 = c2s * qp, c3 = c3s * qp * vp;
+                const float lx = o0.x < o1.x ? o0.x : o1.x, ly = o0.y < o1.y ? o0.y : o1.y;
+                // the first of the particle's own WN points, from the window's first
+                const int ox = (int)floorf(lx - 0.5f * (float)(ORDER + 1)) + 1 - B0, oy = (int)floorf(ly - 0.5f * (float)(ORDER + 1)) + 1 - B0;
+                // an order-2 particle that moves back by more than half a cell leaves the window, and 0 times a
+                // non-finite charge would spread over it: such a particle on its own
+                if (ox < 0 || oy < 0 || !(isfinite(c1) && isfinite(c2) && isfinite(c3))) {
+                    deposit_alone<ORDER>(J1, J2, J3, n1, n2, cc, o0, o1, c1, c2, c3);
+                    continue;
+                }
+                float Sx0[N], Sx1[N], Sy0[N], Sy1[N], p1[N], sx[N];
+                window_shapes<ORDER>(o0.x, o1.x, Sx0, Sx1);
+                window_shapes<ORDER>(o0.y, o1.y, Sy0, Sy1);
+                float p = 0.f;
+#pragma unroll
+                for (int e = 0; e < N; e++) {
+                    p += Sx1[e] - Sx0[e];
+                    p1[e] = c1 * p;
+                    sx[e] = 0.5f * (Sx0[e] + Sx1[e]);
+                }
+                if (ox == 0) p1[N - 1] = 0.f;            // past the particle's own points the sum is back to 0
+                p = 0.f;
+#pragma unroll
+                for (int e = 0; e < N; e++) {
+                    const float y0 = Sy0[e], y1 = Sy1[e];
+                    p += y1 - y0;
+                    const float sy = 0.5f * (y0 + y1), p2 = e == N - 1 && oy == 0 ? 0.f : c2 * p;
+                    const float a = c3 * ((y0 + y0 + y1) * (1.f / 6.f)), b = c3 * ((y0 + y1 + y1) * (1.f / 6.f));
+#pragma unroll
+                    for (int i = 0; i < N; i++) {
+                        a1[e][i] = fmaf(p1[i], sy, a1[e][i]);
+                        a2[e][i] = fmaf(sx[i], p2, a2[e][i]);
+                        a3[e][i] = fmaf(Sx0[i], a, fmaf(Sx1[i], b, a3[e][i]));
+                    }
                 }
             }
+            if (row) {
+                // column c0.x + B0 + lane gets point i of lane - i; the last lanes' points beyond lane 31
+                // come round to the first lanes (tail)
+                const int col = (c0.x + B0 + lane) & (n1 - 1), tcol = (c0.x + B0 + 32 + lane) & (n1 - 1);
+                auto rowsum = [&](const float (&v)[N], float* J) {
+                    float s = v[0], tail = 0.f;
+#pragma unroll
+                    for (int i = 1; i < N; i++) {
+                        const float o = __shfl_sync(0xffffffffu, v[i], (lane - i) & 31);
+                        s += lane >= i ? o : 0.f;
+                        tail += lane >= i ? 0.f : o;
+                    }
+                    if (s != 0.f) atomicAdd(J + col, s);
+                    if (lane < N - 1 && tail != 0.f) atomicAdd(J + tcol, tail);
+                };
+#pragma unroll
+                for (int j = 0; j < N; j++) {
+                    const int64_t at = (int64_t)wrapi(c0.y + B0 + j, n2) * n1;
+                    rowsum(a1[j], J1 + at);
+                    rowsum(a2[j], J2 + at);
+                    rowsum(a3[j], J3 + at);
+                }
+            } else if (inside) {
+                int col[N];
+#pragma unroll
+                for (int i = 0; i < N; i++) col[i] = (cc.x + B0 + i) & (n1 - 1);
+#pragma unroll
+                for (int j = 0; j < N; j++) {
+                    const int64_t at = (int64_t)wrapi(cc.y + B0 + j, n2) * n1;
+#pragma unroll
+                    for (int i = 0; i < N; i++) {
+                        if (a1[j][i] != 0.f) atomicAdd(J1 + at + col[i], a1[j][i]);
+                        if (a2[j][i] != 0.f) atomicAdd(J2 + at + col[i], a2[j][i]);
+                        if (a3[j][i] != 0.f) atomicAdd(J3 + at + col[i], a3[j][i]);
+                    }
+                }
+            }
+        } else {
+            // ---- scattered: a particle per lane
+            if (end > 32) end &= ~31;                                // whole warps; the rest in the next round
+            for (int i = lane; i < end; i += 32) {
+                const int2 pc = cell[base + i];
+                const float2 o0 = off0[base + i], o1 = off1[base + i];
+                if (!move_ok(pc.x, pc.y, o0.x, o1.x, o0.y, o1.y, n1, n2)) {
+                    atomicOr(flag, 1);
+                    continue;
+                }
+                const float qp = q[base + i];
+                deposit_alone<ORDER>(J1, J2, J3, n1, n2, pc, o0, o1, c1s * qp, c2s * qp, v3 ? c3s * qp * v3[base + i] : 0.f);
+            }
         }
+        base += end;
     }
 }
 
@@ -173,6 +433,20 @@ __global__ void k_deposit3d(T* __restrict__ J1, T* __restrict__ J2, T* __restric
     }
 }
 
+template <int ORDER>
+static cudaError_t launch_runs(hyb_grid* g, float* J1, float* J2, float* J3, const int32_t* cell, const float* off_old,
+                               const float* off_new, const float* v3, const float* q, int64_t np, float c1, float c2, float c3) {
+    auto kern = k_deposit2d_runs<ORDER>;
+    // a contiguous range of particles per warp, four waves of resident blocks
+    const int64_t warps = (int64_t)resident_grid((const void*)kern, 32 * kRunWarps, 0) * kRunWarps * 4;
+    const int64_t per = std::max<int64_t>(32, ((np + warps - 1) / warps + 255) / 256 * 256);
+    const unsigned blocks = (unsigned)((np + per * kRunWarps - 1) / (per * kRunWarps));
+    kern<<<blocks, 32 * kRunWarps, 0, g->stream>>>(J1, J2, J3, g->d.n1, g->d.n2, reinterpret_cast<const int2*>(cell),
+                                                   reinterpret_cast<const float2*>(off_old),
+                                                   reinterpret_cast<const float2*>(off_new), v3, q, np, per, c1, c2, c3, g->dflag);
+    return cudaGetLastError();
+}
+
 template <typename T>
 hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* off_new, const T* v3, const T* q,
                    int64_t np, int order) {
@@ -181,18 +455,30 @@ hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* 
     for (int c = 0; c < 3; c++) HYB_CUDA_TRY(cudaMemsetAsync(g->J[c], 0, bytes, g->stream));
     if (np == 0) return HYB_OK;
     T* J1 = (T*)g->J[0]; T* J2 = (T*)g->J[1]; T* J3 = (T*)g->J[2];
-    const int threads = kDepThreads;
     int dev_sms = 0;
     cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, g->device);
-    int64_t want = (np + threads - 1) / threads;
-    unsigned blocks = (unsigned)(want < (int64_t)dev_sms * 32 ? want : (int64_t)dev_sms * 32);
-    if (blocks == 0) blocks = 1;
     if (d.dims == 2) {
         const T c1 = (T)(-1.0 / (d.dt * d.dx2)), c2 = (T)(-1.0 / (d.dt * d.dx1)), c3 = (T)(1.0 / (d.dx1 * d.dx2));
+        // the run kernel reads a particle's pairs at once
+        const bool pairs = ((((uintptr_t)cell | (uintptr_t)off_old | (uintptr_t)off_new) & 7) == 0);
+        if constexpr (std::is_same<T, float>::value) {
+            if (pairs) {
+#define HYB_DEPR(O) HYB_CUDA_TRY((launch_runs<O>(g, J1, J2, J3, cell, off_old, off_new, v3, q, np, c1, c2, c3)))
+                if (order == 1) HYB_DEPR(1); else if (order == 2) HYB_DEPR(2); else HYB_DEPR(3);
+#undef HYB_DEPR
+                return HYB_OK;
+            }
+        }
+        // small calls: smaller blocks, so that the particles spread over the SMs
+        int threads = kDepThreads;
+        while (threads > 32 && np < (int64_t)threads * dev_sms) threads >>= 1;
+        const unsigned blocks = (unsigned)std::min<int64_t>((np + threads - 1) / threads, (int64_t)dev_sms * 32);
 #define HYB_DEP2(O) k_deposit2d<T, O><<<blocks, threads, 0, g->stream>>>(J1, J2, J3, d.n1, d.n2, cell, off_old, off_new, v3, q, np, c1, c2, c3, g->dflag)
         if (order == 1) HYB_DEP2(1); else if (order == 2) HYB_DEP2(2); else HYB_DEP2(3);
 #undef HYB_DEP2
     } else {
+        const int threads = kDepThreads;
+        const unsigned blocks = (unsigned)std::min<int64_t>((np + threads - 1) / threads, (int64_t)dev_sms * 32);
         const T c1 = (T)(-1.0 / (d.dt * d.dx2 * d.dx3)), c2 = (T)(-1.0 / (d.dt * d.dx1 * d.dx3)), c3 = (T)(-1.0 / (d.dt * d.dx1 * d.dx2));
 #define HYB_DEP3(O) k_deposit3d<T, O><<<blocks, threads, 0, g->stream>>>(J1, J2, J3, d.n1, d.n2, d.n3, cell, off_old, off_new, q, np, c1, c2, c3, g->dflag)
         if (order == 1) HYB_DEP3(1); else if (order == 2) HYB_DEP3(2); else HYB_DEP3(3);
