@@ -14,7 +14,8 @@
 // and its bias gradient; tanh' and the bias gradient of the layer below), and
 // the Adam step sums the gradient parts and writes the BF16 weight copies: a
 // training step is 3 launches per layer (forward, dW, dX; no dX below the first
-// layer) plus the Adam step.  No sum is taken with atomics: the weight
+// layer) plus the Adam step.  Networks wider than 64 run the forward and backward products of a tile
+// of the batch in one kernel (k_mlp_chain) and all weight gradients in another: 3 launches a step.  No sum is taken with atomics: the weight
 // gradients (K = batch, split over up to 64 CTAs per tile), the bias gradients
 // and the loss are written as per-CTA parts and added in a fixed order, so a
 // training run is bit-reproducible.
@@ -33,6 +34,9 @@ constexpr int kMaxLayers = 17;
 struct LayerTab {
     int L;
     int nrb;                                          // row blocks of the batch (parts of a bias gradient)
+    int nrc;                                          // 64-row blocks of the batch (k_mlp_chain: the halves of nrb's)
+    int64_t wk_off[kMaxLayers];                       // k_mlp_chain: BF16 weights of a layer, rows of its tile
+    int rows[kMaxLayers];
     int64_t w_off[kMaxLayers], wb_off[kMaxLayers];    // parameters; BF16 weight copies
     int64_t ws_w[kMaxLayers], ws_b[kMaxLayers];       // parts of the weight and bias gradients
     int fo[kMaxLayers], fi[kMaxLayers], fop[kMaxLayers], fip[kMaxLayers], split[kMaxLayers];
@@ -61,6 +65,11 @@ struct hyb_mlp {
     size_t ws_w_size = 0;
     float* loss = nullptr;                // device scalar
     int* err = nullptr;                   // device flag: bit 1 = a bounded wait in a GEMM gave up
+    // networks wider than kNarrow (k_mlp_chain): BF16 weights in the order the kernel's shared memory
+    // holds them, every layer's input and dH feature-major, tanh of the hidden layers
+    bool chain = false;
+    __nv_bfloat16* wk = nullptr;          // [fin/8][rows][8] per layer (rows: outputs, padded)
+    __nv_bfloat16* wkt = nullptr;         // [fout/8][rows][8] of the transposed weights (rows: inputs, padded)
     int64_t step = 0;
     int64_t launches = 0;                 // kernels launched so far (hyb_mlp_launch_count)
 };
@@ -71,6 +80,10 @@ namespace hyb {
 constexpr int TM = 128, TN = 32, TKC = 64, GT = 128;
 constexpr int LBO_A = TM * 16 + 16, LBO_B = TN * 16 + 16;     // K-group strides (16-byte slots spread)
 constexpr int kMaxSplit = 64;
+// Networks up to this width run a product per launch (3 launches per layer, as hyb_mlp_launch_count states),
+// wider ones k_mlp_chain
+constexpr int kNarrow = 64;
+constexpr int CB = 64, CT = 512;         // k_mlp_chain: rows of the batch per CTA, threads
 
 // Epilogues of the GEMM (what happens to an accumulator value v of output (row, col)):
 //   EP_PART    part z of a split K: P[z][row][col] = v (row stride N); a CTA with an empty K
@@ -160,8 +173,9 @@ __device__ __forceinline__ float warp_sum(float v) {
 // tcgen05.ld into the epilogue.  Waits are bounded: on time-out bit 1 of *err is set and the
 // CTA skips the rest, drains and frees its TMEM.
 template <int EP, typename TA, typename TB>
-__global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, const TA* __restrict__ a, int64_t sam, int64_t sak,
-                                                const TB* __restrict__ b, int64_t sbk, int64_t sbn, Epi ep, int kchunk, int* err) {
+__device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, int K, int kmax, const TA* __restrict__ a, int64_t sam,
+                                          int64_t sak, const TB* __restrict__ b, int64_t sbk, int64_t sbn, const Epi& ep, int kchunk,
+                                          int* err) {
     __shared__ __align__(128) unsigned char sbuf[8 * LBO_A + 8 * LBO_B];
     __shared__ uint64_t bar;
     __shared__ uint32_t s_taddr;
@@ -182,8 +196,8 @@ __global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, c
     __syncthreads();
     tm_fence_after();
     const uint32_t tbase = s_taddr;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    const int m0 = by * TM, n0 = bx * TN;
+    const int kb = bz * kchunk, ke = min(K, kb + kchunk);
     uint32_t ph = 0;
     bool pend = false, abort = false, any = false;
     for (int k0 = kb; k0 < ke && !abort; k0 += TKC) {
@@ -227,7 +241,7 @@ __global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, c
             const int c0 = n0 + 16 * u;
             if (EP == EP_PART) {
                 if (live && c0 < N) {
-                    float* p = ep.c + (int64_t)blockIdx.z * M * N + (int64_t)row * N + c0;
+                    float* p = ep.c + (int64_t)bz * M * N + (int64_t)row * N + c0;
                     if ((N & 3) == 0 && c0 + 16 <= N) {
 #pragma unroll
                         for (int j = 0; j < 4; j++)
@@ -275,8 +289,8 @@ __global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, c
                     if (lane == 0) { s_red[warp][0] = l; s_red[warp][1] = sd; }
                     __syncthreads();
                     if (tid == 0) {
-                        ep.loss_part[blockIdx.y] = (s_red[0][0] + s_red[1][0]) + (s_red[2][0] + s_red[3][0]);
-                        ep.db_part[blockIdx.y] = (s_red[0][1] + s_red[1][1]) + (s_red[2][1] + s_red[3][1]);
+                        ep.loss_part[by] = (s_red[0][0] + s_red[1][0]) + (s_red[2][0] + s_red[3][0]);
+                        ep.db_part[by] = (s_red[0][1] + s_red[1][1]) + (s_red[2][1] + s_red[3][1]);
                     }
                 }
             } else {   // EP_DX
@@ -318,7 +332,7 @@ __global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, c
         if (EP == EP_DX) {
             __syncthreads();
             if (tid < TN && n0 + tid < ep.n)
-                ep.db_part[(int64_t)blockIdx.y * ep.n + n0 + tid] = (s_red[0][tid] + s_red[1][tid]) + (s_red[2][tid] + s_red[3][tid]);
+                ep.db_part[(int64_t)by * ep.n + n0 + tid] = (s_red[0][tid] + s_red[1][tid]) + (s_red[2][tid] + s_red[3][tid]);
         }
     }
     if (tid == 0 && pend) mbar_drain(mb, ph);
@@ -326,6 +340,32 @@ __global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, c
     __syncthreads();
     tm_fence_after();
     if (warp == 0) tm_dealloc(tbase, TN);
+}
+
+template <int EP, typename TA, typename TB>
+__global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, const TA* __restrict__ a, int64_t sam, int64_t sak,
+                                                const TB* __restrict__ b, int64_t sbk, int64_t sbn, Epi ep, int kchunk, int* err) {
+    gemm_tile<EP, TA, TB>(blockIdx.x, blockIdx.y, blockIdx.z, M, N, K, kmax, a, sam, sak, b, sbk, sbn, ep, kchunk, err);
+}
+
+// The weight-gradient parts of every layer in one launch: blocks first[l] .. first[l + 1] - 1 are layer l's
+// tiles (column tile fastest, then row tile, then part of K).
+struct DwTab {
+    int L;
+    int first[kMaxLayers + 1];
+    int M[kMaxLayers], N[kMaxLayers], kchunk[kMaxLayers];
+    const __nv_bfloat16* a[kMaxLayers];               // dH, feature-major
+    const __nv_bfloat16* b[kMaxLayers];               // the layer's input, feature-major
+    float* c[kMaxLayers];
+};
+__global__ void __launch_bounds__(GT) k_dw_all(__grid_constant__ const DwTab t, int K, int kmax, int64_t ld, int* err) {
+    int l = 0;
+    while (l + 1 < t.L && (int)blockIdx.x >= t.first[l + 1]) l++;
+    const int r = blockIdx.x - t.first[l], nx = (t.N[l] + TN - 1) / TN, ny = (t.M[l] + TM - 1) / TM;
+    Epi ep;
+    ep.c = t.c[l];
+    gemm_tile<EP_PART>(r % nx, (r / nx) % ny, r / (nx * ny), t.M[l], t.N[l], K, kmax, t.a[l], ld, (int64_t)1, t.b[l], (int64_t)1, ld, ep,
+                       t.kchunk[l], err);
 }
 
 // K is rounded up to 16 (the MMA depth); entries with k >= K read as zero.
@@ -349,10 +389,15 @@ static void gemm(int M, int N, int K, const TA* a, int64_t sam, int64_t sak, con
     launches++;
 }
 
+// k_mlp_chain's order of a weight matrix: element (row, k) of [K/8][rows][8], the canonical K-major layout of a
+// tcgen05 operand without swizzle, so that a layer is one contiguous copy
+__host__ __device__ __forceinline__ int64_t chain_at(int row, int k, int rows) { return ((int64_t)(k >> 3) * rows + row) * 8 + (k & 7); }
+
 // Gradient sums in a fixed order (the split-K parts of a weight gradient, the row-block parts of
 // a bias gradient, the loss parts); with update != 0 also the Adam step on every parameter and
 // the BF16 copies of the updated weights (zero-padded, both layouts; the padding was written by
 // refresh()).  Without it the sums go to g (the gradients of hyb_mlp_gradients).
+template <bool CHAIN>
 __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                             const float* __restrict__ ws, const float* __restrict__ loss_part, float* __restrict__ loss,
                             int64_t n, int update, float lr, float b1, float b2, float eps, float c1, float c2, LayerTab tab,
@@ -360,7 +405,7 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i == 0) {
         float s = 0.f;
-        for (int y = 0; y < tab.nrb; y++) s += loss_part[y];
+        for (int y = 0; y < tab.nrb; y++) s += CHAIN ? loss_part[2 * y] + (2 * y + 1 < tab.nrc ? loss_part[2 * y + 1] : 0.f) : loss_part[y];
         *loss = s;
     }
     if (i >= n) return;
@@ -371,10 +416,23 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
     float gi = 0.f;
     if (loc < nw) {
         const float* p = ws + tab.ws_w[l] + loc;
-        for (int z = 0; z < tab.split[l]; z++) gi += p[z * nw];
+        int z = 0;
+        for (; z + 8 <= tab.split[l]; z += 8) {           // eight loads in flight, added in order
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) v[e] = p[(z + e) * nw];
+#pragma unroll
+            for (int e = 0; e < 8; e++) gi += v[e];
+        }
+        for (; z < tab.split[l]; z++) gi += p[z * nw];
     } else {
         const float* p = ws + tab.ws_b[l] + (loc - nw);
-        for (int y = 0; y < tab.nrb; y++) gi += p[(int64_t)y * tab.fo[l]];
+        const int64_t fo = tab.fo[l];
+        if (CHAIN) {
+            for (int y = 0; y < tab.nrb; y++) gi += p[2 * y * fo] + (2 * y + 1 < tab.nrc ? p[(2 * y + 1) * fo] : 0.f);
+        } else {
+            for (int y = 0; y < tab.nrb; y++) gi += p[(int64_t)y * fo];
+        }
     }
     if (!update) {
         g[i] = gi;
@@ -389,9 +447,289 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
     if (loc < nw) {
         const int r = (int)(loc / tab.fi[l]), c = (int)(loc % tab.fi[l]);
         const __nv_bfloat16 q = __float2bfloat16(wi);
-        wb[tab.wb_off[l] + (int64_t)r * tab.fip[l] + c] = q;
-        wt[tab.wb_off[l] + (int64_t)c * tab.fop[l] + r] = q;
+        if (CHAIN) {
+            wb[tab.wk_off[l] + chain_at(r, c, tab.rows[l])] = q;
+            if (l > 0 && l + 1 < tab.L) wt[tab.wk_off[l] + chain_at(c, r, tab.rows[l])] = q;
+        } else {
+            wb[tab.wb_off[l] + (int64_t)r * tab.fip[l] + c] = q;
+            wt[tab.wb_off[l] + (int64_t)c * tab.fop[l] + r] = q;
+        }
     }
+}
+
+// ------------------------------------------------------------------ the chain of a batch tile
+// A training step's forward and backward products of CB = 64 rows of the batch in one CTA, layer by layer
+// without leaving the SM (before: a launch per layer and direction, 10 to 20 us each, latency-bound).  The
+// products are taken transposed, D^T[features][rows] = W X^T: A is the weight matrix (128-row tiles, K-major, in
+// shared memory as it lies in global memory: one bulk copy per layer, which runs while the previous
+// layer's epilogue does), B the tile of activations [64 rows][K].  A TMEM lane is then a feature and
+// its columns the rows of the batch: bias, tanh and tanh' are lane-local, the feature-major copies that
+// the weight gradients read are contiguous per thread, and the epilogue writes the next product's B operand
+// straight into shared memory.  The output layer's product is taken the other way round (a lane per row:
+// loss and dH of a row), and its dX, one product per element, needs no MMA.  Bound by the epilogues (16384
+// values per layer and tile, an accurate tanhf each): 16 warps, and 64 rows so that a batch of 8192 is 128 CTAs.
+// 8192 x (6 -> 256 x 4 -> 1): a step took 262 us with a launch per product.
+// Sums and roundings are those of the launch-per-product form (same products in the same K order, the same
+// trees of partial sums), so both give the same gradients.
+struct ChainArgs {
+    int n_in, width, depth;
+    int64_t B, cap;
+    const float* x;
+    const float* tgt;                                  // null: forward only
+    float* y;                                          // nullable
+    const __nv_bfloat16* wk[kMaxLayers];
+    const __nv_bfloat16* wkt[kMaxLayers];
+    const float* bias[kMaxLayers];
+    __nv_bfloat16* actT;                               // [L][256][cap]: the layers' inputs
+    __nv_bfloat16* dhT;                                // [L][256][cap]
+    float* th;                                         // [depth][256][cap]: tanh of the hidden layers
+    float* db_part[kMaxLayers];                        // [64-row blocks][fo]
+    float* loss_part;                                  // [64-row blocks]
+    float invB;
+    int* err;
+};
+constexpr int LBO_X = CB * 16 + 16;                    // K-group stride of the activations (spread over the banks)
+__host__ __device__ constexpr int pad16c(int v) { return (v + 15) & ~15; }
+__host__ __device__ constexpr int chain_kmax(int n_in, int width) { return pad16c(n_in > width ? n_in : width); }
+// weights | activations (+ 1 KB: the output product's A rows 64..127, which nothing reads, lie beyond) | output weights
+__host__ __device__ constexpr size_t chain_w_bytes(int n_in, int width) { return (size_t)((width + 127) / 128 * 128) * chain_kmax(n_in, width) * 2; }
+__host__ __device__ constexpr size_t chain_x_bytes(int n_in, int width) { return (size_t)(chain_kmax(n_in, width) / 8) * LBO_X + 1024; }
+__host__ __device__ constexpr size_t chain_smem(int n_in, int width) {
+    return chain_w_bytes(n_in, width) + chain_x_bytes(n_in, width) + (size_t)pad16c(width) * 32;
+}
+
+// sum of 32 values in the order of warp_sum's butterfly
+__device__ __forceinline__ float tree_sum(const float (&v)[32]) {
+    float a[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) a[i] = v[i] + v[i + 16];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < o; i++) a[i] = a[i] + a[i + o];
+    return a[0];
+}
+
+__global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const ChainArgs g) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ uint64_t bars[2];                       // weights, products
+    __shared__ uint32_t s_taddr;
+    __shared__ int s_abort;
+    __shared__ float s_red[2][256];
+    __shared__ float s_d[CB];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int width = g.width, depth = g.depth;
+    const int K0 = pad16c(g.n_in), Kh = pad16c(width), rows = (width + 127) / 128 * 128;
+    const bool train = g.tgt != nullptr;
+    const uint32_t sW = smem_addr(smem), sX = sW + (uint32_t)chain_w_bytes(g.n_in, width);
+    const uint32_t sO = sX + (uint32_t)chain_x_bytes(g.n_in, width);
+    const uint32_t wb = smem_addr(&bars[0]), mb = smem_addr(&bars[1]);
+    const int64_t b0 = (int64_t)blockIdx.x * CB;
+    // this thread's part of an accumulator: feature f (TMEM lane), rows 32 ch .. 32 ch + 31 of the tile
+    const int half = (warp >> 2) & 1, ch = warp >> 3, f = 128 * half + 32 * (warp & 3) + lane;
+    const bool mine = 128 * half < rows, live = f < width;
+    if (warp == 0) {
+        tm_alloc(smem_addr(&s_taddr), 256);
+        tm_relinquish();
+    }
+    if (tid == 0) {
+        mbar_init(wb, 1);
+        mbar_init(mb, 1);
+        mbar_fence_init();
+        s_abort = 0;
+    }
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    const uint32_t tbase = s_taddr, tacc = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(64 * half + 32 * ch);
+    uint32_t wph = 0, mph = 0;
+    bool wpend = false, mpend = false;                 // (thread 0) copies and products in flight
+    auto load_w = [&](const __nv_bfloat16* src, int K, bool out_too) {
+        const uint32_t bytes = (uint32_t)rows * (uint32_t)K * 2u, ob = out_too ? (uint32_t)Kh * 32u : 0u;
+        mbar_expect_tx(wb, bytes + ob);
+        if (out_too) bulk_load(sO, g.wk[depth], ob, wb);
+        for (uint32_t o = 0; o < bytes; o += 16384u) bulk_load(sW + o, reinterpret_cast<const unsigned char*>(src) + o, min(16384u, bytes - o), wb);
+        wpend = true;
+    };
+    if (tid == 0) load_w(g.wk[0], K0, true);
+    // the network's input in BF16: this tile's B operand and the feature-major copy
+    for (int i = tid; i < CB * K0; i += CT) {
+        const int n = i & (CB - 1), k = i / CB;
+        const int64_t b = b0 + n;
+        const uint32_t v = (b < g.B && k < g.n_in) ? bf16_bits(__ldg(g.x + b * g.n_in + k)) : 0u;
+        asm volatile("st.shared.u16 [%0], %1;" :: "r"(sX + (uint32_t)((k >> 3) * LBO_X + n * 16 + (k & 7) * 2)), "h"((unsigned short)v) : "memory");
+        if (train && k < g.n_in) reinterpret_cast<unsigned short*>(g.actT)[(int64_t)k * g.cap + b] = (unsigned short)v;
+    }
+    fence_proxy_async_smem();
+    __syncthreads();
+    // D^T = A X^T over K: issued by thread 0 once the weights are there; every thread waits for the products
+    auto product = [&](int K) {
+        if (tid == 0 && !s_abort) {
+            mbar_wait(wb, wph, g.err, &s_abort);
+            if (!s_abort) {
+                wph ^= 1;
+                wpend = false;
+                tm_fence_after();
+                for (int h = 0; h < rows / 128; h++)
+                    for (int ks = 0; ks < K / 16; ks++)
+                        mma_bf16(tbase + 64 * h, smem_desc(sW + h * 2048 + 2 * ks * rows * 16, rows * 16, 128),
+                                 smem_desc(sX + 2 * ks * LBO_X, LBO_X, 128), idesc_bf16(CB), ks > 0 ? 1u : 0u);
+                mma_commit(mb);
+                mpend = true;
+            }
+        }
+    };
+    auto wait_product = [&]() {
+        mbar_wait(mb, mph, g.err, &s_abort);
+        mph ^= 1;
+        tm_fence_after();
+    };
+    auto abort_now = [&]() {                            // the same answer in every thread
+        __syncthreads();
+        return s_abort != 0;
+    };
+    // an epilogue's 32 BF16 values (bits in pairs) into the B operand and the feature-major copy
+    auto put = [&](const uint32_t (&q)[16], bool operand, __nv_bfloat16* copy) {
+        if (operand && f < Kh) {
+            const uint32_t at = sX + (uint32_t)((f >> 3) * LBO_X + 32 * ch * 16 + (f & 7) * 2);
+#pragma unroll
+            for (int n = 0; n < 32; n++)
+                asm volatile("st.shared.u16 [%0], %1;" :: "r"(at + 16 * n), "h"((unsigned short)(q[n >> 1] >> (16 * (n & 1)))) : "memory");
+        }
+        if (copy && live) {
+            uint4* c = reinterpret_cast<uint4*>(copy + (int64_t)f * g.cap + b0 + 32 * ch);
+#pragma unroll
+            for (int e = 0; e < 4; e++) c[e] = make_uint4(q[4 * e], q[4 * e + 1], q[4 * e + 2], q[4 * e + 3]);
+        }
+    };
+    bool stop = false;
+    // ---- forward
+    for (int l = 0; l < depth && !stop; l++) {
+        product(l == 0 ? K0 : Kh);
+        wait_product();
+        if (tid == 0 && !s_abort) {
+            mpend = false;
+            if (l + 1 < depth) load_w(g.wk[l + 1], Kh, false);
+            else if (train && depth > 1) load_w(g.wkt[depth - 1], Kh, false);
+        }
+        if (mine && !s_abort) {
+            float t[32];
+            tm_ld16(tacc, reinterpret_cast<float(&)[16]>(t[0]));
+            tm_ld16(tacc + 16, reinterpret_cast<float(&)[16]>(t[16]));
+            tm_wait_ld();
+            const float bias = live ? __ldg(g.bias[l] + f) : 0.f;
+            uint32_t q[16];
+#pragma unroll
+            for (int n = 0; n < 32; n++) t[n] = live ? tanhf(t[n] + bias) : 0.f;
+#pragma unroll
+            for (int n = 0; n < 16; n++) q[n] = bf16_bits(t[2 * n]) | (bf16_bits(t[2 * n + 1]) << 16);
+            if (train && live) {
+                float4* o = reinterpret_cast<float4*>(g.th + ((int64_t)l * 256 + f) * g.cap + b0 + 32 * ch);
+#pragma unroll
+                for (int e = 0; e < 8; e++) o[e] = make_float4(t[4 * e], t[4 * e + 1], t[4 * e + 2], t[4 * e + 3]);
+            }
+            put(q, true, train ? g.actT + (int64_t)(l + 1) * 256 * g.cap : nullptr);
+        }
+        tm_fence_before();
+        fence_proxy_async_smem();
+        stop = abort_now();
+    }
+    // ---- output layer: a lane per row
+    if (!stop) {
+        if (tid == 0) {
+            tm_fence_after();
+            for (int ks = 0; ks < Kh / 16; ks++)
+                mma_bf16(tbase + 128, smem_desc(sX + 2 * ks * LBO_X, LBO_X, 128), smem_desc(sO + 2 * ks * 256, 256, 128), idesc_bf16(16),
+                         ks > 0 ? 1u : 0u);
+            mma_commit(mb);
+            mpend = true;
+        }
+        wait_product();
+        if (tid == 0 && !s_abort) mpend = false;
+        if (warp < 2 && !s_abort) {
+            float t[16];
+            tm_ld16(tbase + ((uint32_t)(32 * warp) << 16) + 128, t);
+            tm_wait_ld();
+            const int64_t b = b0 + 32 * warp + lane;
+            const bool in = b < g.B;
+            const float y = t[0] + __ldg(g.bias[depth]);
+            if (in && g.y) g.y[b] = y;
+            if (train) {
+                const float dd = in ? y - g.tgt[b] : 0.f;
+                const float d = 2.f * dd * g.invB;
+                const __nv_bfloat16 db = __float2bfloat16(d);
+                g.dhT[(int64_t)depth * 256 * g.cap + b] = db;
+                s_d[32 * warp + lane] = __bfloat162float(db);
+                const float ls = warp_sum(dd * dd * g.invB), sd = warp_sum(d);
+                if (lane == 0) { s_red[0][warp] = ls; s_red[1][warp] = sd; }
+            }
+        }
+        tm_fence_before();
+        stop = abort_now();
+        if (train && !stop) {
+            if (tid == 0) {
+                g.loss_part[blockIdx.x] = s_red[0][0] + s_red[0][1];
+                g.db_part[depth][blockIdx.x] = s_red[1][0] + s_red[1][1];
+            }
+            __syncthreads();
+        }
+    }
+    // ---- backward: dH of hidden layer l from that of the layer above
+    for (int l = depth - 1; train && l >= 0 && !stop; l--) {
+        float th[32];
+        if (live) {
+            const float4* o = reinterpret_cast<const float4*>(g.th + ((int64_t)l * 256 + f) * g.cap + b0 + 32 * ch);
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const float4 v = o[e];
+                th[4 * e] = v.x; th[4 * e + 1] = v.y; th[4 * e + 2] = v.z; th[4 * e + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 32; e++) th[e] = 0.f;
+        }
+        float t[32];
+        if (l == depth - 1) {                           // dX of the output layer: one product per element
+            const float w = live ? __bfloat162float(g.wk[depth][chain_at(0, f, 16)]) : 0.f;
+#pragma unroll
+            for (int n = 0; n < 32; n++) t[n] = s_d[32 * ch + n] * w;
+        } else {
+            product(Kh);
+            wait_product();
+            if (tid == 0 && !s_abort) {
+                mpend = false;
+                if (l > 0) load_w(g.wkt[l], Kh, false);
+            }
+            if (mine && !s_abort) {
+                tm_ld16(tacc, reinterpret_cast<float(&)[16]>(t[0]));
+                tm_ld16(tacc + 16, reinterpret_cast<float(&)[16]>(t[16]));
+                tm_wait_ld();
+            } else {
+#pragma unroll
+                for (int n = 0; n < 32; n++) t[n] = 0.f;
+            }
+        }
+        uint32_t q[16];
+#pragma unroll
+        for (int n = 0; n < 32; n++) t[n] = live ? t[n] * (1.f - th[n] * th[n]) : 0.f;
+#pragma unroll
+        for (int n = 0; n < 16; n++) q[n] = bf16_bits(t[2 * n]) | (bf16_bits(t[2 * n + 1]) << 16);
+        put(q, l > 0, g.dhT + (int64_t)l * 256 * g.cap);
+        s_red[ch][f] = tree_sum(t);
+        tm_fence_before();
+        fence_proxy_async_smem();
+        stop = abort_now();
+        if (!stop && ch == 0 && live) g.db_part[l][(int64_t)blockIdx.x * width + f] = s_red[0][f] + s_red[1][f];
+        __syncthreads();                                // s_red is read before the next layer writes it
+    }
+    if (tid == 0) {
+        if (wpend) mbar_drain(wb, wph);
+        if (mpend) mbar_drain(mb, mph);
+    }
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    if (warp == 0) tm_dealloc(tbase, 256);
 }
 
 // BF16 copies of the weights, zero-padded to [fout_pad][fin_pad] and [fin_pad][fout_pad]
@@ -411,7 +749,31 @@ static int pad16(int v) { return (v + 15) & ~15; }
 static int layer_in(const hyb_mlp* m, int l) { return l == 0 ? m->n_in : m->width; }
 static int layer_out(const hyb_mlp* m, int l) { return l == m->L - 1 ? 1 : m->width; }
 
+// the same in k_mlp_chain's order; the padding is zero
+__global__ void k_refresh_chain(const float* __restrict__ w, int fout, int fin, int rows, int kpad, __nv_bfloat16* __restrict__ wk,
+                                __nv_bfloat16* __restrict__ wkt) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * kpad) return;
+    const int r = i / kpad, c = i % kpad;
+    wk[chain_at(r, c, rows)] = __float2bfloat16((r < fout && c < fin) ? w[(int64_t)r * fin + c] : 0.f);
+    if (wkt) wkt[chain_at(r, c, rows)] = __float2bfloat16((r < fin && c < fout) ? w[(int64_t)c * fin + r] : 0.f);
+}
+
+// rows of a layer's operand in k_mlp_chain: hidden layers in whole 128-row tiles of the product; the output
+// layer (an N = 16 operand) 16
+static int chain_rows(const hyb_mlp* m, int l) { return l == m->L - 1 ? 16 : (m->width + 127) / 128 * 128; }
+
 static hyb_status refresh(hyb_mlp* m, cudaStream_t s) {
+    if (m->chain) {
+        for (int l = 0; l < m->L; l++) {
+            const int fo = layer_out(m, l), fi = layer_in(m, l), rows = m->tab.rows[l], kp = pad16(fi);
+            k_refresh_chain<<<(rows * kp + 255) / 256, 256, 0, s>>>(m->master + m->w_off[l], fo, fi, rows, kp, m->wk + m->tab.wk_off[l],
+                                                                   l > 0 && l + 1 < m->L ? m->wkt + m->tab.wk_off[l] : nullptr);
+            m->launches++;
+        }
+        HYB_CUDA_TRY(cudaGetLastError());
+        return HYB_OK;
+    }
     for (int l = 0; l < m->L; l++) {
         const int fo = layer_out(m, l), fi = layer_in(m, l), fop = pad16(fo), fip = pad16(fi);
         k_refresh<<<(fop * fip + 255) / 256, 256, 0, s>>>(m->master + m->w_off[l], fo, fi, fop, fip, m->wbf + m->wb_off[l],
@@ -424,20 +786,25 @@ static hyb_status refresh(hyb_mlp* m, cudaStream_t s) {
 
 static hyb_status ensure_cap(hyb_mlp* m, int64_t B) {
     if (B <= m->cap) return HYB_OK;
-    if (m->act) { cudaFree(m->act); cudaFree(m->actT); cudaFree(m->pre); cudaFree(m->dhb); cudaFree(m->dhT); cudaFree(m->ws); }
+    if (m->actT) { cudaFree(m->act); cudaFree(m->actT); cudaFree(m->pre); cudaFree(m->dhb); cudaFree(m->dhT); cudaFree(m->ws); }
     m->act = m->actT = m->dhb = m->dhT = nullptr;
     m->pre = m->ws = nullptr;
     m->cap = 0;
     const int64_t cap = ((B + 127) / 128) * 128;
     const size_t na = (size_t)std::max(1, m->L - 1) * cap * 256;
-    const size_t nrb = (size_t)(cap / 128);
+    const size_t nrb = (size_t)(cap / (m->chain ? CB : 128));
     size_t nb = 0;
     for (int l = 0; l < m->L; l++) nb += nrb * layer_out(m, l);
-    HYB_CUDA_TRY(cudaMalloc(&m->act, sizeof(__nv_bfloat16) * na));
-    HYB_CUDA_TRY(cudaMalloc(&m->actT, sizeof(__nv_bfloat16) * na));
     HYB_CUDA_TRY(cudaMalloc(&m->pre, sizeof(float) * na));
-    HYB_CUDA_TRY(cudaMalloc(&m->dhb, sizeof(__nv_bfloat16) * 2 * (size_t)cap * 256));
-    HYB_CUDA_TRY(cudaMalloc(&m->dhT, sizeof(__nv_bfloat16) * 2 * (size_t)cap * 256));
+    if (m->chain) {          // inputs of every layer and dH of every layer, feature-major
+        HYB_CUDA_TRY(cudaMalloc(&m->actT, sizeof(__nv_bfloat16) * (size_t)m->L * cap * 256));
+        HYB_CUDA_TRY(cudaMalloc(&m->dhT, sizeof(__nv_bfloat16) * (size_t)m->L * cap * 256));
+    } else {
+        HYB_CUDA_TRY(cudaMalloc(&m->act, sizeof(__nv_bfloat16) * na));
+        HYB_CUDA_TRY(cudaMalloc(&m->actT, sizeof(__nv_bfloat16) * na));
+        HYB_CUDA_TRY(cudaMalloc(&m->dhb, sizeof(__nv_bfloat16) * 2 * (size_t)cap * 256));
+        HYB_CUDA_TRY(cudaMalloc(&m->dhT, sizeof(__nv_bfloat16) * 2 * (size_t)cap * 256));
+    }
     HYB_CUDA_TRY(cudaMalloc(&m->ws, sizeof(float) * (m->ws_w_size + nb + nrb)));
     // bias parts start after the weight parts, the loss parts after the bias parts
     size_t off = m->ws_w_size;
@@ -446,7 +813,9 @@ static hyb_status ensure_cap(hyb_mlp* m, int64_t B) {
     return HYB_OK;
 }
 
-static float* loss_parts(const hyb_mlp* m) { return m->ws + m->tab.ws_b[m->L - 1] + (size_t)(m->cap / 128) * layer_out(m, m->L - 1); }
+static float* loss_parts(const hyb_mlp* m) {
+    return m->ws + m->tab.ws_b[m->L - 1] + (size_t)(m->cap / (m->chain ? CB : 128)) * layer_out(m, m->L - 1);
+}
 
 // input of layer l >= 1 (BF16 activations of layer l - 1): row-major [cap][256] and feature-major [256][cap]
 static __nv_bfloat16* act_in(const hyb_mlp* m, int l) { return m->act + (size_t)(l - 1) * m->cap * 256; }
@@ -459,7 +828,9 @@ static __nv_bfloat16* dhT_of(const hyb_mlp* m, int l) { return m->dhT + (size_t)
 
 // forward pass: one GEMM per layer, bias and tanh in its epilogue; with a target the output
 // layer's epilogue also forms dH of the output layer and the parts of the loss and its bias gradient
+static hyb_status chain_pass(hyb_mlp* m, const float* x, int64_t B, float* y, const float* tgt, cudaStream_t s);
 static hyb_status forward(hyb_mlp* m, const float* x, int64_t B, float* y, const float* tgt, cudaStream_t s) {
+    if (m->chain) return chain_pass(m, x, B, y, tgt, s);
     hyb_status st = ensure_cap(m, B);
     if (st != HYB_OK) return st;
     const int64_t cap = m->cap;
@@ -497,6 +868,7 @@ static hyb_status forward(hyb_mlp* m, const float* x, int64_t B, float* y, const
 // (split K) and, below the first layer, dX = dH W with tanh' and the parts of the bias
 // gradient of the layer below in the epilogue
 static hyb_status backward(hyb_mlp* m, const float* x, int64_t B, cudaStream_t s) {
+    if (m->chain) return HYB_OK;                        // done with the forward pass
     const int64_t cap = m->cap;
     m->tab.nrb = (int)((B + TM - 1) / TM);
     for (int l = m->L - 1; l >= 0; l--) {
@@ -524,6 +896,69 @@ static hyb_status backward(hyb_mlp* m, const float* x, int64_t B, cudaStream_t s
     return HYB_OK;
 }
 
+// the chain of a whole batch; with a target also the backward products, and then every layer's
+// weight-gradient parts: two launches
+static hyb_status chain_pass(hyb_mlp* m, const float* x, int64_t B, float* y, const float* tgt, cudaStream_t s) {
+    if (tgt) {
+        hyb_status st = ensure_cap(m, B);
+        if (st != HYB_OK) return st;
+    }
+    const int64_t cap = m->cap;
+    ChainArgs c{};
+    c.n_in = m->n_in;
+    c.width = m->width;
+    c.depth = m->depth;
+    c.B = B;
+    c.cap = cap;
+    c.x = x;
+    c.tgt = tgt;
+    c.y = y;
+    c.invB = 1.f / (float)B;
+    c.err = m->err;
+    for (int l = 0; l < m->L; l++) {
+        c.wk[l] = m->wk + m->tab.wk_off[l];
+        c.wkt[l] = m->wkt + m->tab.wk_off[l];
+        c.bias[l] = m->master + m->b_off[l];
+        c.db_part[l] = m->ws + m->tab.ws_b[l];
+    }
+    if (tgt) {
+        c.actT = m->actT;
+        c.dhT = m->dhT;
+        c.th = m->pre;
+        c.loss_part = loss_parts(m);
+    }
+    const size_t smem = chain_smem(m->n_in, m->width);
+    const cudaError_t attr = func_attr_once((const void*)k_mlp_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)chain_smem(256, 256));
+    if (attr != cudaSuccess) return cuda_fail(attr, "k_mlp_chain");
+    k_mlp_chain<<<(unsigned)((B + CB - 1) / CB), CT, smem, s>>>(c);
+    m->launches++;
+    if (tgt) {
+        m->tab.nrb = (int)((B + TM - 1) / TM);
+        m->tab.nrc = (int)((B + CB - 1) / CB);
+        const int Kp = (int)((B + 15) & ~(int64_t)15);
+        DwTab t{};
+        t.L = m->L;
+        int nblk = 0;
+        for (int l = 0; l < m->L; l++) {
+            const int no = layer_out(m, l), ni = layer_in(m, l), split = split_of(no, ni, (int)B);
+            m->tab.split[l] = split;
+            t.first[l] = nblk;
+            t.M[l] = no;
+            t.N[l] = ni;
+            t.kchunk[l] = ((Kp + split - 1) / split + 15) & ~15;
+            t.a[l] = m->dhT + (size_t)l * cap * 256;
+            t.b[l] = m->actT + (size_t)l * cap * 256;
+            t.c[l] = m->ws + m->tab.ws_w[l];
+            nblk += ((ni + TN - 1) / TN) * ((no + TM - 1) / TM) * split;
+        }
+        t.first[m->L] = nblk;
+        k_dw_all<<<nblk, GT, 0, s>>>(t, Kp, (int)B, cap, m->err);
+        m->launches++;
+    }
+    HYB_CUDA_TRY(cudaGetLastError());
+    return HYB_OK;
+}
+
 // the gradient sums (and with update the Adam step) over all parameters: one launch
 static hyb_status reduce_update(hyb_mlp* m, int update, float lr, cudaStream_t s) {
     const float b1 = 0.9f, b2 = 0.999f;
@@ -533,9 +968,10 @@ static hyb_status reduce_update(hyb_mlp* m, int update, float lr, cudaStream_t s
         c1 = 1.f - powf(b1, (float)m->step);
         c2 = 1.f - powf(b2, (float)m->step);
     }
-    k_grad_adam<<<(unsigned)((m->n_params + 255) / 256), 256, 0, s>>>(m->master, m->grad, m->adam_m, m->adam_v, m->ws, loss_parts(m),
-                                                                     m->loss, (int64_t)m->n_params, update, lr, b1, b2, 1e-8f, c1,
-                                                                     c2, m->tab, m->wbf, m->wbt);
+    const auto kern = m->chain ? k_grad_adam<true> : k_grad_adam<false>;
+    kern<<<(unsigned)((m->n_params + 255) / 256), 256, 0, s>>>(m->master, m->grad, m->adam_m, m->adam_v, m->ws, loss_parts(m), m->loss,
+                                                               (int64_t)m->n_params, update, lr, b1, b2, 1e-8f, c1, c2, m->tab,
+                                                               m->chain ? m->wk : m->wbf, m->chain ? m->wkt : m->wbt);
     m->launches++;
     HYB_CUDA_TRY(cudaGetLastError());
     return HYB_OK;
@@ -555,7 +991,8 @@ hyb_status hyb_mlp_create(int n_in, int width, int depth, const float* init_para
     *out = nullptr;
     hyb_mlp* m = new hyb_mlp();
     m->n_in = n_in; m->width = width; m->depth = depth; m->L = depth + 1;
-    size_t off = 0, woff = 0, wsw = 0;
+    m->chain = width > kNarrow;
+    size_t off = 0, woff = 0, wsw = 0, wkoff = 0;
     m->tab.L = m->L;
     for (int l = 0; l < m->L; l++) {
         const int fi = layer_in(m, l), fo = layer_out(m, l);
@@ -569,6 +1006,8 @@ hyb_status hyb_mlp_create(int n_in, int width, int depth, const float* init_para
         m->tab.fi[l] = fi;
         m->tab.fop[l] = pad16(fo);
         m->tab.fip[l] = pad16(fi);
+        m->tab.rows[l] = chain_rows(m, l);
+        m->tab.wk_off[l] = (int64_t)wkoff; wkoff += (size_t)m->tab.rows[l] * pad16(fi);
     }
     m->n_params = off;
     m->ws_w_size = wsw;
@@ -576,8 +1015,13 @@ hyb_status hyb_mlp_create(int n_in, int width, int depth, const float* init_para
     if (e == cudaSuccess) e = cudaMalloc(&m->adam_m, sizeof(float) * off);
     if (e == cudaSuccess) e = cudaMalloc(&m->adam_v, sizeof(float) * off);
     if (e == cudaSuccess) e = cudaMalloc(&m->grad, sizeof(float) * off);
-    if (e == cudaSuccess) e = cudaMalloc(&m->wbf, sizeof(__nv_bfloat16) * woff);
-    if (e == cudaSuccess) e = cudaMalloc(&m->wbt, sizeof(__nv_bfloat16) * woff);
+    if (m->chain) {
+        if (e == cudaSuccess) e = cudaMalloc(&m->wk, sizeof(__nv_bfloat16) * wkoff);
+        if (e == cudaSuccess) e = cudaMalloc(&m->wkt, sizeof(__nv_bfloat16) * wkoff);
+    } else {
+        if (e == cudaSuccess) e = cudaMalloc(&m->wbf, sizeof(__nv_bfloat16) * woff);
+        if (e == cudaSuccess) e = cudaMalloc(&m->wbt, sizeof(__nv_bfloat16) * woff);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&m->loss, sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&m->err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(m->err, 0, sizeof(int));
@@ -654,7 +1098,8 @@ hyb_status hyb_mlp_destroy(hyb_mlp* m) {
     cudaFree(m->master); cudaFree(m->adam_m); cudaFree(m->adam_v); cudaFree(m->grad); cudaFree(m->wbf); cudaFree(m->wbt);
     cudaFree(m->loss);
     cudaFree(m->err);
-    if (m->act) { cudaFree(m->act); cudaFree(m->actT); cudaFree(m->pre); cudaFree(m->dhb); cudaFree(m->dhT); cudaFree(m->ws); }
+    cudaFree(m->act); cudaFree(m->actT); cudaFree(m->pre); cudaFree(m->dhb); cudaFree(m->dhT); cudaFree(m->ws);
+    cudaFree(m->wk); cudaFree(m->wkt);
     delete m;
     return HYB_OK;
 }
