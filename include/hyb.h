@@ -163,7 +163,12 @@ HYB_API hyb_status hyb_push(hyb_grid* g, int32_t* cell, void* off, void* u, cons
  *   hyb_push with E^n, B^n (u^{n+1/2}, x^{n+1});  hyb_deposit (j^{n+1/2});
  *   hyb_advance (E^{n+1}, B^{n+1/2});  off <- off_new.
  * hyb_pic_create borrows g (which must stay bound to the same arrays) and
- * allocates a second grid of the same description and 9 scratch fields.
+ * allocates 3 scratch fields on the three-pass path (path 1), a second grid of
+ * the same description and 9 scratch fields on the others.  2D steps of at least
+ * 65536 particles list scattered particles cell by cell and visit them in that
+ * order; the list (an int per particle and per cell) is allocated by the first
+ * such step (not while the grid's stream is being captured: the particles are
+ * then visited as stored) and freed by hyb_pic_destroy.
  * When g is k1-resident (hyb_set_resident) the step takes B^n from the
  * resident spectra instead (B^{n-1/2} + Faraday(E^n)/2 per mode, transformed
  * into scratch), and its advance transforms only j forward: 12 row transforms
@@ -187,7 +192,7 @@ HYB_API hyb_status hyb_pic_create(hyb_grid* g, hyb_pic** out);
 HYB_API hyb_status hyb_pic_step(hyb_pic* p, int32_t* cell, void* off, void* u, const void* qm, const void* q,
                                 void* off_new, void* v3, int64_t np, int shape_order, int nsteps);
 
-/* Frees the PIC step's second grid and scratch (not g). */
+/* Frees the PIC step's second grid, scratch and list (not g). */
 HYB_API hyb_status hyb_pic_destroy(hyb_pic* p);
 
 /* Eq. currentcorrection alone, in place on the bound J1:

@@ -117,16 +117,18 @@ __device__ __forceinline__ void deposit_one(T* J1, T* J2, T* J3, int n1, int n2,
 // 2D, one thread per particle (FP64): lanes take particles BS / 32 apart within each chunk of BS, so
 // that for a sorted chunk the lanes of a warp sit in different (mostly consecutive) cells and their
 // atomic adds at the same window offset go to different, neighbouring addresses.
-template <typename T, int ORDER>
+template <typename T, int ORDER, bool VISIT>
 __global__ void __launch_bounds__(kDepThreads) k_deposit2d(T* __restrict__ J1, T* __restrict__ J2, T* __restrict__ J3,
                                                           int n1, int n2, const int32_t* __restrict__ cell,
                                                           const T* __restrict__ off0, const T* __restrict__ off1,
                                                           const T* __restrict__ v3, const T* __restrict__ q, int64_t np,
-                                                          T c1s, T c2s, T c3s, int* __restrict__ flag) {
+                                                          T c1s, T c2s, T c3s, int* __restrict__ flag, Visit visit) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int* const perm = VISIT ? visit_perm(visit) : nullptr;
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < np; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = base + lane * (int)(blockDim.x >> 5) + warp;
-        if (p >= np) continue;
+        const int64_t i = base + lane * (int)(blockDim.x >> 5) + warp;
+        if (i >= np) continue;
+        const int64_t p = visit_at(perm, i);
         const int cx = cell[2 * p], cy = cell[2 * p + 1];
         const T x0 = off0[2 * p], y0 = off0[2 * p + 1], x1 = off1[2 * p], y1 = off1[2 * p + 1];
         if (!move_ok(cx, cy, x0, x1, y0, y1, n1, n2)) {
@@ -211,16 +213,17 @@ __device__ __noinline__ void deposit_alone(float* J1, float* J2, float* J3, int 
 constexpr int kRunWarps = 4, kRunScan = 512;      // warps per block; particles looked at for 32 runs
 constexpr int kRunMax = 32;                       // a longer run is cut (at multiples of this many particles)
 
-template <int ORDER>
+template <int ORDER, bool VISIT>
 __global__ void __launch_bounds__(32 * kRunWarps, ORDER == 3 ? 3 : 4)
 k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restrict__ J3, int n1, int n2,
                  const int2* __restrict__ cell, const float2* __restrict__ off0, const float2* __restrict__ off1,
                  const float* __restrict__ v3, const float* __restrict__ q, int64_t np, int64_t per_warp, float c1s, float c2s,
-                 float c3s, int* __restrict__ flag) {
+                 float c3s, int* __restrict__ flag, Visit visit) {
     constexpr int WN = ORDER + 2, N = ORDER + 3, B0 = ORDER == 3 ? -2 : -1;
     __shared__ int s_start[kRunWarps][64];       // at most 32 + 32 heads
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* const start = s_start[warp];
+    const int* const perm = VISIT ? visit_perm(visit) : nullptr;
     const int64_t first = ((int64_t)blockIdx.x * kRunWarps + warp) * per_warp;
     const int64_t last = first + per_warp < np ? first + per_warp : np;
     int64_t base = first;
@@ -231,12 +234,12 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
         int2 carry = make_int2(0, 0);
         while (seen < avail && nr <= 32) {
             const int i = seen + lane;
-            const int2 c = i < avail ? cell[base + i] : make_int2(0, 0);
+            const int2 c = i < avail ? cell[visit_at(perm, base + i)] : make_int2(0, 0);
             {   // the rest of these particles into L2: two 128-byte lines of either offset array, one of q and v3
                 const int64_t g = base + seen + (lane & 1) * 16;
                 const void* line = lane < 2 ? (const void*)(off0 + g) : lane < 4 ? (const void*)(off1 + g)
                                    : lane == 4 ? (const void*)(q + g) : (const void*)(v3 + g);
-                if (g < last && lane < (v3 ? 7 : 5) && lane != 5) asm volatile("prefetch.global.L2 [%0];" :: "l"(line));
+                if (!perm && g < last && lane < (v3 ? 7 : 5) && lane != 5) asm volatile("prefetch.global.L2 [%0];" :: "l"(line));
             }
             int2 pc = make_int2(__shfl_up_sync(0xffffffffu, c.x, 1), __shfl_up_sync(0xffffffffu, c.y, 1));
             if (lane == 0) pc = carry;
@@ -251,7 +254,7 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
         const int runs = min(nr, 32);
         int end = nr > 32 ? start[32] : min(seen, avail);                   // particles of these runs
         const int s0 = lane < runs ? start[lane] : end, s1 = lane + 1 < runs ? start[lane + 1] : end;
-        const int2 cc = lane < runs ? cell[base + s0] : make_int2(-1, -1);
+        const int2 cc = lane < runs ? cell[visit_at(perm, base + s0)] : make_int2(-1, -1);
         const bool inside = cc.x >= 0 && cc.x < n1 && cc.y >= 0 && cc.y < n2;
         __syncwarp();
         // ---- which way: consecutive cells of a row; else by the sectors touched
@@ -267,12 +270,15 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
                 for (int i = 0; i < N; i++) a1[j][i] = a2[j][i] = a3[j][i] = 0.f;
             float2 n0 = make_float2(0.f, 0.f), nw = n0;
             float nq = 0.f, nv = 0.f;
+            int nat = VISIT && perm && s0 < s1 ? perm[base + s0] : 0;      // a listed particle's place, one fetch ahead
             auto fetch = [&](int i) {
                 if (i < s1) {
-                    n0 = off0[base + i];
-                    nw = off1[base + i];
-                    nq = q[base + i];
-                    nv = v3 ? v3[base + i] : 0.f;
+                    const int64_t p = VISIT && perm ? (int64_t)nat : base + i;
+                    if (VISIT && perm && i + 1 < s1) nat = perm[base + i + 1];
+                    n0 = off0[p];
+                    nw = off1[p];
+                    nq = q[p];
+                    nv = v3 ? v3[p] : 0.f;
                 }
             };
             fetch(s0);
@@ -364,14 +370,15 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
             // ---- scattered: a particle per lane
             if (end > 32) end &= ~31;                                // whole warps; the rest in the next round
             for (int i = lane; i < end; i += 32) {
-                const int2 pc = cell[base + i];
-                const float2 o0 = off0[base + i], o1 = off1[base + i];
+                const int64_t p = visit_at(perm, base + i);
+                const int2 pc = cell[p];
+                const float2 o0 = off0[p], o1 = off1[p];
                 if (!move_ok(pc.x, pc.y, o0.x, o1.x, o0.y, o1.y, n1, n2)) {
                     atomicOr(flag, 1);
                     continue;
                 }
-                const float qp = q[base + i];
-                deposit_alone<ORDER>(J1, J2, J3, n1, n2, pc, o0, o1, c1s * qp, c2s * qp, v3 ? c3s * qp * v3[base + i] : 0.f);
+                const float qp = q[p];
+                deposit_alone<ORDER>(J1, J2, J3, n1, n2, pc, o0, o1, c1s * qp, c2s * qp, v3 ? c3s * qp * v3[p] : 0.f);
             }
         }
         base += end;
@@ -433,37 +440,46 @@ __global__ void k_deposit3d(T* __restrict__ J1, T* __restrict__ J2, T* __restric
     }
 }
 
+__global__ void k_zero3(uint4* __restrict__ a, uint4* __restrict__ b, uint4* __restrict__ c, int64_t n) {
+    uint4* const p = blockIdx.y == 0 ? a : blockIdx.y == 1 ? b : c;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 template <int ORDER>
 static cudaError_t launch_runs(hyb_grid* g, float* J1, float* J2, float* J3, const int32_t* cell, const float* off_old,
-                               const float* off_new, const float* v3, const float* q, int64_t np, float c1, float c2, float c3) {
-    auto kern = k_deposit2d_runs<ORDER>;
+                               const float* off_new, const float* v3, const float* q, int64_t np, float c1, float c2, float c3, const Visit& visit) {
+    const auto kern = visit.perm ? k_deposit2d_runs<ORDER, true> : k_deposit2d_runs<ORDER, false>;
     // a contiguous range of particles per warp, four waves of resident blocks
     const int64_t warps = (int64_t)resident_grid((const void*)kern, 32 * kRunWarps, 0) * kRunWarps * 4;
     const int64_t per = std::max<int64_t>(32, ((np + warps - 1) / warps + 255) / 256 * 256);
     const unsigned blocks = (unsigned)((np + per * kRunWarps - 1) / (per * kRunWarps));
     kern<<<blocks, 32 * kRunWarps, 0, g->stream>>>(J1, J2, J3, g->d.n1, g->d.n2, reinterpret_cast<const int2*>(cell),
                                                    reinterpret_cast<const float2*>(off_old),
-                                                   reinterpret_cast<const float2*>(off_new), v3, q, np, per, c1, c2, c3, g->dflag);
+                                                   reinterpret_cast<const float2*>(off_new), v3, q, np, per, c1, c2, c3, g->dflag, visit);
     return cudaGetLastError();
 }
 
 template <typename T>
 hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* off_new, const T* v3, const T* q,
-                   int64_t np, int order) {
+                   int64_t np, int order, Visit visit) {
     const hyb_grid_desc& d = g->d;
-    const size_t bytes = (size_t)g->cells * sizeof(T);
-    for (int c = 0; c < 3; c++) HYB_CUDA_TRY(cudaMemsetAsync(g->J[c], 0, bytes, g->stream));
-    if (np == 0) return HYB_OK;
-    T* J1 = (T*)g->J[0]; T* J2 = (T*)g->J[1]; T* J3 = (T*)g->J[2];
     int dev_sms = 0;
     cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, g->device);
+    {   // one launch for the three arrays (16-byte aligned, a whole number of 16-byte words: n1 >= 8)
+        const int64_t n = g->cells * (int64_t)sizeof(T) / 16;
+        const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)dev_sms * 8);
+        k_zero3<<<dim3(blocks, 3), 256, 0, g->stream>>>((uint4*)g->J[0], (uint4*)g->J[1], (uint4*)g->J[2], n);
+        HYB_CUDA_TRY(cudaGetLastError());
+    }
+    if (np == 0) return HYB_OK;
+    T* J1 = (T*)g->J[0]; T* J2 = (T*)g->J[1]; T* J3 = (T*)g->J[2];
     if (d.dims == 2) {
         const T c1 = (T)(-1.0 / (d.dt * d.dx2)), c2 = (T)(-1.0 / (d.dt * d.dx1)), c3 = (T)(1.0 / (d.dx1 * d.dx2));
         // the run kernel reads a particle's pairs at once
         const bool pairs = ((((uintptr_t)cell | (uintptr_t)off_old | (uintptr_t)off_new) & 7) == 0);
         if constexpr (std::is_same<T, float>::value) {
             if (pairs) {
-#define HYB_DEPR(O) HYB_CUDA_TRY((launch_runs<O>(g, J1, J2, J3, cell, off_old, off_new, v3, q, np, c1, c2, c3)))
+#define HYB_DEPR(O) HYB_CUDA_TRY((launch_runs<O>(g, J1, J2, J3, cell, off_old, off_new, v3, q, np, c1, c2, c3, visit)))
                 if (order == 1) HYB_DEPR(1); else if (order == 2) HYB_DEPR(2); else HYB_DEPR(3);
 #undef HYB_DEPR
                 return HYB_OK;
@@ -473,7 +489,7 @@ hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* 
         int threads = kDepThreads;
         while (threads > 32 && np < (int64_t)threads * dev_sms) threads >>= 1;
         const unsigned blocks = (unsigned)std::min<int64_t>((np + threads - 1) / threads, (int64_t)dev_sms * 32);
-#define HYB_DEP2(O) k_deposit2d<T, O><<<blocks, threads, 0, g->stream>>>(J1, J2, J3, d.n1, d.n2, cell, off_old, off_new, v3, q, np, c1, c2, c3, g->dflag)
+#define HYB_DEP2(O) (visit.perm ? k_deposit2d<T, O, true> : k_deposit2d<T, O, false>)<<<blocks, threads, 0, g->stream>>>(J1, J2, J3, d.n1, d.n2, cell, off_old, off_new, v3, q, np, c1, c2, c3, g->dflag, visit)
         if (order == 1) HYB_DEP2(1); else if (order == 2) HYB_DEP2(2); else HYB_DEP2(3);
 #undef HYB_DEP2
     } else {
@@ -488,7 +504,7 @@ hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* 
     return HYB_OK;
 }
 
-template hyb_status deposit<float>(hyb_grid*, const int32_t*, const float*, const float*, const float*, const float*, int64_t, int);
-template hyb_status deposit<double>(hyb_grid*, const int32_t*, const double*, const double*, const double*, const double*, int64_t, int);
+template hyb_status deposit<float>(hyb_grid*, const int32_t*, const float*, const float*, const float*, const float*, int64_t, int, Visit);
+template hyb_status deposit<double>(hyb_grid*, const int32_t*, const double*, const double*, const double*, const double*, int64_t, int, Visit);
 
 }  // namespace hyb

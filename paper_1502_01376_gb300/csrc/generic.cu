@@ -538,7 +538,7 @@ template <> const ModeTables<double>& tables<double>(hyb_grid* g) { return g->td
 static bool amp_fused(const hyb_grid* g) { return g->d.precision == 32 && g->d.n1 == 1024 && g->path < 3 && g->d.dims != 20; }
 
 template <typename T>
-hyb_status generic_advance(hyb_grid* g, int nsteps) {
+hyb_status generic_advance(hyb_grid* g, int nsteps, bool have_spectra) {
     using C = cplx<T>;
     const ModeTables<T>& t = tables<T>(g);
     const int n1 = g->d.n1, nk = g->nk;
@@ -555,7 +555,7 @@ hyb_status generic_advance(hyb_grid* g, int nsteps) {
         if (g->ev_start) HYB_CUDA_TRY(cudaEventRecord(g->ev_start, g->stream));
         // k1-resident state: the spectra of E and B left by the previous step are this step's
         // input, so only j is transformed (the first step after hyb_set_resident imports E, B)
-        const int f0 = (g->resident && !g->res_stale) ? 6 : 0;
+        const int f0 = (g->resident && !g->res_stale) || (have_spectra && s == 0) ? 6 : 0;
         RowPtrs fin{};
         for (int c = f0; c < 9; c++) fin.p[c - f0] = src9[c];
         C* spec_in = spec + (int64_t)f0 * rows * nk;
@@ -673,8 +673,8 @@ template hyb_status generic_b_half<double>(hyb_grid*, void* const*);
 
 int generic_launches_per_step(const hyb_grid* g) { return (amp_fused(g) || g->d.dims == 20) ? 3 : 4; }
 
-template hyb_status generic_advance<float>(hyb_grid*, int);
-template hyb_status generic_advance<double>(hyb_grid*, int);
+template hyb_status generic_advance<float>(hyb_grid*, int, bool);
+template hyb_status generic_advance<double>(hyb_grid*, int, bool);
 template hyb_status generic_process_current<float>(hyb_grid*, bool, bool);
 template hyb_status generic_process_current<double>(hyb_grid*, bool, bool);
 

@@ -308,7 +308,9 @@ hyb_status cuda_fail(cudaError_t e, const char* what);
     } while (0)
 
 // three-pass path (generic.cu)
-template <typename T> hyb_status generic_advance(hyb_grid* g, int nsteps);
+// have_spectra: the spectra of the bound E, B are already in the scratch (generic_resident_import), so that only
+// j is transformed (first step)
+template <typename T> hyb_status generic_advance(hyb_grid* g, int nsteps, bool have_spectra = false);
 template <typename T> hyb_status generic_process_current(hyb_grid* g, bool corr, bool filt);
 // k1-resident state (three-pass path): import E, B into the spectra; B^n = B^{n-1/2} + Faraday/2
 // from the spectra into the real arrays Bh (the PIC step's gather)
@@ -347,10 +349,58 @@ void dftgemm_destroy(hyb_grid* g);
 hyb_status dftgemm_forward(hyb_grid* g, const float* const* fields, int nf, float2* spec);
 hyb_status dftgemm_inverse(hyb_grid* g, const float2* spec, int nf, float* const* fields);
 
+// An order in which the particle kernels visit the particles: the i-th is perm[i] when *jumps (counted on the
+// device, order.cu) exceeds limit, else i.  A default one visits them as stored.
+struct Visit {
+    const int* perm = nullptr;
+    const unsigned* jumps = nullptr;
+    unsigned limit = 0;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ const int* visit_perm(const Visit& v) { return v.perm && *v.jumps > v.limit ? v.perm : nullptr; }
+__device__ __forceinline__ int64_t visit_at(const int* perm, int64_t i) { return perm ? (int64_t)perm[i] : i; }
+#endif
+
+#ifdef __CUDACC__
+// periodic index: one add or subtract for the stencil's range (-n <= i < 2n), a modulo only
+// for grids narrower than the stencil
+__device__ __forceinline__ int pwrap(int i, int n) {
+    i = i < 0 ? i + n : i;
+    i = i >= n ? i - n : i;
+    if ((unsigned)i >= (unsigned)n) i = ((i % n) + n) % n;
+    return i;
+}
+
+// moves a particle to the cell that holds it (offsets in [-1, 2) on entry); the decision and the new
+// offset are taken in T, so that off ends in [0, 1)
+template <typename T>
+__device__ __forceinline__ bool renormalise(int& c, T& o, int n) {
+    if (!(o >= (T)-1 && o < (T)2)) return false;
+    if (o < (T)0) { o += (T)1; c -= 1; }
+    else if (o >= (T)1) { o -= (T)1; c += 1; }
+    if (o >= (T)1) { o = (T)0; c += 1; }          // o = -tiny rounded up to 1
+    c = pwrap(c, n);
+    return true;
+}
+#endif
+
+// cell order of scattered particles (order.cu): perm[0 .. np) lists the particles cell by cell
+struct Order {
+    int* perm = nullptr;          // [cap]
+    int* count = nullptr;         // [cells]: particles of a cell, then its next place in the list
+    unsigned* ctl = nullptr;      // jumps, cursor
+    int64_t cap = 0, cells = 0;
+    std::vector<void*> blocks;    // allocations, the current one last
+};
+void order_free(Order& o);
+// room for np particles of g (false: none, e.g. while a stream is captured; the particles are then visited as stored)
+bool order_reserve(Order& o, const hyb_grid* g, int64_t np);
+template <typename T> hyb_status order_particles(Order& o, hyb_grid* g, const int32_t* cell, const T* off, int64_t np, Visit* v);
+
 // deposit (deposit.cu)
 template <typename T>
 hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* off_new, const T* v3,
-                   const T* q, int64_t np, int order);
+                   const T* q, int64_t np, int order, Visit visit = Visit());
 
 // field gather and Boris push (push.cu)
 template <typename T>
@@ -358,7 +408,7 @@ hyb_status push(hyb_grid* g, int32_t* cell, T* off, T* u, const T* qm, T* off_ne
 // the same with the fields given explicitly (E[3], B[3] of the grid's shape and precision)
 template <typename T>
 hyb_status push_fields(hyb_grid* g, void* const E[3], void* const B[3], int32_t* cell, T* off, T* u, const T* qm,
-                       T* off_new, T* v3, int64_t np, int order);
+                       T* off_new, T* v3, int64_t np, int order, Visit visit = Visit());
 
 // diagnostics (diag.cu)
 template <typename T> hyb_status diag(hyb_grid* g, double out[9]);

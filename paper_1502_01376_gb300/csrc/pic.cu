@@ -6,9 +6,11 @@
 //
 // One step, with E = E^n, B = B^{n-1/2} bound to the grid and the particles at
 // x^n (cell, off) with u^{n-1/2}:
-//   1. B^{n+1/2} = B^{n-1/2} + Faraday(E^n): a copy of E and B is advanced one
-//      step by a second grid of the same description with zero current (its E
-//      is discarded); then B^n = (B^{n-1/2} + B^{n+1/2}) / 2 in that copy;
+//   1. B^n = (B^{n-1/2} + B^{n+1/2}) / 2, B^{n+1/2} = B^{n-1/2} + Faraday(E^n).  Three-pass
+//      grids (path 1) transform E and B, form B^{n-1/2} + Faraday(E^n)/2 mode by mode and transform
+//      it back; step 4 goes on from the same spectra (18 row transforms a step).  On the other paths a
+//      copy of E and B is advanced one step by a second grid of the same description with zero
+//      current (its E is discarded) and averaged with B;
 //   2. gather E^n, B^n and Boris push: u^{n+1/2}, x^{n+1} (hyb_push);
 //   3. deposit j^{n+1/2} from x^n -> x^{n+1} (hyb_deposit);
 //   4. the hybrid advance: E^{n+1}, B^{n+1/2} (hyb_advance);
@@ -16,15 +18,16 @@
 // With k1-resident fields (hyb_set_resident) step 1 needs no second grid: B^n =
 // B^{n-1/2} + Faraday(E^n)/2 is formed mode by mode from the resident spectra and
 // transformed back into scratch arrays, and step 4 transforms only j forward, so a
-// step takes 12 row transforms (3 for B^n, 3 for j, 6 for E, B) instead of two
-// full advances (30) and the copies of E and B.
+// step takes 12 row transforms (3 for B^n, 3 for j, 6 for E, B).
+// Scattered particles (2D) are visited cell by cell in steps 2 and 3 (order.cu).
 #include "hyb_internal.cuh"
 
 struct hyb_pic {
     hyb_grid* g = nullptr;        // the caller's grid (borrowed)
     hyb_grid* shadow = nullptr;   // the same description, bound to the scratch copy and zero current
-    void* scratch = nullptr;      // E'[3], B'[3], J'[3] = 0
+    void* scratch = nullptr;      // with a shadow grid E'[3], B'[3], J'[3] = 0; else B'[3]
     size_t field_bytes = 0;
+    hyb::Order order;             // cell order of scattered particles
     // one step captured as a CUDA graph, replayed for the later steps of a call (and of later calls
     // with the same arguments): its own stream, fork/join events, and the arguments it was taken with
     cudaStream_t cs = nullptr;
@@ -57,15 +60,20 @@ template <typename T>
 static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm, const T* q, T* off_new, T* v3,
                            int64_t np, int order) {
     hyb_grid* g = p->g;
-    if (g->resident) {
+    Visit visit;
+    if (order_reserve(p->order, g, np)) {
+        hyb_status st = order_particles<T>(p->order, g, cell, off, np, &visit);
+        if (st != HYB_OK) return st;
+    }
+    if (g->resident || !p->shadow) {
         void* Bh[3];
-        for (int c = 0; c < 3; c++) Bh[c] = (char*)p->scratch + (size_t)(3 + c) * p->field_bytes;
+        for (int c = 0; c < 3; c++) Bh[c] = (char*)p->scratch + (size_t)((p->shadow ? 3 : 0) + c) * p->field_bytes;
         hyb_status st = HYB_OK;
-        if (g->res_stale) st = generic_resident_import<T>(g);                  // E^n, B^{n-1/2} spectra
+        if (!g->resident || g->res_stale) st = generic_resident_import<T>(g);  // E^n, B^{n-1/2} spectra
         if (st == HYB_OK) st = generic_b_half<T>(g, Bh);                        // B^n
-        if (st == HYB_OK) st = push_fields<T>(g, g->E, Bh, cell, off, u, qm, off_new, v3, np, order);
-        if (st == HYB_OK) st = hyb_deposit(g, cell, off, off_new, v3, q, np, order);
-        if (st == HYB_OK) st = hyb_advance(g, 1);                               // j forward only
+        if (st == HYB_OK) st = push_fields<T>(g, g->E, Bh, cell, off, u, qm, off_new, v3, np, order, visit);
+        if (st == HYB_OK) st = deposit<T>(g, cell, off, off_new, v3, q, np, order, visit);
+        if (st == HYB_OK) st = g->resident ? hyb_advance(g, 1) : generic_advance<T>(g, 1, true);   // j forward only
         if (st != HYB_OK) return st;
         if (np > 0)
             HYB_CUDA_TRY(cudaMemcpyAsync(off, off_new, sizeof(T) * (size_t)np * g->d.dims, cudaMemcpyDeviceToDevice, g->stream));
@@ -91,9 +99,9 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
                                                         (const T*)g->B[1], (const T*)g->B[2], g->cells);
         HYB_CUDA_TRY(cudaGetLastError());
     }
-    st = push_fields<T>(g, g->E, Bs, cell, off, u, qm, off_new, v3, np, order);   // u^{n+1/2}, x^{n+1}
+    st = push_fields<T>(g, g->E, Bs, cell, off, u, qm, off_new, v3, np, order, visit);   // u^{n+1/2}, x^{n+1}
     if (st != HYB_OK) return st;
-    st = hyb_deposit(g, cell, off, off_new, v3, q, np, order);  // j^{n+1/2}
+    st = deposit<T>(g, cell, off, off_new, v3, q, np, order, visit);  // j^{n+1/2}
     if (st != HYB_OK) return st;
     st = hyb_advance(g, 1);                                      // E^{n+1}, B^{n+1/2}
     if (st != HYB_OK) return st;
@@ -116,8 +124,13 @@ hyb_status hyb_pic_create(hyb_grid* g, hyb_pic** out) {
     hyb_pic* p = new hyb_pic();
     p->g = g;
     p->field_bytes = (size_t)g->cells * (g->d.precision == 32 ? 4 : 8);
-    cudaError_t e = cudaMalloc(&p->scratch, 9 * p->field_bytes);
+    const bool shadow = g->path != 1;                            // the three-pass path forms B^n from its own spectra
+    cudaError_t e = cudaMalloc(&p->scratch, (shadow ? 9 : 3) * p->field_bytes);
     if (e != cudaSuccess) { p->scratch = nullptr; hyb_pic_destroy(p); return cuda_fail(e, "cudaMalloc(pic scratch)"); }
+    if (!shadow) {
+        *out = p;
+        return HYB_OK;
+    }
     e = cudaMemset((char*)p->scratch + 6 * p->field_bytes, 0, 3 * p->field_bytes);
     if (e != cudaSuccess) { hyb_pic_destroy(p); return cuda_fail(e, "cudaMemset(pic scratch)"); }
     hyb_grid_desc d = g->d;
@@ -227,6 +240,7 @@ hyb_status hyb_pic_destroy(hyb_pic* p) {
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
     if (p->ev_join) cudaEventDestroy(p->ev_join);
     if (p->cs) cudaStreamDestroy(p->cs);
+    order_free(p->order);
     if (p->scratch) cudaFree(p->scratch);
     delete p;
     return HYB_OK;

@@ -49,27 +49,6 @@ __device__ __forceinline__ int pweights(T p, T (&w)[L + 1]) {
 __device__ __forceinline__ float prsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double prsqrt(double x) { return 1.0 / sqrt(x); }
 
-// periodic index: one add or subtract for the stencil's range (-n <= i < 2n), a modulo only
-// for grids narrower than the stencil
-__device__ __forceinline__ int pwrap(int i, int n) {
-    i = i < 0 ? i + n : i;
-    i = i >= n ? i - n : i;
-    if ((unsigned)i >= (unsigned)n) i = ((i % n) + n) % n;
-    return i;
-}
-
-// moves a particle to the cell that holds it (offsets in [-1, 2) on entry); the decision and the new
-// offset are taken in T, so that off ends in [0, 1)
-template <typename T>
-__device__ __forceinline__ bool renormalise(int& c, T& o, int n) {
-    if (!(o >= (T)-1 && o < (T)2)) return false;
-    if (o < (T)0) { o += (T)1; c -= 1; }
-    else if (o >= (T)1) { o -= (T)1; c += 1; }
-    if (o >= (T)1) { o = (T)0; c += 1; }          // o = -tiny rounded up to 1
-    c = pwrap(c, n);
-    return true;
-}
-
 template <typename T>
 __device__ __forceinline__ void boris(T (&u)[3], const T (&E)[3], const T (&B)[3], T h) {
     T um[3], t[3], up[3], s[3];
@@ -102,11 +81,11 @@ struct PushFields { const void* E[3]; const void* B[3]; };
 constexpr int kPushThreads = 256;
 constexpr int kReach = 2;
 
-template <typename T, int L>
+template <typename T, int L, bool VISIT>
 __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1, int n2, int32_t* __restrict__ cell,
                                                           T* __restrict__ off, T* __restrict__ u, const T* __restrict__ qm,
                                                           T* __restrict__ off_new, T* __restrict__ v3, int64_t np, T hdt,
-                                                          T s1, T s2, int* __restrict__ flag) {
+                                                          T s1, T s2, int* __restrict__ flag, Visit visit) {
     constexpr int kTile = sizeof(T) == 4 ? 1024 : 512;        // points per component in the shared tile
     __shared__ T tile[6][kTile];
     __shared__ int red[kPushThreads / 32][4];
@@ -114,23 +93,36 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
                        (const T*)F.B[0], (const T*)F.B[1], (const T*)F.B[2]};
     using V2 = cplx<T>;                      // a particle's two offsets, one 8- or 16-byte access
     const int64_t stride = (int64_t)gridDim.x * kPushThreads;
+    const int* const perm = VISIT ? visit_perm(visit) : nullptr;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the next particle's cell and offsets are loaded while this one is gathered and pushed
     int2 ncc = make_int2(0, 0);
     V2 noo;
     noo.x = noo.y = (T)0;
+    int64_t np_at = 0;
     {
-        const int64_t p = blockIdx.x * (int64_t)kPushThreads + threadIdx.x;
-        if (p < np) { ncc = reinterpret_cast<const int2*>(cell)[p]; noo = reinterpret_cast<const V2*>(off)[p]; }
+        const int64_t i = blockIdx.x * (int64_t)kPushThreads + threadIdx.x;
+        if (i < np) {
+            np_at = visit_at(perm, i);
+            ncc = reinterpret_cast<const int2*>(cell)[np_at];
+            noo = reinterpret_cast<const V2*>(off)[np_at];
+        }
     }
     for (int64_t base = blockIdx.x * (int64_t)kPushThreads; base < np; base += stride) {
-        const int64_t p = base + threadIdx.x;
-        const bool live = p < np;
+        const int64_t p = np_at;
+        const bool live = base + threadIdx.x < np;
         const int2 cc = ncc;
         const V2 oo = noo;
-        if (p + stride < np) {
-            ncc = reinterpret_cast<const int2*>(cell)[p + stride];
-            noo = reinterpret_cast<const V2*>(off)[p + stride];
+        if (base + threadIdx.x + stride < np) {
+            np_at = visit_at(perm, base + threadIdx.x + stride);
+            ncc = reinterpret_cast<const int2*>(cell)[np_at];
+            noo = reinterpret_cast<const V2*>(off)[np_at];
+        }
+        // asked for before the tile is staged, used after it
+        T uu[3] = {(T)0, (T)0, (T)0}, qmp = (T)0;
+        if (live) {
+            uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2];
+            qmp = qm[p];
         }
         int cx = cc.x, cy = cc.y;
         T ox = oo.x, oy = oo.y;
@@ -165,7 +157,6 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
         }
         __syncthreads();
         if (ok) {
-            T uu[3] = {u[3 * p], u[3 * p + 1], u[3 * p + 2]};
             // weights for the integer (0) and half (1) positions along each axis
             T wx[2][L + 1], wy[2][L + 1];
             const int ix0 = pweights<L>(ox, wx[0]), ix1 = pweights<L>(ox - (T)0.5, wx[1]);
@@ -211,7 +202,7 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
                 }
             }
             const T Ev[3] = {e1, e2, e3}, Bv[3] = {b1, b2, b3};
-            boris(uu, Ev, Bv, hdt * qm[p]);
+            boris(uu, Ev, Bv, hdt * qmp);
             const T gi = prsqrt((T)1 + uu[0] * uu[0] + uu[1] * uu[1] + uu[2] * uu[2]);
             reinterpret_cast<int2*>(cell)[p] = make_int2(cx, cy);
             V2 on;
@@ -297,7 +288,7 @@ __global__ void __launch_bounds__(256) k_push3d(PushFields F, int n1, int n2, in
 
 template <typename T>
 hyb_status push_fields(hyb_grid* g, void* const E[3], void* const B[3], int32_t* cell, T* off, T* u, const T* qm,
-                       T* off_new, T* v3, int64_t np, int order) {
+                       T* off_new, T* v3, int64_t np, int order, Visit visit) {
     const hyb_grid_desc& d = g->d;
     if (np == 0) return HYB_OK;
     PushFields F;
@@ -310,7 +301,7 @@ hyb_status push_fields(hyb_grid* g, void* const E[3], void* const B[3], int32_t*
     const T hdt = (T)(0.5 * d.dt);
     const T s1 = (T)(d.dt / d.dx1), s2 = (T)(d.dt / d.dx2), s3 = (T)(d.dt / d.dx3);
     if (d.dims == 2) {
-#define HYB_PUSH2(O) k_push2d<T, O><<<blocks, threads, 0, g->stream>>>(F, d.n1, d.n2, cell, off, u, qm, off_new, v3, np, hdt, s1, s2, g->dflag)
+#define HYB_PUSH2(O) (visit.perm ? k_push2d<T, O, true> : k_push2d<T, O, false>)<<<blocks, threads, 0, g->stream>>>(F, d.n1, d.n2, cell, off, u, qm, off_new, v3, np, hdt, s1, s2, g->dflag, visit)
         if (order == 1) HYB_PUSH2(1); else if (order == 2) HYB_PUSH2(2); else HYB_PUSH2(3);
 #undef HYB_PUSH2
     } else {
@@ -330,8 +321,8 @@ hyb_status push(hyb_grid* g, int32_t* cell, T* off, T* u, const T* qm, T* off_ne
 template hyb_status push<float>(hyb_grid*, int32_t*, float*, float*, const float*, float*, float*, int64_t, int);
 template hyb_status push<double>(hyb_grid*, int32_t*, double*, double*, const double*, double*, double*, int64_t, int);
 template hyb_status push_fields<float>(hyb_grid*, void* const*, void* const*, int32_t*, float*, float*, const float*,
-                                       float*, float*, int64_t, int);
+                                       float*, float*, int64_t, int, Visit);
 template hyb_status push_fields<double>(hyb_grid*, void* const*, void* const*, int32_t*, double*, double*,
-                                        const double*, double*, double*, int64_t, int);
+                                        const double*, double*, double*, int64_t, int, Visit);
 
 }  // namespace hyb
