@@ -66,7 +66,7 @@ struct hyb_mlp {
     float* loss = nullptr;                // device scalar
     int* err = nullptr;                   // device flag: bit 1 = a bounded wait in a GEMM gave up
     // networks wider than kNarrow (k_mlp_chain): BF16 weights in the order the kernel's shared memory
-    // holds them, every layer's input and dH feature-major, tanh of the hidden layers
+    // holds them; every layer's input (actT) and dH (dhT) in the order of k_dw_tiles, tanh of the hidden layers (pre)
     bool chain = false;
     __nv_bfloat16* wk = nullptr;          // [fin/8][rows][8] per layer (rows: outputs, padded)
     __nv_bfloat16* wkt = nullptr;         // [fout/8][rows][8] of the transposed weights (rows: inputs, padded)
@@ -173,9 +173,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 // tcgen05.ld into the epilogue.  Waits are bounded: on time-out bit 1 of *err is set and the
 // CTA skips the rest, drains and frees its TMEM.
 template <int EP, typename TA, typename TB>
-__device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, int K, int kmax, const TA* __restrict__ a, int64_t sam,
-                                          int64_t sak, const TB* __restrict__ b, int64_t sbk, int64_t sbn, const Epi& ep, int kchunk,
-                                          int* err) {
+__global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, const TA* __restrict__ a, int64_t sam, int64_t sak,
+                                                const TB* __restrict__ b, int64_t sbk, int64_t sbn, Epi ep, int kchunk, int* err) {
     __shared__ __align__(128) unsigned char sbuf[8 * LBO_A + 8 * LBO_B];
     __shared__ uint64_t bar;
     __shared__ uint32_t s_taddr;
@@ -196,8 +195,8 @@ __device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, 
     __syncthreads();
     tm_fence_after();
     const uint32_t tbase = s_taddr;
-    const int m0 = by * TM, n0 = bx * TN;
-    const int kb = bz * kchunk, ke = min(K, kb + kchunk);
+    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
     uint32_t ph = 0;
     bool pend = false, abort = false, any = false;
     for (int k0 = kb; k0 < ke && !abort; k0 += TKC) {
@@ -241,7 +240,7 @@ __device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, 
             const int c0 = n0 + 16 * u;
             if (EP == EP_PART) {
                 if (live && c0 < N) {
-                    float* p = ep.c + (int64_t)bz * M * N + (int64_t)row * N + c0;
+                    float* p = ep.c + (int64_t)blockIdx.z * M * N + (int64_t)row * N + c0;
                     if ((N & 3) == 0 && c0 + 16 <= N) {
 #pragma unroll
                         for (int j = 0; j < 4; j++)
@@ -289,8 +288,8 @@ __device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, 
                     if (lane == 0) { s_red[warp][0] = l; s_red[warp][1] = sd; }
                     __syncthreads();
                     if (tid == 0) {
-                        ep.loss_part[by] = (s_red[0][0] + s_red[1][0]) + (s_red[2][0] + s_red[3][0]);
-                        ep.db_part[by] = (s_red[0][1] + s_red[1][1]) + (s_red[2][1] + s_red[3][1]);
+                        ep.loss_part[blockIdx.y] = (s_red[0][0] + s_red[1][0]) + (s_red[2][0] + s_red[3][0]);
+                        ep.db_part[blockIdx.y] = (s_red[0][1] + s_red[1][1]) + (s_red[2][1] + s_red[3][1]);
                     }
                 }
             } else {   // EP_DX
@@ -332,7 +331,7 @@ __device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, 
         if (EP == EP_DX) {
             __syncthreads();
             if (tid < TN && n0 + tid < ep.n)
-                ep.db_part[(int64_t)by * ep.n + n0 + tid] = (s_red[0][tid] + s_red[1][tid]) + (s_red[2][tid] + s_red[3][tid]);
+                ep.db_part[(int64_t)blockIdx.y * ep.n + n0 + tid] = (s_red[0][tid] + s_red[1][tid]) + (s_red[2][tid] + s_red[3][tid]);
         }
     }
     if (tid == 0 && pend) mbar_drain(mb, ph);
@@ -340,32 +339,6 @@ __device__ __forceinline__ void gemm_tile(int bx, int by, int bz, int M, int N, 
     __syncthreads();
     tm_fence_after();
     if (warp == 0) tm_dealloc(tbase, TN);
-}
-
-template <int EP, typename TA, typename TB>
-__global__ void __launch_bounds__(GT) k_gemm_tc(int M, int N, int K, int kmax, const TA* __restrict__ a, int64_t sam, int64_t sak,
-                                                const TB* __restrict__ b, int64_t sbk, int64_t sbn, Epi ep, int kchunk, int* err) {
-    gemm_tile<EP, TA, TB>(blockIdx.x, blockIdx.y, blockIdx.z, M, N, K, kmax, a, sam, sak, b, sbk, sbn, ep, kchunk, err);
-}
-
-// The weight-gradient parts of every layer in one launch: blocks first[l] .. first[l + 1] - 1 are layer l's
-// tiles (column tile fastest, then row tile, then part of K).
-struct DwTab {
-    int L;
-    int first[kMaxLayers + 1];
-    int M[kMaxLayers], N[kMaxLayers], kchunk[kMaxLayers];
-    const __nv_bfloat16* a[kMaxLayers];               // dH, feature-major
-    const __nv_bfloat16* b[kMaxLayers];               // the layer's input, feature-major
-    float* c[kMaxLayers];
-};
-__global__ void __launch_bounds__(GT) k_dw_all(__grid_constant__ const DwTab t, int K, int kmax, int64_t ld, int* err) {
-    int l = 0;
-    while (l + 1 < t.L && (int)blockIdx.x >= t.first[l + 1]) l++;
-    const int r = blockIdx.x - t.first[l], nx = (t.N[l] + TN - 1) / TN, ny = (t.M[l] + TM - 1) / TM;
-    Epi ep;
-    ep.c = t.c[l];
-    gemm_tile<EP_PART>(r % nx, (r / nx) % ny, r / (nx * ny), t.M[l], t.N[l], K, kmax, t.a[l], ld, (int64_t)1, t.b[l], (int64_t)1, ld, ep,
-                       t.kchunk[l], err);
 }
 
 // K is rounded up to 16 (the MMA depth); entries with k >= K read as zero.
@@ -397,7 +370,6 @@ __host__ __device__ __forceinline__ int64_t chain_at(int row, int k, int rows) {
 // a bias gradient, the loss parts); with update != 0 also the Adam step on every parameter and
 // the BF16 copies of the updated weights (zero-padded, both layouts; the padding was written by
 // refresh()).  Without it the sums go to g (the gradients of hyb_mlp_gradients).
-template <bool CHAIN>
 __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                             const float* __restrict__ ws, const float* __restrict__ loss_part, float* __restrict__ loss,
                             int64_t n, int update, float lr, float b1, float b2, float eps, float c1, float c2, LayerTab tab,
@@ -405,7 +377,7 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i == 0) {
         float s = 0.f;
-        for (int y = 0; y < tab.nrb; y++) s += CHAIN ? loss_part[2 * y] + (2 * y + 1 < tab.nrc ? loss_part[2 * y + 1] : 0.f) : loss_part[y];
+        for (int y = 0; y < tab.nrb; y++) s += loss_part[y];
         *loss = s;
     }
     if (i >= n) return;
@@ -416,23 +388,10 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
     float gi = 0.f;
     if (loc < nw) {
         const float* p = ws + tab.ws_w[l] + loc;
-        int z = 0;
-        for (; z + 8 <= tab.split[l]; z += 8) {           // eight loads in flight, added in order
-            float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) v[e] = p[(z + e) * nw];
-#pragma unroll
-            for (int e = 0; e < 8; e++) gi += v[e];
-        }
-        for (; z < tab.split[l]; z++) gi += p[z * nw];
+        for (int z = 0; z < tab.split[l]; z++) gi += p[z * nw];
     } else {
         const float* p = ws + tab.ws_b[l] + (loc - nw);
-        const int64_t fo = tab.fo[l];
-        if (CHAIN) {
-            for (int y = 0; y < tab.nrb; y++) gi += p[2 * y * fo] + (2 * y + 1 < tab.nrc ? p[(2 * y + 1) * fo] : 0.f);
-        } else {
-            for (int y = 0; y < tab.nrb; y++) gi += p[(int64_t)y * fo];
-        }
+        for (int y = 0; y < tab.nrb; y++) gi += p[(int64_t)y * tab.fo[l]];
     }
     if (!update) {
         g[i] = gi;
@@ -447,13 +406,8 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
     if (loc < nw) {
         const int r = (int)(loc / tab.fi[l]), c = (int)(loc % tab.fi[l]);
         const __nv_bfloat16 q = __float2bfloat16(wi);
-        if (CHAIN) {
-            wb[tab.wk_off[l] + chain_at(r, c, tab.rows[l])] = q;
-            if (l > 0 && l + 1 < tab.L) wt[tab.wk_off[l] + chain_at(c, r, tab.rows[l])] = q;
-        } else {
-            wb[tab.wb_off[l] + (int64_t)r * tab.fip[l] + c] = q;
-            wt[tab.wb_off[l] + (int64_t)c * tab.fop[l] + r] = q;
-        }
+        wb[tab.wb_off[l] + (int64_t)r * tab.fip[l] + c] = q;
+        wt[tab.wb_off[l] + (int64_t)c * tab.fop[l] + r] = q;
     }
 }
 
@@ -463,12 +417,12 @@ __global__ void k_grad_adam(float* __restrict__ w, float* __restrict__ g, float*
 // products are taken transposed, D^T[features][rows] = W X^T: A is the weight matrix (128-row tiles, K-major, in
 // shared memory as it lies in global memory: one bulk copy per layer, which runs while the previous
 // layer's epilogue does), B the tile of activations [64 rows][K].  A TMEM lane is then a feature and
-// its columns the rows of the batch: bias, tanh and tanh' are lane-local, the feature-major copies that
-// the weight gradients read are contiguous per thread, and the epilogue writes the next product's B operand
-// straight into shared memory.  The output layer's product is taken the other way round (a lane per row:
+// its columns the rows of the batch: bias, tanh and tanh' are lane-local, the copies that the weight gradients
+// read are written in their operands' order, a warp's 512 bytes at a time, and the epilogue writes the
+// next product's B operand straight into shared memory.  The output layer's product is taken the other way round (a lane per row:
 // loss and dH of a row), and its dX, one product per element, needs no MMA.  Bound by the epilogues (16384
 // values per layer and tile, an accurate tanhf each): 16 warps, and 64 rows so that a batch of 8192 is 128 CTAs.
-// 8192 x (6 -> 256 x 4 -> 1): a step took 262 us with a launch per product.
+// 8192 x (6 -> 256 x 4 -> 1): a step took 262 us with a launch per product, 80 us now (40 chain, 16 dW, 13 Adam).
 // Sums and roundings are those of the launch-per-product form (same products in the same K order, the same
 // trees of partial sums), so both give the same gradients.
 struct ChainArgs {
@@ -480,9 +434,10 @@ struct ChainArgs {
     const __nv_bfloat16* wk[kMaxLayers];
     const __nv_bfloat16* wkt[kMaxLayers];
     const float* bias[kMaxLayers];
-    __nv_bfloat16* actT;                               // [L][256][cap]: the layers' inputs
-    __nv_bfloat16* dhT;                                // [L][256][cap]
-    float* th;                                         // [depth][256][cap]: tanh of the hidden layers
+    __nv_bfloat16* act;                                // per layer 256 cap values: its input as [cap/8][rows][8] (rows:
+                                                       // pad16(n_in), then those of a weight tile)
+    __nv_bfloat16* dh;                                 // per layer its dH the same way (16 rows for the output layer)
+    float* th;                                         // tanh of the hidden layers, per layer [cap/4][rows][4]
     float* db_part[kMaxLayers];                        // [64-row blocks][fo]
     float* loss_part;                                  // [64-row blocks]
     float invB;
@@ -558,7 +513,7 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
         const int64_t b = b0 + n;
         const uint32_t v = (b < g.B && k < g.n_in) ? bf16_bits(__ldg(g.x + b * g.n_in + k)) : 0u;
         asm volatile("st.shared.u16 [%0], %1;" :: "r"(sX + (uint32_t)((k >> 3) * LBO_X + n * 16 + (k & 7) * 2)), "h"((unsigned short)v) : "memory");
-        if (train && k < g.n_in) reinterpret_cast<unsigned short*>(g.actT)[(int64_t)k * g.cap + b] = (unsigned short)v;
+        if (train) reinterpret_cast<unsigned short*>(g.act)[chain_at(k, (int)b, K0)] = (unsigned short)v;
     }
     fence_proxy_async_smem();
     __syncthreads();
@@ -596,10 +551,10 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
             for (int n = 0; n < 32; n++)
                 asm volatile("st.shared.u16 [%0], %1;" :: "r"(at + 16 * n), "h"((unsigned short)(q[n >> 1] >> (16 * (n & 1)))) : "memory");
         }
-        if (copy && live) {
-            uint4* c = reinterpret_cast<uint4*>(copy + (int64_t)f * g.cap + b0 + 32 * ch);
+        if (copy && mine) {
 #pragma unroll
-            for (int e = 0; e < 4; e++) c[e] = make_uint4(q[4 * e], q[4 * e + 1], q[4 * e + 2], q[4 * e + 3]);
+            for (int e = 0; e < 4; e++)
+                *reinterpret_cast<uint4*>(copy + ((b0 / 8 + 4 * ch + e) * rows + f) * 8) = make_uint4(q[4 * e], q[4 * e + 1], q[4 * e + 2], q[4 * e + 3]);
         }
     };
     bool stop = false;
@@ -624,11 +579,11 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
 #pragma unroll
             for (int n = 0; n < 16; n++) q[n] = bf16_bits(t[2 * n]) | (bf16_bits(t[2 * n + 1]) << 16);
             if (train && live) {
-                float4* o = reinterpret_cast<float4*>(g.th + ((int64_t)l * 256 + f) * g.cap + b0 + 32 * ch);
+                float4* o = reinterpret_cast<float4*>(g.th + (int64_t)l * 256 * g.cap) + (b0 / 4 + 8 * ch) * rows + f;
 #pragma unroll
-                for (int e = 0; e < 8; e++) o[e] = make_float4(t[4 * e], t[4 * e + 1], t[4 * e + 2], t[4 * e + 3]);
+                for (int e = 0; e < 8; e++) o[e * rows] = make_float4(t[4 * e], t[4 * e + 1], t[4 * e + 2], t[4 * e + 3]);
             }
-            put(q, true, train ? g.actT + (int64_t)(l + 1) * 256 * g.cap : nullptr);
+            put(q, true, train ? g.act + (int64_t)(l + 1) * 256 * g.cap : nullptr);
         }
         tm_fence_before();
         fence_proxy_async_smem();
@@ -658,7 +613,7 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
                 const float dd = in ? y - g.tgt[b] : 0.f;
                 const float d = 2.f * dd * g.invB;
                 const __nv_bfloat16 db = __float2bfloat16(d);
-                g.dhT[(int64_t)depth * 256 * g.cap + b] = db;
+                g.dh[(int64_t)depth * 256 * g.cap + chain_at(0, (int)b, 16)] = db;
                 s_d[32 * warp + lane] = __bfloat162float(db);
                 const float ls = warp_sum(dd * dd * g.invB), sd = warp_sum(d);
                 if (lane == 0) { s_red[0][warp] = ls; s_red[1][warp] = sd; }
@@ -678,10 +633,10 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
     for (int l = depth - 1; train && l >= 0 && !stop; l--) {
         float th[32];
         if (live) {
-            const float4* o = reinterpret_cast<const float4*>(g.th + ((int64_t)l * 256 + f) * g.cap + b0 + 32 * ch);
+            const float4* o = reinterpret_cast<const float4*>(g.th + (int64_t)l * 256 * g.cap) + (b0 / 4 + 8 * ch) * rows + f;
 #pragma unroll
             for (int e = 0; e < 8; e++) {
-                const float4 v = o[e];
+                const float4 v = o[e * rows];
                 th[4 * e] = v.x; th[4 * e + 1] = v.y; th[4 * e + 2] = v.z; th[4 * e + 3] = v.w;
             }
         } else {
@@ -714,7 +669,7 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
         for (int n = 0; n < 32; n++) t[n] = live ? t[n] * (1.f - th[n] * th[n]) : 0.f;
 #pragma unroll
         for (int n = 0; n < 16; n++) q[n] = bf16_bits(t[2 * n]) | (bf16_bits(t[2 * n + 1]) << 16);
-        put(q, l > 0, g.dhT + (int64_t)l * 256 * g.cap);
+        put(q, l > 0, g.dh + (int64_t)l * 256 * g.cap);
         s_red[ch][f] = tree_sum(t);
         tm_fence_before();
         fence_proxy_async_smem();
@@ -730,6 +685,208 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
     __syncthreads();
     tm_fence_after();
     if (warp == 0) tm_dealloc(tbase, 256);
+}
+
+// ------------------------------------------------------------------ the weight gradients after the chain
+// dW parts of every layer in one launch: dW[fo][fi] = dH^T X, K = batch, split as in the launch-per-product form (the
+// same parts, the same bits).  A CTA takes one part of one 128-row tile: both operands lie in global memory in
+// the order of the tensor core's K-major layout (k_mlp_chain wrote them so), so a chunk of 64 rows of the batch is one bulk
+// copy for X and one per K group for the tile's rows of dH; two chunks in flight.  The parts are written
+// [part][column][row], a warp's rows contiguous.  The six launches this replaces loaded their operands through
+// registers, 32 columns a CTA: 33 us for 8192 x (6 -> 256 x 4 -> 1), 15.5 us now.
+constexpr int DT = 256, DK = 64;                       // threads; rows of the batch per chunk
+struct DwTab {
+    int L;
+    int first[kMaxLayers + 1];                         // first block of a layer
+    int M[kMaxLayers], N[kMaxLayers];                  // dW's rows (outputs) and columns (inputs)
+    int ra[kMaxLayers], rb[kMaxLayers];                // rows of the stored dH and X
+    int kchunk[kMaxLayers];
+    const __nv_bfloat16* a[kMaxLayers];
+    const __nv_bfloat16* b[kMaxLayers];
+    float* c[kMaxLayers];
+};
+constexpr int kDwA = 128 * DK * 2, kDwB = 256 * DK * 2, kDwSmem = 2 * (kDwA + kDwB);
+__global__ void __launch_bounds__(DT, 2) k_dw_tiles(const __grid_constant__ DwTab t, int K, int* err) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ uint64_t bars[3];                       // two chunks, the products
+    __shared__ uint32_t s_taddr;
+    __shared__ int s_abort;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int l = 0;
+    while (l + 1 < t.L && (int)blockIdx.x >= t.first[l + 1]) l++;
+    const int M = t.M[l], N = t.N[l], Np = (N + 15) & ~15, ny = (M + 127) / 128;
+    const int r = blockIdx.x - t.first[l], m0 = (r % ny) * 128, z = r / ny;
+    const int kb = z * t.kchunk[l], ke = min(K, kb + t.kchunk[l]), nc = kb < ke ? (ke - kb + DK - 1) / DK : 0;
+    const int ra = t.ra[l], rb = t.rb[l], ma = min(128, ra - m0);       // rows of dH loaded per K group
+    if (warp == 0) {
+        tm_alloc(smem_addr(&s_taddr), 256);
+        tm_relinquish();
+    }
+    if (tid == 0) {
+        for (int i = 0; i < 3; i++) mbar_init(smem_addr(&bars[i]), 1);
+        mbar_fence_init();
+        s_abort = 0;
+    }
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    const uint32_t tbase = s_taddr, mb = smem_addr(&bars[2]);
+    if (tid == 0 && nc > 0) {
+        auto load = [&](int c) {
+            const int s = c & 1, k0 = kb + c * DK, g8 = (min(ke, k0 + DK) - k0) / 8;
+            const uint32_t sa = smem_addr(smem) + s * (kDwA + kDwB), sb = sa + kDwA, bar = smem_addr(&bars[s]);
+            mbar_expect_tx(bar, (uint32_t)g8 * (uint32_t)(ma + rb) * 16u);
+            for (int g = 0; g < g8; g++)
+                bulk_load(sa + g * ma * 16, t.a[l] + ((int64_t)(k0 / 8 + g) * ra + m0) * 8, (uint32_t)ma * 16u, bar);
+            bulk_load(sb, t.b[l] + (int64_t)(k0 / 8) * rb * 8, (uint32_t)g8 * (uint32_t)rb * 16u, bar);
+        };
+        int loaded = 0, done = 0;
+        uint32_t mph = 0;
+        for (; loaded < min(2, nc); loaded++) load(loaded);
+        for (int c = 0; c < nc && !s_abort; c++) {
+            const int s = c & 1, k0 = kb + c * DK, ks_n = (min(ke, k0 + DK) - k0) / 16;
+            mbar_wait(smem_addr(&bars[s]), (c >> 1) & 1, err, &s_abort);
+            if (s_abort) break;
+            done = c + 1;
+            tm_fence_after();
+            const uint32_t sa = smem_addr(smem) + s * (kDwA + kDwB), sb = sa + kDwA;
+            for (int ks = 0; ks < ks_n; ks++)
+                mma_bf16(tbase, smem_desc(sa + 2 * ks * ma * 16, ma * 16, 128), smem_desc(sb + 2 * ks * rb * 16, rb * 16, 128), idesc_bf16(Np),
+                         (c > 0 || ks > 0) ? 1u : 0u);
+            mma_commit(mb);
+            if (loaded < nc) {                           // the chunk's buffers are free once its products are done
+                mbar_wait(mb, mph, err, &s_abort);
+                if (s_abort) { mbar_drain(mb, mph); break; }
+                mph ^= 1;
+                load(loaded++);
+            } else {
+                mbar_wait(mb, mph, err, &s_abort);
+                if (s_abort) { mbar_drain(mb, mph); break; }
+                mph ^= 1;
+            }
+        }
+        for (int c = done; c < loaded; c++) mbar_drain(smem_addr(&bars[c & 1]), (c >> 1) & 1);     // after a give-up
+    }
+    __syncthreads();
+    if (!s_abort) {
+        tm_fence_after();
+        const int row = m0 + 32 * (warp & 3) + lane;
+        float* const P = t.c[l] + (int64_t)z * M * N;
+        for (int c0 = 16 * (warp >> 2); c0 < N; c0 += 32) {
+            float v[16];
+            if (nc > 0) {
+                tm_ld16(tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, v);
+                tm_wait_ld();
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; j++) v[j] = 0.f;
+            }
+            if (row < M) {
+#pragma unroll
+                for (int j = 0; j < 16; j++)
+                    if (c0 + j < N) P[(int64_t)(c0 + j) * M + row] = v[j];
+            }
+        }
+    }
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    if (warp == 0) tm_dealloc(tbase, 256);
+}
+
+// The gradient sums and the Adam step after k_dw_tiles, as k_grad_adam takes them: a block per 32 x 32 tile of a
+// weight matrix (the parts are read along the rows, as they were written, and the weights along the columns, by
+// way of shared memory), then a block per layer for its bias (the last one also adds up the loss).
+struct AdamArgs {
+    float lr, b1, b2, eps, c1, c2;
+    int update;
+};
+__device__ __forceinline__ float adam_step(const AdamArgs& a, float* w, float* m, float* v, int64_t i, float g) {
+    // the moments with the new gradient's product fused, the old one's rounded (as the narrow networks' kernel is
+    // compiled): a weight's last bit decides BF16 roundings of the next step
+    const float mi = __fmaf_rn(1.f - a.b1, g, __fmul_rn(a.b1, m[i]));
+    const float vi = __fmaf_rn(__fmul_rn(1.f - a.b2, g), g, __fmul_rn(a.b2, v[i]));
+    m[i] = mi;
+    v[i] = vi;
+    const float wi = w[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    w[i] = wi;
+    return wi;
+}
+__global__ void __launch_bounds__(256) k_adam_tiles(float* __restrict__ w, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
+                                                    const float* __restrict__ ws, const float* __restrict__ loss_part,
+                                                    float* __restrict__ loss, const __grid_constant__ LayerTab tab,
+                                                    const __grid_constant__ AdamArgs a, __nv_bfloat16* __restrict__ wk,
+                                                    __nv_bfloat16* __restrict__ wkt) {
+    __shared__ float s[32][33];
+    int l = 0, r = blockIdx.x;
+    for (; l < tab.L; l++) {
+        const int n = ((tab.fo[l] + 31) / 32) * ((tab.fi[l] + 31) / 32);
+        if (r < n) break;
+        r -= n;
+    }
+    if (l < tab.L) {
+        const int fo = tab.fo[l], fi = tab.fi[l], tr = (fo + 31) / 32, r0 = (r % tr) * 32, c0 = (r / tr) * 32;
+        const int x = threadIdx.x & 31, y = threadIdx.x >> 5, split = tab.split[l];
+        const int64_t nw = (int64_t)fo * fi;
+        const float* P = ws + tab.ws_w[l];
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int c = c0 + y + 8 * e;
+            if (r0 + x < fo && c < fi) {
+                const float* p = P + (int64_t)c * fo + r0 + x;
+                float sum = 0.f;
+                int z = 0;
+                for (; z + 16 <= split; z += 16) {        // sixteen loads in flight, added in order
+                    float q[16];
+#pragma unroll
+                    for (int i = 0; i < 16; i++) q[i] = __ldcs(p + (z + i) * nw);
+#pragma unroll
+                    for (int i = 0; i < 16; i++) sum += q[i];
+                }
+                for (; z < split; z++) sum += p[z * nw];
+                s[y + 8 * e][x] = sum;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int rr = r0 + y + 8 * e, c = c0 + x;
+            if (rr >= fo || c >= fi) continue;
+            const int64_t i = tab.w_off[l] + (int64_t)rr * fi + c;
+            const float gi = s[x][y + 8 * e];
+            if (!a.update) {
+                g[i] = gi;
+                continue;
+            }
+            const __nv_bfloat16 q = __float2bfloat16(adam_step(a, w, m, v, i, gi));
+            wk[tab.wk_off[l] + chain_at(rr, c, tab.rows[l])] = q;
+            if (l > 0 && l + 1 < tab.L) wkt[tab.wk_off[l] + chain_at(c, rr, tab.rows[l])] = q;
+        }
+        return;
+    }
+    // p[0] + p[stride] + ... over the 64-row blocks, in pairs (the row blocks of the launch-per-product form)
+    auto block_sum = [&](const float* p, int64_t stride) {
+        float sum = 0.f;
+        int y = 0;
+        for (; y + 16 <= tab.nrc; y += 16) {
+            float q[16];
+#pragma unroll
+            for (int i = 0; i < 16; i++) q[i] = p[(y + i) * stride];
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) sum += q[i] + q[i + 1];
+        }
+        for (; y < tab.nrc; y += 2) sum += p[y * stride] + (y + 1 < tab.nrc ? p[(y + 1) * stride] : 0.f);
+        return sum;
+    };
+    l = r;                                                // bias blocks
+    const int fo = tab.fo[l], f = threadIdx.x;
+    if (f < fo) {
+        const int64_t i = tab.w_off[l] + (int64_t)fo * tab.fi[l] + f;
+        const float gi = block_sum(ws + tab.ws_b[l] + f, fo);
+        if (a.update) adam_step(a, w, m, v, i, gi);
+        else g[i] = gi;
+    }
+    if (l == tab.L - 1 && f == 32) *loss = block_sum(loss_part, 1);
 }
 
 // BF16 copies of the weights, zero-padded to [fout_pad][fin_pad] and [fin_pad][fout_pad]
@@ -796,7 +953,7 @@ static hyb_status ensure_cap(hyb_mlp* m, int64_t B) {
     size_t nb = 0;
     for (int l = 0; l < m->L; l++) nb += nrb * layer_out(m, l);
     HYB_CUDA_TRY(cudaMalloc(&m->pre, sizeof(float) * na));
-    if (m->chain) {          // inputs of every layer and dH of every layer, feature-major
+    if (m->chain) {          // input and dH of every layer, in the order of the weight gradients' operands
         HYB_CUDA_TRY(cudaMalloc(&m->actT, sizeof(__nv_bfloat16) * (size_t)m->L * cap * 256));
         HYB_CUDA_TRY(cudaMalloc(&m->dhT, sizeof(__nv_bfloat16) * (size_t)m->L * cap * 256));
     } else {
@@ -922,8 +1079,8 @@ static hyb_status chain_pass(hyb_mlp* m, const float* x, int64_t B, float* y, co
         c.db_part[l] = m->ws + m->tab.ws_b[l];
     }
     if (tgt) {
-        c.actT = m->actT;
-        c.dhT = m->dhT;
+        c.act = m->actT;
+        c.dh = m->dhT;
         c.th = m->pre;
         c.loss_part = loss_parts(m);
     }
@@ -945,14 +1102,18 @@ static hyb_status chain_pass(hyb_mlp* m, const float* x, int64_t B, float* y, co
             t.first[l] = nblk;
             t.M[l] = no;
             t.N[l] = ni;
+            t.ra[l] = m->tab.rows[l];
+            t.rb[l] = l == 0 ? pad16(ni) : m->tab.rows[l - 1];
             t.kchunk[l] = ((Kp + split - 1) / split + 15) & ~15;
             t.a[l] = m->dhT + (size_t)l * cap * 256;
             t.b[l] = m->actT + (size_t)l * cap * 256;
             t.c[l] = m->ws + m->tab.ws_w[l];
-            nblk += ((ni + TN - 1) / TN) * ((no + TM - 1) / TM) * split;
+            nblk += ((no + 127) / 128) * split;
         }
         t.first[m->L] = nblk;
-        k_dw_all<<<nblk, GT, 0, s>>>(t, Kp, (int)B, cap, m->err);
+        const cudaError_t room = func_attr_once((const void*)k_dw_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem);
+        if (room != cudaSuccess) return cuda_fail(room, "k_dw_tiles");
+        k_dw_tiles<<<nblk, DT, kDwSmem, s>>>(t, Kp, m->err);
         m->launches++;
     }
     HYB_CUDA_TRY(cudaGetLastError());
@@ -968,10 +1129,18 @@ static hyb_status reduce_update(hyb_mlp* m, int update, float lr, cudaStream_t s
         c1 = 1.f - powf(b1, (float)m->step);
         c2 = 1.f - powf(b2, (float)m->step);
     }
-    const auto kern = m->chain ? k_grad_adam<true> : k_grad_adam<false>;
-    kern<<<(unsigned)((m->n_params + 255) / 256), 256, 0, s>>>(m->master, m->grad, m->adam_m, m->adam_v, m->ws, loss_parts(m), m->loss,
-                                                               (int64_t)m->n_params, update, lr, b1, b2, 1e-8f, c1, c2, m->tab,
-                                                               m->chain ? m->wk : m->wbf, m->chain ? m->wkt : m->wbt);
+    if (m->chain) {
+        const AdamArgs a{lr, b1, b2, 1e-8f, c1, c2, update};
+        int blocks = m->L;
+        for (int l = 0; l < m->L; l++) blocks += ((layer_out(m, l) + 31) / 32) * ((layer_in(m, l) + 31) / 32);
+        k_adam_tiles<<<blocks, 256, 0, s>>>(m->master, m->grad, m->adam_m, m->adam_v, m->ws, loss_parts(m), m->loss, m->tab, a, m->wk, m->wkt);
+        m->launches++;
+        HYB_CUDA_TRY(cudaGetLastError());
+        return HYB_OK;
+    }
+    k_grad_adam<<<(unsigned)((m->n_params + 255) / 256), 256, 0, s>>>(m->master, m->grad, m->adam_m, m->adam_v, m->ws, loss_parts(m),
+                                                                     m->loss, (int64_t)m->n_params, update, lr, b1, b2, 1e-8f, c1,
+                                                                     c2, m->tab, m->wbf, m->wbt);
     m->launches++;
     HYB_CUDA_TRY(cudaGetLastError());
     return HYB_OK;
