@@ -32,7 +32,7 @@
 // the subdivision, which few pairs need but each for a long time, again one pair
 // at a time with seeds and contour points across the lanes.  With one thread per
 // pair doing all of it (before), the few hard pairs ran alone for tens of
-// milliseconds, 3.6 of 32 lanes live: 69 ms for 32256 samples x 3 aliases, 7.1 ms now, of which
+// milliseconds, 3.6 of 32 lanes live: 69 ms for 32256 samples x 3 aliases, 6.1 ms now, of which
 // the counts take a third and the cubic's seeds most of the rest.
 //
 // Readings (the printed forms are garbled here): s_{l,i} = sinc(k'_i dx_i/2)^(l+1)
@@ -222,12 +222,13 @@ __device__ int winding_rect(const NciMode& m, double x0, double x1, double y0, d
 }
 
 // One attempt of Newton's method on G deflated by the nf zeros in r[], advanced one step per call:
-// 0 = go on, 1 = converged to w, -1 = failed.  An attempt has kNewtonMax steps.  Each step is a
+// 0 = go on, 1 = converged to w, -1 = failed.  An attempt has MAX steps.  Each step is a
 // function of w alone, so an attempt that meets a w it has seen (kept at steps 1, 2, 4, 8, ...:
 // a limit cycle at rounding level) can never converge and fails at once.
-constexpr int kNewtonMax = 80;
+constexpr int kNewtonMax = 80, kNewtonFirst = 40;   // the latter for the first seeds (step 2a)
 struct Newton { Z w, seen; int it; };
 __device__ __forceinline__ Newton newton_start(Z w) { return Newton{w, zc(nan(""), 0.0), 0}; }
+template <int MAX>
 __device__ __forceinline__ int newton_step(const NciMode& m, Newton& s, const Z* r, int nf) {
     Z g, dg;
     nci_G<true>(m, s.w, &g, &dg);
@@ -246,14 +247,14 @@ __device__ __forceinline__ int newton_step(const NciMode& m, Newton& s, const Z*
     if (!(isfinite(s.w.re) && isfinite(s.w.im))) return -1;
     // |step| <= 1e-14 max(1, |w|)
     if (step.re * step.re + step.im * step.im <= 1e-28 * fmax(1.0, s.w.re * s.w.re + s.w.im * s.w.im)) return 1;
-    if (++s.it == kNewtonMax || (s.w.re == s.seen.re && s.w.im == s.seen.im)) return -1;
+    if (++s.it == MAX || (s.w.re == s.seen.re && s.w.im == s.seen.im)) return -1;
     if ((s.it & (s.it - 1)) == 0) s.seen = s.w;
     return 0;
 }
 __device__ bool newton_deflated(const NciMode& m, Z w, const Z* r, int nf, Z* out) {
     Newton s = newton_start(w);
     int st;
-    while ((st = newton_step(m, s, r, nf)) == 0) {}
+    while ((st = newton_step<kNewtonMax>(m, s, r, nf)) == 0) {}
     *out = s.w;
     return st > 0;
 }
@@ -484,7 +485,9 @@ __global__ void __launch_bounds__(kNciThreads) k_nci(const NciSample* __restrict
     }
     if (N < 0 || N > kMaxRoots) { e |= (N < 0) ? NCI_EUNRESOLVED : NCI_ETOOMANY; N = 0; }
     // ---- 2a. the cubic's roots inside the disk and the resonance as seeds, a pair per lane; one
-    // Newton step of every lane's current attempt per turn
+    // Newton step of every lane's current attempt per turn.  An attempt that converges does so in some ten
+    // steps; one that has not after kNewtonFirst would keep the other lanes waiting (with 80 a warp took 72 turns at
+    // 8.3 live lanes), and the rings find what it would have.
     {
         Z cub[3];
         bool have = false;
@@ -503,7 +506,7 @@ __global__ void __launch_bounds__(kNciThreads) k_nci(const NciSample* __restrict
         next();
         while (__any_sync(0xffffffffu, q < 4)) {
             if (q < 4) {
-                const int st = newton_step(m, s, r, nf);
+                const int st = newton_step<kNewtonFirst>(m, s, r, nf);
                 if (st > 0 && zabs(zsub(s.w, zc(c, 0.0))) < rho) {
                     r[nf++] = s.w;
                     // G's coefficients are real: the conjugate of a zero well off the real axis is another
@@ -517,9 +520,9 @@ __global__ void __launch_bounds__(kNciThreads) k_nci(const NciSample* __restrict
             __syncwarp();
         }
     }
-    // ---- 2b. the rings, one pair after the other, a seed per lane: an attempt that finds nothing
-    // leaves the others' deflation as it was, so all run at once; the first that succeeds is kept
-    // and those after it run again, deflated by it too
+    // ---- 2b. the rings, one pair after the other, a seed per lane.  The first attempt that finds a zero adds it to
+    // the deflation, and all start again from their seeds (one that went on from beside that zero could
+    // end on it once more)
     for (unsigned todo = __ballot_sync(0xffffffffu, nf < N); todo; todo &= todo - 1) {
         const int j = __ffs(todo) - 1;
         const NciMode& mj = modes[warp][j];
@@ -527,28 +530,32 @@ __global__ void __launch_bounds__(kNciThreads) k_nci(const NciSample* __restrict
         const Z cj = zc(__shfl_sync(0xffffffffu, c, j), 0.0);
         const double rhoj = __shfl_sync(0xffffffffu, rho, j);
         const int Nj = __shfl_sync(0xffffffffu, N, j);
-        int nj = __shfl_sync(0xffffffffu, nf, j), from = 0;
-        while (nj < Nj && from < kRingSeeds) {
-            bool found = false;
-            Z w = zc(0.0, 0.0);
-            if (lane >= from && lane < kRingSeeds) {
-                const int ring = lane / kRing, k = lane % kRing;
-                const double rr = rhoj * (0.15 + 0.3 * ring);
-                double sn, cs;
-                sincospi((2.0 * k + 0.5 * ring) / kRing, &sn, &cs);
-                found = newton_deflated(mj, zc(cj.re + rr * cs, cj.im + rr * sn), rj, nj, &w) && zabs(zsub(w, cj)) < rhoj;
+        int nj = __shfl_sync(0xffffffffu, nf, j);
+        const int ring = lane / kRing;
+        const double rr = rhoj * (0.15 + 0.3 * ring);
+        double sn, cs;
+        sincospi((2.0 * (lane % kRing) + 0.5 * ring) / kRing, &sn, &cs);
+        const Z seed = zc(cj.re + rr * cs, cj.im + rr * sn);
+        Newton s = newton_start(seed);
+        bool go = lane < kRingSeeds;
+        while (true) {
+            const int st = go ? newton_step<kNewtonMax>(mj, s, rj, nj) : 0;
+            const unsigned hit = __ballot_sync(0xffffffffu, st > 0 && zabs(zsub(s.w, cj)) < rhoj);
+            if (st != 0) go = false;
+            if (hit) {
+                const int win = __ffs(hit) - 1;
+                const bool pair = __shfl_sync(0xffffffffu, fabs(s.w.im) > kPairIm * rhoj, win) && nj + 1 < Nj;
+                if (lane == win) {
+                    rj[nj] = s.w;
+                    if (pair) rj[nj + 1] = zc(s.w.re, -s.w.im);
+                }
+                __syncwarp();
+                nj += pair ? 2 : 1;
+                if (nj >= Nj) break;
+                s = newton_start(seed);
+                go = lane < kRingSeeds;
             }
-            const unsigned hit = __ballot_sync(0xffffffffu, found);
-            if (!hit) break;
-            const int win = __ffs(hit) - 1;
-            const bool pair = __shfl_sync(0xffffffffu, fabs(w.im) > kPairIm * rhoj, win) && nj + 1 < Nj;
-            if (lane == win) {
-                rj[nj] = w;
-                if (pair) rj[nj + 1] = zc(w.re, -w.im);
-            }
-            __syncwarp();
-            nj += pair ? 2 : 1;
-            from = win + 1;
+            if (!__any_sync(0xffffffffu, go)) break;
         }
         // ---- 3. what the seeds left
         int ej = 0;
