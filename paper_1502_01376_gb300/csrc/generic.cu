@@ -354,7 +354,9 @@ static cudaError_t launch_rfft(const RowPtrs& p, int nf, cplx<T>* out, int n1, i
             k_rfft1024<<<(unsigned)blocks, 256, 0, s>>>(p, out, rows, nf, t.tw8, t.twN);
             return cudaGetLastError();
         }
-        if (row_reg_supported(n1, rows)) return row_reg_rfft(p, nf, out, n1, rows, t, s);
+    }
+    if constexpr (std::is_same<Tin, T>::value) {
+        if (row_reg_supported<T>(n1, rows)) return row_reg_rfft(p, nf, out, n1, rows, t, s);
     }
     const int RB = fft_rows_per_launch(n1 / 2, rows * nf);
     const size_t smem = row_fft_smem<T>(n1, RB);
@@ -376,10 +378,9 @@ static cudaError_t launch_irfft(const cplx<T>* in, int f0, const RowPtrsW& p, in
             k_irfft1024<<<dim3((unsigned)((rows + kRows1k - 1) / kRows1k), nf), 256, 0, s>>>(in, p, rows, t.tw8, t.twN, f0);
             return cudaGetLastError();
         }
-        if (row_reg_supported(n1, rows)) {
-            RowPtrsW q = p;
-            return row_reg_irfft(in + (int64_t)f0 * rows * (n1 / 2 + 1), q, nf, n1, rows, t, s);
-        }
+    }
+    if constexpr (std::is_same<T, Tout>::value) {
+        if (row_reg_supported<T>(n1, rows)) return row_reg_irfft(in + (int64_t)f0 * rows * (n1 / 2 + 1), p, nf, n1, rows, t, s);
     }
     const int RB = fft_rows_per_launch(n1 / 2, rows * nf);
     const size_t smem = row_fft_smem<T>(n1, RB);
@@ -538,9 +539,11 @@ template <typename T> static const ModeTables<T>& tables(hyb_grid* g);
 template <> const ModeTables<float>& tables<float>(hyb_grid* g) { return g->tf; }
 template <> const ModeTables<double>& tables<double>(hyb_grid* g) { return g->td; }
 
-// FP32 off the DFT-GEMM path, rows of at least 128 points: Ampere runs inside the inverse transform
+// off the DFT-GEMM path, where the register-resident transforms apply: Ampere runs inside the inverse transform
 static bool amp_fused(const hyb_grid* g) {
-    return g->d.precision == 32 && g->path < 3 && g->d.dims != 20 && (g->d.n1 == 1024 || row_reg_supported(g->d.n1, g->rows));
+    return g->path < 3 && g->d.dims != 20 &&
+           (g->d.precision == 32 ? g->d.n1 == 1024 || row_reg_supported<float>(g->d.n1, g->rows)
+                                 : row_reg_supported<double>(g->d.n1, g->rows));
 }
 
 template <typename T>
@@ -575,25 +578,22 @@ hyb_status generic_advance(hyb_grid* g, int nsteps, bool have_spectra) {
         }
         if (g->resident) g->res_stale = false;
         const dim3 mgrid((unsigned)((int64_t)g->d.n3 * ((g->d.n2 + kModeRows - 1) / kModeRows) * ((nk + 31) / 32))), mblk(32, kModeRows);
-        if constexpr (std::is_same<T, float>::value) {
-            if (amp_fused(g)) {
-                float2* sp = reinterpret_cast<float2*>(spec);
+        if (amp_fused(g)) {
+            const int n3 = d3 ? g->d.n3 : 1;
+            if (d3) k_faraday<T, true><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, n3, rows, t.S, a2, a3);
+            else k_faraday<T, false><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, 1, rows, t.S, a2, a3);
+            HYB_CUDA_TRY(cudaGetLastError());
+            if (std::is_same<T, double>::value || n1 != 1024) {
+                HYB_CUDA_TRY(row_reg_ampere(spec, fout, n1, rows, g->d.n2, n3, d3, g->resident, t, a2, a3, g->stream));
+            } else if constexpr (std::is_same<T, float>::value) {
                 const unsigned nb = (unsigned)((rows + kRows1k - 1) / kRows1k) * 6u;
-                const int n3 = d3 ? g->d.n3 : 1;
-                if (d3) k_faraday<T, true><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, n3, rows, t.S, a2, a3);
-                else k_faraday<T, false><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, 1, rows, t.S, a2, a3);
-                if (n1 != 1024) {
-                    HYB_CUDA_TRY(row_reg_ampere(sp, fout, n1, rows, g->d.n2, n3, d3, g->resident, t, a2, a3, g->stream));
-                    if (g->ev_stop) HYB_CUDA_TRY(cudaEventRecord(g->ev_stop, g->stream));
-                    continue;
-                }
                 auto amp = d3 ? (g->resident ? k_ampere_irfft1024<true, true> : k_ampere_irfft1024<true, false>)
                               : (g->resident ? k_ampere_irfft1024<false, true> : k_ampere_irfft1024<false, false>);
-                amp<<<nb, 256, 0, g->stream>>>(sp, fout, rows, g->d.n2, n3, t.tw8, t.twN, t.S, t.cj1, t.cj, a2, a3);
+                amp<<<nb, 256, 0, g->stream>>>(spec, fout, rows, g->d.n2, n3, t.tw8, t.twN, t.S, t.cj1, t.cj, a2, a3);
                 HYB_CUDA_TRY(cudaGetLastError());
-                if (g->ev_stop) HYB_CUDA_TRY(cudaEventRecord(g->ev_stop, g->stream));
-                continue;
             }
+            if (g->ev_stop) HYB_CUDA_TRY(cudaEventRecord(g->ev_stop, g->stream));
+            continue;
         }
         if (d3) {
             k_faraday<T, true><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, g->d.n3, rows, t.S, a2, a3);

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
         }
         // asked for before the tile is staged, used after it
         T uu[3] = {(T)0, (T)0, (T)0}, qmp = (T)0;
-        if (live) {
+        if (sizeof(T) == 4 && live) {        // (FP64 has no registers to hold them)
             uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2];
             qmp = qm[p];
         }
@@ -157,6 +157,10 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
         }
         __syncthreads();
         if (ok) {
+            if (sizeof(T) == 8) {
+                uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2];
+                qmp = qm[p];
+            }
             // weights for the integer (0) and half (1) positions along each axis
             T wx[2][L + 1], wy[2][L + 1];
             const int ix0 = pweights<L>(ox, wx[0]), ix1 = pweights<L>(ox - (T)0.5, wx[1]);
