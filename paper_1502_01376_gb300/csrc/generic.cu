@@ -3,8 +3,8 @@
 //   (2) per-k1-mode Faraday then Ampere updates with finite differences in
 //       x2 (and x3) (Eqs. hybrid2db1-hybrid2de3; Sec. 2.4 for 3D),
 //   (3) batched inverse real FFT of E, B back in place.
-// For FP32 rows of 1024 points the Ampere update of (2) is folded into (3),
-// which then reads the spectra of E, B, j and writes E, B (three launches).
+// Where the register-resident row transforms apply (rowfft_api.cuh) the Ampere update of (2) is folded into (3), and on
+// larger FP32 grids the transforms of j, then those of B, into the updates (three launches, two in k1-resident steps).
 // It also provides the row FFTs used by the standalone current processing and
 // the diagnostics.  The x1 transform is a shared-memory Stockham FFT (radix 8,
 // then one radix-4 or radix-2 pass; several short rows per block)
@@ -108,232 +108,6 @@ __global__ void __launch_bounds__(kRowThreads) k_irfft_rows(const cplx<T>* __res
     }
 }
 
-// ---------------------------------------------------------------- n1 = 1024, FP32: register-resident row FFT
-// The 512-point complex FFT of z[j] = x[2j] + i x[2j+1], factored 8 x 8 x 8 over 64 threads per
-// row (8 points each), the exchanges through shared memory, then the real-input split in
-// (k, M - k) pairs:
-//   S1  thread t: z[t + 64 n], DFT8 over n -> k1, twiddle W_512^{t k1}          -> A(k1, t)
-//   S2  (t0, k1) = (t & 7, t >> 3): A(k1, t0 + 8 t1), DFT8 over t1 -> k2,
-//       twiddle W_64^{t0 k2}                                                  -> B[9 (8 k1 + k2) + t0]
-//   S3  (k1, k2) = (t >> 3, t & 7): B[9 (8 k1 + k2) + t0], DFT8 over t0 -> Z[k1 + 8 k2 + 64 k3]
-// A(k, t) is stored at 72 k + t and Z[k] at a swizzled position (both against bank conflicts); the
-// twiddles of S1 and S2 come from a table laid out in the order the threads read them.
-// The inverse runs the stages
-// transposed with conjugate twiddles.  Four rows per block, one named barrier per row.
-constexpr int kRows1k = 4;
-constexpr int kBuf1k = 576;
-// Z[k] at k with bits 2 and 1 flipped by bits 4 and 5: a half-warp's 8-byte accesses of the S3
-// scatter (lanes over bits 0, 3, 4, 5 of k) and of the split (16 consecutive k) both reach 16
-// different bank pairs
-__device__ __forceinline__ int zp1k(int k) { return k ^ (((k >> 4) & 1) << 2) ^ (((k >> 5) & 1) << 1); }
-// stage-1 output (k1, t) position
-__device__ __forceinline__ int ap1k(int k, int t) { return 72 * k + t; }
-__device__ __forceinline__ float2 cm(float2 a, float2 b) { return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x)); }
-__device__ __forceinline__ float2 cmc(float2 a, float2 b) { return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y)); }
-
-// Persistent: each 64-thread team (four per block) walks the rows j = team, team + teams, ... of all
-// fields (field j / rows), holding the next row's samples in registers while it transforms the
-// current one, so that every team keeps a row of loads in flight.
-__global__ void __launch_bounds__(256, 3) k_rfft1024(RowPtrs in, float2* __restrict__ out, int64_t rows, int nf,
-                                                  const float2* __restrict__ tw8, const float2* __restrict__ twN) {
-    __shared__ float2 sbuf[kRows1k][2][kBuf1k];
-    const int L = threadIdx.x >> 6, t = threadIdx.x & 63;
-    const int64_t total = rows * nf, teams = (int64_t)gridDim.x * kRows1k;
-    float2* A = sbuf[L][0];
-    float2* B = sbuf[L][1];
-    auto lsync = [&]() { asm volatile("bar.sync %0, %1;" :: "r"(1 + L), "r"(64) : "memory"); };
-    float2 nx[8], w1[8], w2[8];
-#pragma unroll
-    for (int k = 1; k < 8; k++) {
-        w1[k] = tw8[(k - 1) * 64 + t];
-        w2[k] = tw8[448 + (k - 1) * 8 + (t & 7)];
-    }
-    auto fetch = [&](int64_t j) {
-        const int f = (int)(j / rows);
-        const float2* z = reinterpret_cast<const float2*>(in.p[f]) + (j - (int64_t)f * rows) * 512;
-#pragma unroll
-        for (int n = 0; n < 8; n++) nx[n] = __ldcs(z + t + 64 * n);
-    };
-    int64_t j = (int64_t)blockIdx.x * kRows1k + L;
-    if (j < total) fetch(j);
-    for (; j < total; j += teams) {
-        float2 v[8];
-#pragma unroll
-        for (int n = 0; n < 8; n++) v[n] = nx[n];
-        if (j + teams < total) fetch(j + teams);
-        dft8x<false>(v);
-#pragma unroll
-        for (int k = 1; k < 8; k++) v[k] = cm(v[k], w1[k]);
-        lsync();                     // the previous row's split has read A
-#pragma unroll
-        for (int k = 0; k < 8; k++) A[ap1k(k, t)] = v[k];
-        lsync();
-        {
-            const int t0 = t & 7, k1 = t >> 3;
-#pragma unroll
-            for (int n = 0; n < 8; n++) v[n] = A[ap1k(k1, t0 + 8 * n)];
-            dft8x<false>(v);
-#pragma unroll
-            for (int k = 1; k < 8; k++) v[k] = cm(v[k], w2[k]);
-#pragma unroll
-            for (int k = 0; k < 8; k++) B[9 * (8 * k1 + k) + t0] = v[k];
-        }
-        lsync();
-        {
-            const int k1 = t >> 3, k2 = t & 7;
-#pragma unroll
-            for (int n = 0; n < 8; n++) v[n] = B[9 * (8 * k1 + k2) + n];
-            dft8x<false>(v);
-#pragma unroll
-            for (int k = 0; k < 8; k++) A[zp1k(k1 + 8 * k2 + 64 * k)] = v[k];
-        }
-        lsync();
-        float2* X = out + j * 513;   // [field][row][513], j = field * rows + row
-        // X[k] = e - u, X[M-k] = conj(e + u), e = (Z[k] + Z*[M-k])/2, u = (i/2) W_N^k (Z[k] - Z*[M-k])
-        auto pair = [&](int k) {
-            const float2 zk = A[zp1k(k)], zm = A[zp1k((512 - k) & 511)];
-            const float2 e = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-            const float2 wd = cm(twN[k], make_float2(zk.x - zm.x, zk.y + zm.y));
-            X[k] = make_float2(e.x + 0.5f * wd.y, e.y - 0.5f * wd.x);
-            if (k != 256) X[512 - k] = make_float2(e.x - 0.5f * wd.y, -(e.y + 0.5f * wd.x));
-        };
-#pragma unroll
-        for (int m = 0; m < 4; m++) pair(t + 64 * m);
-        if (t == 0) pair(256);
-    }
-}
-
-// Inverse of one row from its spectrum, X[k] = ld(k) for k = 0..M (the stages of k_rfft1024 in
-// reverse with conjugate twiddles); z_out receives the 1024 real samples (nullptr: dead row).
-template <class Ld>
-__device__ __forceinline__ void irfft1024_row(float2* A, float2* B, int L, int t, float2* __restrict__ z_out,
-                                              const float2* __restrict__ tw8, const float2* __restrict__ twN, Ld ld) {
-    auto lsync = [&]() { asm volatile("bar.sync %0, %1;" :: "r"(1 + L), "r"(64) : "memory"); };
-    {
-        // Z[k] = E + iO, Z[M-k] = conj(E - iO), E = (X[k] + X*[M-k])/2, O = conj(W_N^k)(X[k] - X*[M-k])/2;
-        // the imaginary parts of X[0] and X[M] are dropped
-        auto pair = [&](int k) {
-            float2 xk = ld(k);
-            float2 xm = k == 256 ? xk : ld(512 - k);        // each mode loaded once
-            if (k == 0) { xk.y = 0.f; xm.y = 0.f; }
-            const float2 e = make_float2(0.5f * (xk.x + xm.x), 0.5f * (xk.y - xm.y));
-            const float2 o = cmc(make_float2(0.5f * (xk.x - xm.x), 0.5f * (xk.y + xm.y)), twN[k]);
-            A[zp1k(k)] = make_float2(e.x - o.y, e.y + o.x);
-            if (k != 0 && k != 256) A[zp1k(512 - k)] = make_float2(e.x + o.y, o.x - e.y);
-        };
-#pragma unroll
-        for (int m = 0; m < 4; m++) pair(t + 64 * m);
-        if (t == 0) pair(256);
-    }
-    lsync();
-    float2 v[8];
-    {
-        const int k1 = t >> 3, k2 = t & 7;
-#pragma unroll
-        for (int k = 0; k < 8; k++) v[k] = A[zp1k(k1 + 8 * k2 + 64 * k)];
-        dft8x<true>(v);
-#pragma unroll
-        for (int n = 0; n < 8; n++) B[9 * (8 * k1 + k2) + n] = v[n];
-    }
-    lsync();
-    {
-        const int t0 = t & 7, k1 = t >> 3;
-#pragma unroll
-        for (int k = 0; k < 8; k++) v[k] = B[9 * (8 * k1 + k) + t0];
-#pragma unroll
-        for (int k = 1; k < 8; k++) v[k] = cmc(v[k], tw8[448 + (k - 1) * 8 + t0]);
-        dft8x<true>(v);
-#pragma unroll
-        for (int n = 0; n < 8; n++) A[ap1k(k1, t0 + 8 * n)] = v[n];
-    }
-    lsync();
-#pragma unroll
-    for (int k = 0; k < 8; k++) v[k] = A[ap1k(k, t)];
-#pragma unroll
-    for (int k = 1; k < 8; k++) v[k] = cmc(v[k], tw8[(k - 1) * 64 + t]);
-    dft8x<true>(v);
-    if (z_out) {
-        const float inv = 1.f / 512.f;
-#pragma unroll
-        for (int n = 0; n < 8; n++) z_out[t + 64 * n] = make_float2(v[n].x * inv, v[n].y * inv);
-    }
-}
-
-__global__ void __launch_bounds__(256) k_irfft1024(const float2* __restrict__ in, RowPtrsW out, int64_t rows,
-                                                   const float2* __restrict__ tw8, const float2* __restrict__ twN,
-                                                   int in_field0) {
-    __shared__ float2 sbuf[kRows1k][2][kBuf1k];
-    const int L = threadIdx.x >> 6, t = threadIdx.x & 63;
-    const int64_t row = (int64_t)blockIdx.x * kRows1k + L;
-    const bool live = row < rows;
-    const int f = blockIdx.y;
-    const float2* X = in + ((int64_t)(in_field0 + f) * rows + (live ? row : 0)) * 513;
-    float2* z = live ? reinterpret_cast<float2*>(out.p[f]) + row * 512 : nullptr;
-    irfft1024_row(sbuf[L][0], sbuf[L][1], L, t, z, tw8, twN, [&](int k) { return X[k]; });
-}
-
-// Ampere (Eqs. hybrid2de1-hybrid2de3; the x3 differences of Sec. 2.4) fused into the inverse
-// transform of E, B: blocks of kRows1k rows of one field, the six fields of a row group in
-// consecutive blocks so that the B rows three of them read come from L2.  Fields 0-2 apply Ampere
-// to E_f mode by mode as they load it (Sm = -conj(S) = c dt sigma-):
-//   E1 += a2 d2-B3 - a3 d3-B2 - cj1 J1;  E2 += a3 d3-B1 - Sm B3 - cj J2;  E3 += Sm B2 - a2 d2-B1 - cj J3
-// fields 3-5 invert B.  Without WB the spectral scratch is only read; with WB (k1-resident
-// state) the updated E spectrum is also stored back in place (each mode of a row is loaded once,
-// by the block of that row and field).
-template <bool D3, bool WB>
-__global__ void __launch_bounds__(256, 3) k_ampere_irfft1024(float2* __restrict__ spec, RowPtrsW out, int64_t rows, int n2, int n3,
-                                                          const float2* __restrict__ tw8, const float2* __restrict__ twN,
-                                                          const float2* __restrict__ S, const float* __restrict__ cj1,
-                                                          const float* __restrict__ cj, float a2, float a3) {
-    __shared__ float2 sbuf[kRows1k][2][kBuf1k];
-    const int L = threadIdx.x >> 6, t = threadIdx.x & 63;
-    const int f = blockIdx.x % 6;
-    const int64_t row = (int64_t)(blockIdx.x / 6) * kRows1k + L;
-    const bool live = row < rows;
-    const int64_t r = live ? row : 0;
-    const int64_t i3 = r / n2;
-    const int i2 = (int)(r - i3 * n2);
-    const int64_t fs = rows * 513;
-    float2* Xr = spec + r * 513;                                                  // field 0 of row r
-    const float2* Xm2 = spec + (i3 * n2 + (i2 == 0 ? n2 - 1 : i2 - 1)) * 513;     // row i2 - 1
-    const float2* Xm3 = spec + ((D3 ? (i3 == 0 ? n3 - 1 : i3 - 1) : i3) * n2 + i2) * 513;   // row i3 - 1
-    float2* z = live ? reinterpret_cast<float2*>(out.p[f]) + row * 512 : nullptr;
-    auto sub = [](float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); };
-    auto axpy = [](float2 y, float s, float2 x) { return make_float2(fmaf(s, x.x, y.x), fmaf(s, x.y, y.y)); };
-    auto keep = [&](float2* at, float2 e) {
-        if (WB && live) *at = e;
-        return e;
-    };
-    if (f == 0) {
-        irfft1024_row(sbuf[L][0], sbuf[L][1], L, t, z, tw8, twN, [&](int k) {
-            float2 e = axpy(Xr[k], a2, sub(Xr[5 * fs + k], Xm2[5 * fs + k]));
-            if (D3) e = axpy(e, -a3, sub(Xr[4 * fs + k], Xm3[4 * fs + k]));
-            return keep(Xr + k, axpy(e, -cj1[k], Xr[6 * fs + k]));
-        });
-    } else if (f == 1) {
-        irfft1024_row(sbuf[L][0], sbuf[L][1], L, t, z, tw8, twN, [&](int k) {
-            const float2 s = S[k], b3 = Xr[5 * fs + k];
-            // - Sm B3 = conj(S) B3
-            float2 e = Xr[fs + k];
-            e = make_float2(e.x + (s.x * b3.x + s.y * b3.y), e.y + (s.x * b3.y - s.y * b3.x));
-            if (D3) e = axpy(e, a3, sub(Xr[3 * fs + k], Xm3[3 * fs + k]));
-            return keep(Xr + fs + k, axpy(e, -cj[k], Xr[7 * fs + k]));
-        });
-    } else if (f == 2) {
-        irfft1024_row(sbuf[L][0], sbuf[L][1], L, t, z, tw8, twN, [&](int k) {
-            const float2 s = S[k], b2 = Xr[4 * fs + k];
-            // + Sm B2 = - conj(S) B2
-            float2 e = Xr[2 * fs + k];
-            e = make_float2(e.x - (s.x * b2.x + s.y * b2.y), e.y - (s.x * b2.y - s.y * b2.x));
-            e = axpy(e, -a2, sub(Xr[3 * fs + k], Xm2[3 * fs + k]));
-            return keep(Xr + 2 * fs + k, axpy(e, -cj[k], Xr[8 * fs + k]));
-        });
-    } else {
-        const float2* X = Xr + f * fs;
-        irfft1024_row(sbuf[L][0], sbuf[L][1], L, t, z, tw8, twN, [&](int k) { return X[k]; });
-    }
-}
-
 template <typename T>
 static size_t row_fft_smem(int n1, int RB) { return sizeof(cplx<T>) * 2 * fpad_size((size_t)RB * (n1 / 2)); }
 template <typename T>
@@ -345,16 +119,6 @@ static size_t max_row_fft_smem() {
 
 template <typename Tin, typename T>
 static cudaError_t launch_rfft(const RowPtrs& p, int nf, cplx<T>* out, int n1, int64_t rows, const ModeTables<T>& t, cudaStream_t s) {
-    if constexpr (std::is_same<Tin, float>::value && std::is_same<T, float>::value) {
-        if (n1 == 1024) {
-            const cudaError_t carve = func_attr_once((const void*)k_rfft1024, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-            if (carve != cudaSuccess) return carve;
-            const int resident = resident_grid((const void*)k_rfft1024, 256, 0);
-            const int64_t blocks = std::min<int64_t>((rows * nf + kRows1k - 1) / kRows1k, resident);
-            k_rfft1024<<<(unsigned)blocks, 256, 0, s>>>(p, out, rows, nf, t.tw8, t.twN);
-            return cudaGetLastError();
-        }
-    }
     if constexpr (std::is_same<Tin, T>::value) {
         if (row_reg_supported<T>(n1, rows)) return row_reg_rfft(p, nf, out, n1, rows, t, s);
     }
@@ -371,14 +135,6 @@ static cudaError_t launch_rfft(const RowPtrs& p, int nf, cplx<T>* out, int n1, i
 
 template <typename T, typename Tout>
 static cudaError_t launch_irfft(const cplx<T>* in, int f0, const RowPtrsW& p, int nf, int n1, int64_t rows, const ModeTables<T>& t, cudaStream_t s) {
-    if constexpr (std::is_same<T, float>::value && std::is_same<Tout, float>::value) {
-        if (n1 == 1024) {
-            const cudaError_t carve = func_attr_once((const void*)k_irfft1024, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-            if (carve != cudaSuccess) return carve;
-            k_irfft1024<<<dim3((unsigned)((rows + kRows1k - 1) / kRows1k), nf), 256, 0, s>>>(in, p, rows, t.tw8, t.twN, f0);
-            return cudaGetLastError();
-        }
-    }
     if constexpr (std::is_same<T, Tout>::value) {
         if (row_reg_supported<T>(n1, rows)) return row_reg_irfft(in + (int64_t)f0 * rows * (n1 / 2 + 1), p, nf, n1, rows, t, s);
     }
@@ -539,11 +295,10 @@ template <typename T> static const ModeTables<T>& tables(hyb_grid* g);
 template <> const ModeTables<float>& tables<float>(hyb_grid* g) { return g->tf; }
 template <> const ModeTables<double>& tables<double>(hyb_grid* g) { return g->td; }
 
-// off the DFT-GEMM path, where the register-resident transforms apply: Ampere runs inside the inverse transform
-static bool amp_fused(const hyb_grid* g) {
+// off the DFT-GEMM path, where the register-resident transforms apply, the updates run inside them
+static bool row_reg_step(const hyb_grid* g) {
     return g->path < 3 && g->d.dims != 20 &&
-           (g->d.precision == 32 ? g->d.n1 == 1024 || row_reg_supported<float>(g->d.n1, g->rows)
-                                 : row_reg_supported<double>(g->d.n1, g->rows));
+           (g->d.precision == 32 ? row_reg_supported<float>(g->d.n1, g->rows) : row_reg_supported<double>(g->d.n1, g->rows));
 }
 
 template <typename T>
@@ -564,33 +319,39 @@ hyb_status generic_advance(hyb_grid* g, int nsteps, bool have_spectra) {
         if (g->ev_start) HYB_CUDA_TRY(cudaEventRecord(g->ev_start, g->stream));
         // k1-resident state: the spectra of E and B left by the previous step are this step's
         // input, so only j is transformed (the first step after hyb_set_resident imports E, B)
-        const int f0 = (g->resident && !g->res_stale) || (have_spectra && s == 0) ? 6 : 0;
+        const bool have = (g->resident && !g->res_stale) || (have_spectra && s == 0);
+        const int f0 = have ? 6 : 0;
+        const bool in_rows = row_reg_step(g);
+        // FP32: the updates transform j, or j and B, themselves (with E and B in k1 space always: two launches)
+        RowForm form = RowForm::kAll;
+        if (in_rows && std::is_same<T, float>::value) form = have ? RowForm::kEB : row_form(n1, rows * n1);
+        const int f1 = form == RowForm::kAll ? 9 : form == RowForm::kEB ? 6 : 3;
         RowPtrs fin{};
-        for (int c = f0; c < 9; c++) fin.p[c - f0] = src9[c];
+        for (int c = f0; c < f1; c++) fin.p[c - f0] = src9[c];
         C* spec_in = spec + (int64_t)f0 * rows * nk;
         if (g->path >= 3) {
             const float* fsrc[9];
             for (int c = f0; c < 9; c++) fsrc[c - f0] = (const float*)src9[c];
             hyb_status st = dftgemm_forward(g, fsrc, 9 - f0, reinterpret_cast<float2*>(spec_in));
             if (st != HYB_OK) return st;
-        } else {
-            HYB_CUDA_TRY((launch_rfft<T, T>(fin, 9 - f0, spec_in, n1, rows, t, g->stream)));
+        } else if (f1 > f0) {
+            HYB_CUDA_TRY((launch_rfft<T, T>(fin, f1 - f0, spec_in, n1, rows, t, g->stream)));
         }
         if (g->resident) g->res_stale = false;
         const dim3 mgrid((unsigned)((int64_t)g->d.n3 * ((g->d.n2 + kModeRows - 1) / kModeRows) * ((nk + 31) / 32))), mblk(32, kModeRows);
-        if (amp_fused(g)) {
+        if (in_rows) {
             const int n3 = d3 ? g->d.n3 : 1;
-            if (d3) k_faraday<T, true><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, n3, rows, t.S, a2, a3);
-            else k_faraday<T, false><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, 1, rows, t.S, a2, a3);
-            HYB_CUDA_TRY(cudaGetLastError());
-            if (std::is_same<T, double>::value || n1 != 1024) {
+            if (form != RowForm::kE) {
+                if (d3) k_faraday<T, true><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, n3, rows, t.S, a2, a3);
+                else k_faraday<T, false><<<mgrid, mblk, 0, g->stream>>>(spec, nk, g->d.n2, 1, rows, t.S, a2, a3);
+                HYB_CUDA_TRY(cudaGetLastError());
+            }
+            if (form == RowForm::kAll) {
                 HYB_CUDA_TRY(row_reg_ampere(spec, fout, n1, rows, g->d.n2, n3, d3, g->resident, t, a2, a3, g->stream));
             } else if constexpr (std::is_same<T, float>::value) {
-                const unsigned nb = (unsigned)((rows + kRows1k - 1) / kRows1k) * 6u;
-                auto amp = d3 ? (g->resident ? k_ampere_irfft1024<true, true> : k_ampere_irfft1024<true, false>)
-                              : (g->resident ? k_ampere_irfft1024<false, true> : k_ampere_irfft1024<false, false>);
-                amp<<<nb, 256, 0, g->stream>>>(spec, fout, rows, g->d.n2, n3, t.tw8, t.twN, t.S, t.cj1, t.cj, a2, a3);
-                HYB_CUDA_TRY(cudaGetLastError());
+                RowPtrs j{};
+                for (int c = 0; c < 3; c++) j.p[c] = g->J[c];
+                HYB_CUDA_TRY(row_reg_update(spec, fout, j, n1, rows, g->d.n2, n3, d3, form == RowForm::kE, g->resident, t, a2, a3, g->stream));
             }
             if (g->ev_stop) HYB_CUDA_TRY(cudaEventRecord(g->ev_stop, g->stream));
             continue;
@@ -682,7 +443,10 @@ template hyb_status generic_resident_import<double>(hyb_grid*);
 template hyb_status generic_b_half<float>(hyb_grid*, void* const*);
 template hyb_status generic_b_half<double>(hyb_grid*, void* const*);
 
-int generic_launches_per_step(const hyb_grid* g) { return (amp_fused(g) || g->d.dims == 20) ? 3 : 4; }
+int generic_launches_per_step(const hyb_grid* g) {
+    if (g->resident && g->d.precision == 32 && row_reg_step(g)) return 2;      // j is transformed inside the Ampere update
+    return (row_reg_step(g) || g->d.dims == 20) ? 3 : 4;
+}
 
 template hyb_status generic_advance<float>(hyb_grid*, int, bool);
 template hyb_status generic_advance<double>(hyb_grid*, int, bool);

@@ -135,9 +135,8 @@ static hyb_status upload_tables(hyb_grid* g, const HostModes& h, ModeTables<T>& 
         const double b = -2.0 * kPi * (double)j / (double)d.n1;
         twN[j] = mkc<C>((T)cos(b), (T)sin(b));
     }
-    const std::vector<C> tw8 = M == 512 ? tw8_table<C>() : std::vector<C>();
     const std::vector<C> twS = stockham_twiddles<C>(M);
-    const size_t bytes = sizeof(C) * (4 * (size_t)nk + 3 * (size_t)M + tw8.size()) + sizeof(T) * 4 * (size_t)nk + 256;
+    const size_t bytes = sizeof(C) * (4 * (size_t)nk + 3 * (size_t)M) + sizeof(T) * 4 * (size_t)nk + 256;
     char* base = nullptr;
     HYB_CUDA_TRY(cudaMalloc(&base, bytes));
     char* p = base;
@@ -150,7 +149,6 @@ static hyb_status upload_tables(hyb_grid* g, const HostModes& h, ModeTables<T>& 
     t.cj = (T*)take(sizeof(T) * nk);
     t.corr = (T*)take(sizeof(T) * nk);
     t.filt = (T*)take(sizeof(T) * nk);
-    if (!tw8.empty()) t.tw8 = (C*)take(sizeof(C) * tw8.size());
     t.twS = (C*)take(sizeof(C) * M);
     HYB_CUDA_TRY(cudaMemcpy(t.S, S.data(), sizeof(C) * nk, cudaMemcpyHostToDevice));
     HYB_CUDA_TRY(cudaMemcpy(t.sgp, sgp.data(), sizeof(C) * nk, cudaMemcpyHostToDevice));
@@ -160,7 +158,6 @@ static hyb_status upload_tables(hyb_grid* g, const HostModes& h, ModeTables<T>& 
     HYB_CUDA_TRY(cudaMemcpy(t.cj, cj.data(), sizeof(T) * nk, cudaMemcpyHostToDevice));
     HYB_CUDA_TRY(cudaMemcpy(t.corr, corr.data(), sizeof(T) * nk, cudaMemcpyHostToDevice));
     HYB_CUDA_TRY(cudaMemcpy(t.filt, filt.data(), sizeof(T) * nk, cudaMemcpyHostToDevice));
-    if (!tw8.empty()) HYB_CUDA_TRY(cudaMemcpy(t.tw8, tw8.data(), sizeof(C) * tw8.size(), cudaMemcpyHostToDevice));
     HYB_CUDA_TRY(cudaMemcpy(t.twS, twS.data(), sizeof(C) * M, cudaMemcpyHostToDevice));
     return HYB_OK;
 }

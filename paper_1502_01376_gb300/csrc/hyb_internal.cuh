@@ -127,8 +127,6 @@ __device__ __forceinline__ void stockham_rows(C*& src, C*& dst, int M, int nrow,
     }
 }
 
-constexpr int kTw8 = 504;   // entries of ModeTables::tw8
-
 // x1 wavenumbers of mode kappa in FP64: k1 = 2 pi kappa / (n1 dx1); the Yee symbol
 // [k]1 = sin(k1 dx1/2)/(dx1/2); and the wavenumber the advance differentiates with
 // (Sec. 2.1: [k]1 replaced by k1; the Yee symbol itself in Yee-recovery mode; k1 plus the
@@ -178,12 +176,6 @@ __host__ __device__ inline void stockham_tw_frac(int M, int i, int* num, int* de
         lgNs += lgR;
     }
 }
-// Entry i of ModeTables::tw8 as W = exp(-2 pi i num/den)
-__host__ __device__ inline void tw8_frac(int i, int* num, int* den) {
-    if (i < 448) { *num = (i % 64) * (1 + i / 64); *den = 512; }
-    else { *num = ((i - 448) % 8) * (1 + (i - 448) / 8); *den = 64; }
-}
-
 // The twiddles of the passes stockham_rows makes for M points, in pass order: the pass with span
 // Ns and radix R holds W_{R Ns}^{r k} (r = 1..R-1, k < Ns) at Ns - 1 + (r - 1) Ns + k, so the
 // passes fill entries 0..M-2 (computed in FP64, rounded once).
@@ -193,19 +185,6 @@ inline std::vector<C> stockham_twiddles(int M) {
     for (int i = 0; i < M; i++) {
         int num, den;
         stockham_tw_frac(M, i, &num, &den);
-        const double a = -2.0 * 3.14159265358979323846 * (double)num / (double)den;
-        tw[(size_t)i] = mkc<C>((decltype(C::x))std::cos(a), (decltype(C::x))std::sin(a));
-    }
-    return tw;
-}
-
-// ModeTables::tw8 for M = 512 (computed in FP64, rounded once)
-template <typename C>
-inline std::vector<C> tw8_table() {
-    std::vector<C> tw(kTw8);
-    for (int i = 0; i < kTw8; i++) {
-        int num, den;
-        tw8_frac(i, &num, &den);
         const double a = -2.0 * 3.14159265358979323846 * (double)num / (double)den;
         tw[(size_t)i] = mkc<C>((decltype(C::x))std::cos(a), (decltype(C::x))std::sin(a));
     }
@@ -246,11 +225,7 @@ struct ModeTables {
     cplx<T>* twM = nullptr;   // W_M^j = exp(-2 pi i j / M), j < M, M = n1/2
     cplx<T>* twN = nullptr;   // W_N^k = exp(-2 pi i k / n1), k < M
     cplx<T>* sgp = nullptr;   // sigma+ (without c dt), for diagnostics
-    cplx<T>* twS = nullptr;   // stockham_twiddles(M): the shared-memory row FFTs
-    // M = 512 only (n1 = 1024, factored 8 x 8 x 8): the twiddles of the first two stages in the
-    // order the threads read them, [(k - 1) 64 + t] = W_512^{t k} (k = 1..7, t < 64), then
-    // [448 + (k - 1) 8 + t0] = W_64^{t0 k} (t0 < 8)
-    cplx<T>* tw8 = nullptr;
+    cplx<T>* twS = nullptr;   // stockham_twiddles(M): the row transforms
 };
 
 struct FusedPlan;   // defined in fused_api.cuh

@@ -33,5 +33,11 @@ cudaError_t row_reg_ampere(float2* spec, const RowPtrsW& p, int n1, int64_t rows
     HYB_ROW_LG(HYB_CALL)
 #undef HYB_CALL
 }
+cudaError_t row_reg_update(float2* spec, const RowPtrsW& EB, const RowPtrs& J, int n1, int64_t rows, int n2, int n3, bool d3, bool faraday, bool wb,
+                           const ModeTables<float>& t, float a2, float a3, cudaStream_t s) {
+#define HYB_CALL(LG) update_lg<float, LG>(spec, EB, J, rows, n2, n3, d3, faraday, wb, t, a2, a3, s)
+    HYB_ROW_LG(HYB_CALL)
+#undef HYB_CALL
+}
 
 }  // namespace hyb

@@ -13,12 +13,14 @@
 // order of the passes (8 points; W_M^j read at strides took 16 us more of the 8192 x 512 step).
 //
 // FP32 P = 8 (16 points for rows of 4096, three passes instead of four, measured the same: 94 and 93 against 88 and
-// 95 us for 8192 x 512); FP64 P = 4: an FP64 instruction occupies a quarter of an SM for about 50 cycles however many
+// 95 us for 8192 x 512, twiddles from L1); FP64 P = 4: an FP64 instruction occupies a quarter of an SM for about 50 cycles however many
 // lanes it has, so the few rows of a small grid want few instructions per warp (128 x 64: forward 10.7 -> 7, Ampere and
 // inverse 15.3 -> 9.5 us).
 #pragma once
 #include "hyb_internal.cuh"
 #include "packed_dev.cuh"
+#include "tm_dev.cuh"
+#include "tm_sched.cuh"
 
 namespace hyb {
 
@@ -41,7 +43,7 @@ template <bool INV, typename C> __device__ __forceinline__ void rdft(C (&v)[8]) 
 
 template <typename T, int LG> constexpr int pts() { return sizeof(T) == 8 ? 4 : 8; }
 
-template <typename T, int LG>
+template <typename T, int LG, bool TM = false>
 struct RowFft {
     using C = cplx<T>;
     static constexpr int P = pts<T, LG>(), LGP = P == 8 ? 3 : 2;
@@ -57,6 +59,60 @@ struct RowFft {
         return P == 8 ? tw[NS - 1 + (r - 1) * NS + k] : tw[(M / (R * NS)) * r * k];
     }
 
+    // TM: a thread's twiddles in tensor memory, words from ta on: 16 per radix-8 pass after the first (7 twiddles), 16
+    // (radix 4) or 8 (radix 2) of the last, then H of the split.  The threads of a lane quarter with the same t share them.
+    static constexpr int FULL = LG / LGP - 1, REST = LG % LGP, OFF_N = 16 * FULL + (REST == 2 ? 16 : REST == 1 ? 8 : 0);
+    static constexpr int SETS = TT > 128 ? TT / 128 : 1, COLS = 64 * SETS;
+    static_assert(!TM || (sizeof(T) == 4 && OFF_N + 2 * H <= 64), "tensor-memory twiddles");
+    uint32_t ta;
+    __device__ __forceinline__ void tm_fill(const C* __restrict__ twN) const {
+        if constexpr (TM) fill_pass<LGP>(twN);
+    }
+    template <int LGNS>
+    __device__ __forceinline__ void fill_pass(const C* __restrict__ twN) const {
+        constexpr int NS = 1 << LGNS, LEFT = LG - LGNS, OFF = 16 * (LGNS / LGP - 1);
+        float r[16];
+#pragma unroll
+        for (int i = 0; i < 16; i++) r[i] = 0.f;
+        if constexpr (LEFT >= LGP) {
+#pragma unroll
+            for (int k = 1; k < P; k++) { const C w = twiddle<P, NS>(k, t & (NS - 1)); r[2 * k - 2] = w.x; r[2 * k - 1] = w.y; }
+            tm_st16(ta + OFF, r);
+            fill_pass<LGNS + LGP>(twN);
+        } else {
+            if constexpr (LEFT > 0) {
+                constexpr int RR = 1 << LEFT, Q = P / RR;
+#pragma unroll
+                for (int m = 0; m < Q; m++)
+#pragma unroll
+                    for (int k = 1; k < RR; k++) {
+                        const C w = twiddle<RR, NS>(k, t + TT * m);
+                        r[2 * (m * (RR - 1) + k - 1)] = w.x;
+                        r[2 * (m * (RR - 1) + k - 1) + 1] = w.y;
+                    }
+                if constexpr (RR == 4) tm_st16(ta + OFF, r);
+                else { float q[8]; for (int i = 0; i < 8; i++) q[i] = r[i]; tm_st8(ta + OFF, q); }
+            }
+            float q[8];
+#pragma unroll
+            for (int i = 0; i < H; i++) { const C w = twN[t + TT * i]; q[2 * i] = w.x; q[2 * i + 1] = w.y; }
+            tm_st8(ta + OFF_N, q);
+        }
+    }
+    // the split's twiddles W_N^{t + TT i}
+    __device__ __forceinline__ void split_tw(const C* __restrict__ twN, C (&w)[H]) const {
+        if constexpr (TM) {
+            float q[8];
+            tm_ld8(ta + OFF_N, q);
+            tm_wait_ld();
+#pragma unroll
+            for (int i = 0; i < H; i++) w[i] = mkc<C>(q[2 * i], q[2 * i + 1]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < H; i++) w[i] = twN[t + TT * i];
+        }
+    }
+
     __device__ __forceinline__ void sync() const {
         if (TT <= 32) __syncwarp();
         else asm volatile("bar.sync %0, %1;" :: "r"(bar), "r"(TT) : "memory");
@@ -66,15 +122,20 @@ struct RowFft {
 
     template <bool INV, int LGNS>
     __device__ __forceinline__ void pass(C (&v)[P]) {
-        constexpr int NS = 1 << LGNS, REST = LG - LGNS;
-        if constexpr (REST >= LGP) {
+        constexpr int NS = 1 << LGNS, LEFT = LG - LGNS;
+        if constexpr (LEFT >= LGP) {
             const int k = t & (NS - 1);
-            if constexpr (LGNS > 0) {
+            if constexpr (LGNS > 0 && TM) {
+                C w[8];
+                tw_tmem(ta + 16 * (LGNS / LGP - 1), w);
+#pragma unroll
+                for (int r = 1; r < P; r++) v[r] = turn<INV>(v[r], w[r]);
+            } else if constexpr (LGNS > 0) {
 #pragma unroll
                 for (int r = 1; r < P; r++) v[r] = turn<INV>(v[r], twiddle<P, NS>(r, k));
             }
             rdft<INV>(v);
-            if constexpr (REST > LGP) {
+            if constexpr (LEFT > LGP) {
                 const int o = (t - k) * P + k;
 #pragma unroll
                 for (int r = 0; r < P; r++) a[rswz(o + r * NS)] = v[r];
@@ -84,14 +145,26 @@ struct RowFft {
                 swap();
                 pass<INV, LGNS + LGP>(v);
             }
-        } else if constexpr (REST > 0) {                // P/R butterflies of the radix R = 4 or 2 that is left: span M/R
-            constexpr int R = 1 << REST, Q = P / R;
+        } else if constexpr (LEFT > 0) {                // P/R butterflies of the radix R = 4 or 2 that is left: span M/R
+            constexpr int R = 1 << LEFT, Q = P / R;
+            float q[16];
+            if constexpr (TM && R == 4) { tm_ld16(ta + 16 * (LGNS / LGP - 1), q); tm_wait_ld(); }
+            if constexpr (TM && R == 2) {
+                float q8[8];
+                tm_ld8(ta + 16 * (LGNS / LGP - 1), q8);
+                tm_wait_ld();
+#pragma unroll
+                for (int i = 0; i < 8; i++) q[i] = q8[i];
+            }
 #pragma unroll
             for (int m = 0; m < Q; m++) {
                 C x[R];
                 x[0] = v[m];
 #pragma unroll
-                for (int r = 1; r < R; r++) x[r] = turn<INV>(v[m + Q * r], twiddle<R, NS>(r, t + TT * m));
+                for (int r = 1; r < R; r++) {
+                    const int e = 2 * (m * (R - 1) + r - 1);
+                    x[r] = turn<INV>(v[m + Q * r], TM ? mkc<C>((T)q[e], (T)q[e + 1]) : twiddle<R, NS>(r, t + TT * m));
+                }
                 if constexpr (R == 2) { const C y = x[0]; x[0] = cadd(y, x[1]); x[1] = csub(y, x[1]); }
                 else rdft<INV>(x);
 #pragma unroll
@@ -100,7 +173,9 @@ struct RowFft {
         }
     }
 
-    // v[i] = z[t + TT i] -> coefficients: put(k, X[k]) for k = 0..M
+    // A thread's coefficients: slot i < H holds k = t + TT i, slot H + i holds M - k, slot P (thread 0 only) M/2;
+    // forward() leaves them where inverse() wants them.
+    // v[i] = z[t + TT i] -> coefficients: put(slot, k, X[k]) for k = 0..M
     template <class Put>
     __device__ __forceinline__ void forward(C (&v)[P], const C* __restrict__ twN, Put put) {
         pass<false, 0>(v);
@@ -108,40 +183,55 @@ struct RowFft {
         for (int i = 0; i < H; i++) a[i * TT + t] = v[H + i];
         sync();
         // X[k] = e - u, X[M-k] = conj(e + u), e = (Z[k] + Z*[M-k])/2, u = (i/2) W_N^k (Z[k] - Z*[M-k])
-        auto pair = [&](int k, C zk, C zm, bool both) {
+        C w[H];
+        split_tw(twN, w);
+        auto pair = [&](int slot, int k, C zk, C zm, C wk, bool both) {
             const C e = mkc<C>((T)0.5 * (zk.x + zm.x), (T)0.5 * (zk.y - zm.y));
-            const C wd = rmul(twN[k], mkc<C>(zk.x - zm.x, zk.y + zm.y));
-            put(k, mkc<C>(e.x + (T)0.5 * wd.y, e.y - (T)0.5 * wd.x));
-            if (both) put(M - k, mkc<C>(e.x - (T)0.5 * wd.y, -(e.y + (T)0.5 * wd.x)));
+            const C wd = rmul(wk, mkc<C>(zk.x - zm.x, zk.y + zm.y));
+            put(slot, k, mkc<C>(e.x + (T)0.5 * wd.y, e.y - (T)0.5 * wd.x));
+            if (both) put(H + slot, M - k, mkc<C>(e.x - (T)0.5 * wd.y, -(e.y + (T)0.5 * wd.x)));
         };
 #pragma unroll
-        for (int i = 0; i < H; i++) pair(t + TT * i, v[i], i == 0 && t == 0 ? v[0] : a[(H - i) * TT - t], true);
-        if (t == 0) pair(M / 2, v[H], v[H], false);
+        for (int i = 0; i < H; i++) pair(i, t + TT * i, v[i], i == 0 && t == 0 ? v[0] : a[(H - i) * TT - t], w[i], true);
+        if (t == 0) pair(P, M / 2, v[H], v[H], twN[M / 2], false);
         swap();
     }
 
-    // X[k] = ld(k), k = 0..M (each once) -> v[i] = z[t + TT i] M (unscaled); imaginary parts of X[0], X[M] dropped
+    // each(slot, k) for this thread's coefficients
+    template <class Each>
+    __device__ __forceinline__ void modes(Each each) const {
+#pragma unroll
+        for (int i = 0; i < H; i++) {
+            each(i, t + TT * i);
+            each(H + i, M - t - TT * i);
+        }
+        if (t == 0) each(P, M / 2);
+    }
+
+    // X[k] = ld(slot, k), k = 0..M (each once) -> v[i] = z[t + TT i] M (unscaled); imaginary parts of X[0], X[M] dropped
     template <class Ld>
     __device__ __forceinline__ void inverse(C (&v)[P], const C* __restrict__ twN, Ld ld) {
         // Z[k] = E + iO, Z[M-k] = conj(E - iO), E = (X[k] + X*[M-k])/2, O = conj(W_N^k)(X[k] - X*[M-k])/2
-        auto pair = [&](int k, C xk, C xm, C& zm) {
+        C w[H];
+        split_tw(twN, w);
+        auto pair = [&](C xk, C xm, C wk, C& zm) {
             const C e = mkc<C>((T)0.5 * (xk.x + xm.x), (T)0.5 * (xk.y - xm.y));
-            const C o = rmulc(mkc<C>((T)0.5 * (xk.x - xm.x), (T)0.5 * (xk.y + xm.y)), twN[k]);
+            const C o = rmulc(mkc<C>((T)0.5 * (xk.x - xm.x), (T)0.5 * (xk.y + xm.y)), wk);
             zm = mkc<C>(e.x + o.y, o.x - e.y);
             return mkc<C>(e.x - o.y, e.y + o.x);
         };
 #pragma unroll
         for (int i = 0; i < H; i++) {
             const int k = t + TT * i;
-            C xk = ld(k), xm = ld(M - k), zm;
+            C xk = ld(i, k), xm = ld(H + i, M - k), zm;
             if (i == 0 && t == 0) { xk.y = (T)0; xm.y = (T)0; }
-            v[i] = pair(k, xk, xm, zm);
+            v[i] = pair(xk, xm, w[i], zm);
             if (i > 0 || t > 0) a[(H - i) * TT - t] = zm;
         }
         if (t == 0) {
-            const C x = ld(M / 2);
+            const C x = ld(P, M / 2);
             C zm;
-            a[0] = pair(M / 2, x, x, zm);
+            a[0] = pair(x, x, twN[M / 2], zm);
         }
         sync();
 #pragma unroll

@@ -19,6 +19,24 @@ cudaError_t row_reg_rfft(const RowPtrs& p, int nf, float2* out, int n1, int64_t 
 cudaError_t row_reg_irfft(const float2* in, const RowPtrsW& p, int nf, int n1, int64_t rows, const ModeTables<float>& t, cudaStream_t s);
 cudaError_t row_reg_ampere(float2* spec, const RowPtrsW& p, int n1, int64_t rows, int n2, int n3, bool d3, bool wb, const ModeTables<float>& t,
                            float a2, float a3, cudaStream_t s);
+// A step in FP32, by the cells of the grid (us per step of each form; the fields whose rows are transformed before the updates):
+//   all nine, then Faraday, then row_reg_ampere: up to 2^20 cells, where the three launches' own time counts and a
+//     second transform in the last one shows (8192 x 64: 31 against 33, 8192 x 128 50 against 53, 1024 x 30 10.4 against 12.4);
+//   E and B, j inside the update (row_reg_update): above (4096 x 300: 51 -> 47, 2048 x 64 x 16 89 -> 76, 8192 x 512 208 -> 172);
+//   E only, B and j inside the updates (row_reg_update, faraday): from 2^23 cells, where the nine fields and their spectra are
+//     many times the L2 and the passes over them count (30 instead of 39: 1024 x 256 x 256 2020 -> 1870, 512 x 16384 226 -> 193,
+//     4096 x 128 x 64 1198 -> 1168; but 1024 x 128 x 32 131 and 132, 2048 x 64 x 16 76 and 83), rows of 8192 points
+//     excepted (8192 x 64 x 64 1380 and 1398).
+enum class RowForm { kAll, kEB, kE };
+inline RowForm row_form(int n1, int64_t cells) {
+    if (cells <= (int64_t)1 << 20) return RowForm::kAll;
+    return cells >= (int64_t)1 << 23 && n1 < 8192 ? RowForm::kE : RowForm::kEB;
+}
+// The updates of a step with the transforms that run inside them (spec: E's spectra).  faraday: B's rows are transformed,
+// updated, stored as spectra and as rows; without it B's updated spectra are in spec and their rows are written.  Then Ampere
+// with j's transforms, and E's rows; wb: E's updated spectra are stored too.
+cudaError_t row_reg_update(float2* spec, const RowPtrsW& EB, const RowPtrs& J, int n1, int64_t rows, int n2, int n3, bool d3, bool faraday, bool wb,
+                           const ModeTables<float>& t, float a2, float a3, cudaStream_t s);
 cudaError_t row_reg_rfft(const RowPtrs& p, int nf, double2* out, int n1, int64_t rows, const ModeTables<double>& t, cudaStream_t s);
 cudaError_t row_reg_irfft(const double2* in, const RowPtrsW& p, int nf, int n1, int64_t rows, const ModeTables<double>& t, cudaStream_t s);
 cudaError_t row_reg_ampere(double2* spec, const RowPtrsW& p, int n1, int64_t rows, int n2, int n3, bool d3, bool wb, const ModeTables<double>& t,
