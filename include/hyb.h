@@ -166,13 +166,15 @@ HYB_API hyb_status hyb_push(hyb_grid* g, int32_t* cell, void* off, void* u, cons
  * allocates 3 scratch fields on the three-pass path (path 1), a second grid of
  * the same description and 9 scratch fields on the others.  2D steps of at least
  * 65536 particles list scattered particles cell by cell and visit them in that
- * order; the list (an int per particle and per cell) is allocated by the first
- * such step (not while the grid's stream is being captured: the particles are
- * then visited as stored) and freed by hyb_pic_destroy.
- * When g is k1-resident (hyb_set_resident) the step takes B^n from the
- * resident spectra instead (B^{n-1/2} + Faraday(E^n)/2 per mode, transformed
- * into scratch), and its advance transforms only j forward: 12 row transforms
- * per step instead of two full advances. */
+ * order.  The list (an int per particle and per cell) for up to 32 particles per
+ * cell and 4 M particles of grids of at most 2^20 cells comes with the scratch;
+ * a larger one is allocated by the first step that needs it (not while the
+ * grid's stream is being captured: the particles are then visited as stored).
+ * hyb_pic_destroy frees all of it.
+ * On the three-pass path, and on any path when g is k1-resident
+ * (hyb_set_resident), the step takes B^n from the spectra of E^n and B^{n-1/2}
+ * (B^{n-1/2} + Faraday(E^n)/2 per mode, transformed into scratch), and its
+ * advance transforms only j forward; k1-resident: 12 row transforms per step. */
 typedef struct hyb_pic hyb_pic;   /* opaque */
 HYB_API hyb_status hyb_pic_create(hyb_grid* g, hyb_pic** out);
 
@@ -449,9 +451,12 @@ HYB_API hyb_status hyb_mlp_gradients(hyb_mlp* m, const float* x, const float* ta
  * the loss before the step is written to loss_dev (device FP32, nullable). */
 HYB_API hyb_status hyb_mlp_train_step(hyb_mlp* m, const float* x, const float* target, int64_t B, float lr, float* loss_dev,
                                       void* stream);
-/* Kernels this network has launched so far (instrumentation: a training step
- * of L = depth + 1 layers launches 3 L (one GEMM per layer forward, two per
- * layer backward but one for the first layer, the Adam step), a forward pass L). */
+/* Kernels this network has launched so far (instrumentation).  Hidden layers
+ * wider than 64: a training step launches 3 (forward and backward of tiles of
+ * the batch through all layers, the weight gradients, the Adam step), a forward
+ * pass 1.  Narrower, with L = depth + 1 layers: a training step launches 3 L (one
+ * GEMM per layer forward, two per layer backward but one for the first layer,
+ * the Adam step), a forward pass L. */
 HYB_API int64_t hyb_mlp_launch_count(const hyb_mlp* m);
 HYB_API hyb_status hyb_mlp_destroy(hyb_mlp* m);
 

@@ -367,6 +367,8 @@ struct Order {
     int64_t cap = 0, cells = 0;
     std::vector<void*> blocks;    // allocations, the current one last
 };
+size_t order_bytes(const hyb_grid* g);               // of a list that order_place puts into the caller's memory
+void order_place(Order& o, const hyb_grid* g, void* at);
 void order_free(Order& o);
 // room for np particles of g (false: none, e.g. while a stream is captured; the particles are then visited as stored)
 bool order_reserve(Order& o, const hyb_grid* g, int64_t np);

@@ -100,6 +100,25 @@ void order_free(Order& o) {
     o = Order();
 }
 
+static void order_at(Order& o, const hyb_grid* g, int* p, int64_t n) {
+    o.ctl = reinterpret_cast<unsigned*>(p);
+    o.count = p + 4;
+    o.perm = o.count + g->cells;
+    o.cap = n;
+    o.cells = g->cells;
+}
+// A first list beside the step's scratch: 32 particles per cell, at most 16 MB (an allocation inside the first step
+// cost it 50 us, half its time on a grid of this size); none for sets that stay as stored
+static int64_t order_first(const hyb_grid* g) {
+    const int64_t n = std::min<int64_t>(32 * (int64_t)g->cells, 1 << 22);
+    return g->d.dims == 2 && g->cells <= 1 << 20 && n >= kOrderMin ? n : 0;
+}
+size_t order_bytes(const hyb_grid* g) {
+    const int64_t n = order_first(g);
+    return n ? sizeof(int) * (size_t)(4 + g->cells + n) : 0;
+}
+void order_place(Order& o, const hyb_grid* g, void* at) { order_at(o, g, reinterpret_cast<int*>(at), order_first(g)); }
+
 bool order_reserve(Order& o, const hyb_grid* g, int64_t np) {
     // 2D; small sets stay as stored (their kernels are bound by launches and latency); places are ints
     if (g->d.dims != 2 || np < kOrderMin || np > INT32_MAX || g->cells > INT32_MAX) return false;
@@ -112,11 +131,7 @@ bool order_reserve(Order& o, const hyb_grid* g, int64_t np) {
     int* p = nullptr;
     if (cudaMalloc(&p, sizeof(int) * (size_t)(4 + g->cells + n)) != cudaSuccess) { cudaGetLastError(); return false; }
     o.blocks.push_back(p);
-    o.ctl = reinterpret_cast<unsigned*>(p);
-    o.count = p + 4;
-    o.perm = o.count + g->cells;
-    o.cap = n;
-    o.cells = g->cells;
+    order_at(o, g, p, n);
     return true;
 }
 

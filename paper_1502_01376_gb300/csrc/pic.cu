@@ -125,8 +125,16 @@ hyb_status hyb_pic_create(hyb_grid* g, hyb_pic** out) {
     p->g = g;
     p->field_bytes = (size_t)g->cells * (g->d.precision == 32 ? 4 : 8);
     const bool shadow = g->path != 1;                            // the three-pass path forms B^n from its own spectra
-    cudaError_t e = cudaMalloc(&p->scratch, (shadow ? 9 : 3) * p->field_bytes);
+    const size_t fields = (shadow ? 9 : 3) * p->field_bytes;
+    size_t list = order_bytes(g);
+    cudaError_t e = cudaMalloc(&p->scratch, fields + list);
+    if (e != cudaSuccess && list) {                              // the step does without the list
+        cudaGetLastError();
+        list = 0;
+        e = cudaMalloc(&p->scratch, fields);
+    }
     if (e != cudaSuccess) { p->scratch = nullptr; hyb_pic_destroy(p); return cuda_fail(e, "cudaMalloc(pic scratch)"); }
+    if (list) order_place(p->order, g, (char*)p->scratch + fields);
     if (!shadow) {
         *out = p;
         return HYB_OK;

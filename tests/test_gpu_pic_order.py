@@ -94,3 +94,30 @@ def test_particle_sets_of_several_sizes():
         assert np.array_equal(a[0], b[0])
         for x, y in zip(a[1:], b[1:]):
             assert rel_err(x, y) < 1e-9                     # atomic sums in another order, over up to ten steps
+
+
+@pytest.mark.parametrize("n1,n2,n", [(64, 45, 66000), (64, 45, 64 * 45 * 32), (64, 45, 64 * 45 * 32 + 1), (1024, 1024, 70000), (2048, 1024, 70000)])
+def test_list_beside_the_scratch_and_beyond(n1, n2, n):
+    """Sets that fit the list made with the Pic, fill it, and outgrow it, and a grid without one: the order in which
+    shuffled particles are stored makes no difference."""
+    need_gpu()
+    hyb = hyb_module()
+    out = []
+    for shuffle in (False, True):
+        w, g, F, E, B = _setup(hyb, 64, False, n1=n1, n2=n2, ppc=1)
+        gen = torch.Generator(device="cuda").manual_seed(4)
+        cell = torch.stack([torch.randint(0, k, (n,), generator=gen, device="cuda", dtype=torch.int32) for k in (n1, n2)], 1).contiguous()
+        off = torch.rand(n, 2, generator=gen, device="cuda", dtype=torch.float64)
+        u = torch.randn(n, 3, generator=gen, device="cuda", dtype=torch.float64)
+        if not shuffle:
+            key = torch.argsort(cell[:, 1].long() * n1 + cell[:, 0], stable=True)
+            cell, off, u = [t[key].contiguous() for t in (cell, off, u)]
+        qm = torch.ones(n, device="cuda", dtype=torch.float64)
+        pic = hyb.Pic(g)
+        pic.step(cell, off, u, qm, qm * 1e-4, torch.empty_like(off), torch.empty_like(qm), order=2, nsteps=1)
+        g.check()
+        out.append([t.cpu().numpy() for t in E + B])
+        pic.close()
+        g.close()
+    for x, y in zip(*out):
+        assert rel_err(x, y) < 1e-9                         # atomic sums in another order
