@@ -676,9 +676,9 @@ def measure_resident(hyb, w, E, B, J, steps, warmup, stream, flush, fused_kms, p
            "row_transforms_per_step": {"resident": "3 forward (j) + 6 inverse (E, B)",
                                        "fused_single_pass": "8 forward + 5 inverse (E1..3, B2, B3, j1..3; B1 "
                                                             "in real space)"},
-           "algorithmic_bytes_per_cell": {"resident_three_pass": 156, "fused_single_pass": BYTES_PER_CELL_STEP},
+           "algorithmic_bytes_per_cell": {"resident_three_pass": 108, "fused_single_pass": BYTES_PER_CELL_STEP},
            "fused_kernel_ms": fused_kms,
-           "achieved_gbs": 156 * w.cells / (ms / 1e3) / 1e9}
+           "achieved_gbs": 108 * w.cells / (ms / 1e3) / 1e9}
     out["frac"] = out["achieved_gbs"] / peak
     g.close()
     return out
