@@ -19,18 +19,19 @@ cudaError_t row_reg_rfft(const RowPtrs& p, int nf, float2* out, int n1, int64_t 
 cudaError_t row_reg_irfft(const float2* in, const RowPtrsW& p, int nf, int n1, int64_t rows, const ModeTables<float>& t, cudaStream_t s);
 cudaError_t row_reg_ampere(float2* spec, const RowPtrsW& p, int n1, int64_t rows, int n2, int n3, bool d3, bool wb, const ModeTables<float>& t,
                            float a2, float a3, cudaStream_t s);
-// A step in FP32, by the cells of the grid (us per step of each form; the fields whose rows are transformed before the updates):
-//   all nine, then Faraday, then row_reg_ampere: up to 2^20 cells, where the three launches' own time counts and a
-//     second transform in the last one shows (8192 x 64: 31 against 33, 8192 x 128 50 against 53, 1024 x 30 10.4 against 12.4);
-//   E and B, j inside the update (row_reg_update): above (4096 x 300: 51 -> 47, 2048 x 64 x 16 89 -> 76, 8192 x 512 208 -> 172);
-//   E only, B and j inside the updates (row_reg_update, faraday): from 2^23 cells, where the nine fields and their spectra are
-//     many times the L2 and the passes over them count (30 instead of 39: 1024 x 256 x 256 2020 -> 1870, 512 x 16384 226 -> 193,
-//     4096 x 128 x 64 1198 -> 1168; but 1024 x 128 x 32 131 and 132, 2048 x 64 x 16 76 and 83), rows of 8192 points
-//     excepted (8192 x 64 x 64 1380 and 1398).
+// A step in FP32, by the cells of the grid (us per step; the fields whose rows are transformed before the updates):
+//   all nine, then Faraday, then row_reg_ampere: small grids, where the three launches' own time counts and a second
+//     transform in the last one shows (8192 x 64 29 against 31, 8192 x 128 45 against 47, 1024 x 300 17 against 18.5);
+//   E and B, j inside the update (row_reg_update): 4096 x 1024 140 -> 130, 8192 x 512 157 -> 152, 4096 x 64 x 16 149 -> 141;
+//   E only, B and j inside the updates (row_reg_update, faraday): rows of up to 1024 points, whose transforms are short
+//     against the passes they save (1024 x 777 29 -> 25, 512 x 4000 58 -> 51, 1024 x 128 x 32 117 -> 113), and any rows of
+//     grids many times the L2 (1024 x 256 x 256 1832 -> 1625, 2048 x 64 x 64 259 -> 240, 8192 x 64 x 64 1218 -> 1193;
+//     but 8192 x 512 152 and 162, 2048 x 64 x 16 72 and 75).
 enum class RowForm { kAll, kEB, kE };
 inline RowForm row_form(int n1, int64_t cells) {
+    if (n1 <= 1024) return cells < (int64_t)1 << 19 ? RowForm::kAll : RowForm::kE;
     if (cells <= (int64_t)1 << 20) return RowForm::kAll;
-    return cells >= (int64_t)1 << 23 && n1 < 8192 ? RowForm::kE : RowForm::kEB;
+    return cells >= (int64_t)1 << 23 ? RowForm::kE : RowForm::kEB;
 }
 // The updates of a step with the transforms that run inside them (spec: E's spectra).  faraday: B's rows are transformed,
 // updated, stored as spectra and as rows; without it B's updated spectra are in spec and their rows are written.  Then Ampere

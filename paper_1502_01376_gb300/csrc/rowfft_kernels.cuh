@@ -383,16 +383,20 @@ static int threads_for(int64_t total_rows) {
 }
 template <typename T, int LG>
 static size_t smem_for(int threads) { return sizeof(cplx<T>) * 2 * RowFft<T, LG>::M * (size_t)(threads / RowFft<T, LG>::TT); }
-static cudaError_t room(const void* kern, size_t smem_max) {
+// shared memory for the kernel's largest block, and a carveout that holds `blocks` of them and leaves the rest to L1: rows
+// of spectra and the mode tables are read from it (with all of it as shared memory the 1024 x 256 x 256 step took 1896 us
+// instead of 1666, 8192 x 512 170 instead of 160)
+static cudaError_t room(const void* kern, size_t smem_max, int blocks) {
+    const int percent = std::min<int>(100, (int)(100 * blocks * (smem_max + 1024) / (228 * 1024)) + 1);
     cudaError_t e = func_attr_once(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-    return e == cudaSuccess ? func_attr_once(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) : e;
+    return e == cudaSuccess ? func_attr_once(kern, cudaFuncAttributePreferredSharedMemoryCarveout, percent) : e;
 }
 
 template <typename T, int LG>
 static cudaError_t rfft_lg(const RowPtrs& p, int nf, cplx<T>* out, int64_t rows, const ModeTables<T>& t, cudaStream_t s) {
     if (!RowFft<T, LG>::table(t) || !t.twN) return cudaErrorInvalidValue;
     const int64_t total = rows * nf;
-    cudaError_t e = room((const void*)k_rfft_reg<T, LG, false>, smem_for<T, LG>((row_threads<T, LG>())));
+    cudaError_t e = room((const void*)k_rfft_reg<T, LG, false>, smem_for<T, LG>((row_threads<T, LG>())), row_blocks<T, LG>());
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4) {
         constexpr int th = row_threads<T, LG>(), R = th / RowFft<T, LG>::TT;
@@ -400,7 +404,7 @@ static cudaError_t rfft_lg(const RowPtrs& p, int nf, cplx<T>* out, int64_t rows,
         const int resident = resident_grid((const void*)k_rfft_reg<T, LG, false>, th, smem);     // of the same launch bounds
         if (total >= (int64_t)kTmRounds * R * resident) {
             const auto kern = k_rfft_reg<T, LG, true>;
-            e = room((const void*)kern, smem);
+            e = room((const void*)kern, smem, row_blocks<T, LG>());
             if (e != cudaSuccess) return e;
             kern<<<resident, th, smem, s>>>(p, out, (unsigned)rows, (unsigned)total, RowFft<T, LG>::table(t), t.twN);
             return cudaGetLastError();
@@ -417,7 +421,7 @@ template <typename T, int LG>
 static cudaError_t irfft_lg(const cplx<T>* in, const RowPtrsW& p, int nf, int64_t rows, const ModeTables<T>& t, cudaStream_t s) {
     if (!RowFft<T, LG>::table(t) || !t.twN) return cudaErrorInvalidValue;
     const auto kern = k_irfft_reg<T, LG>;
-    cudaError_t e = room((const void*)kern, smem_for<T, LG>((row_threads<T, LG>())));
+    cudaError_t e = room((const void*)kern, smem_for<T, LG>((row_threads<T, LG>())), row_blocks<T, LG>());
     if (e != cudaSuccess) return e;
     const int th = threads_for<T, LG>(rows * nf), R = th / RowFft<T, LG>::TT;
     kern<<<dim3((unsigned)((rows + R - 1) / R), nf), th, smem_for<T, LG>(th), s>>>(in, p, (unsigned)rows, RowFft<T, LG>::table(t), t.twN);
@@ -429,7 +433,7 @@ static cudaError_t ampere_lg(cplx<T>* spec, const RowPtrsW& p, int64_t rows, int
     if (!RowFft<T, LG>::table(t) || !t.twN || !t.S || !t.cj1 || !t.cj) return cudaErrorInvalidValue;
     const auto kern = d3 ? (wb ? k_ampere_irfft_reg<T, LG, true, true> : k_ampere_irfft_reg<T, LG, true, false>)
                          : (wb ? k_ampere_irfft_reg<T, LG, false, true> : k_ampere_irfft_reg<T, LG, false, false>);
-    cudaError_t e = room((const void*)kern, smem_for<T, LG>((row_threads<T, LG>())));
+    cudaError_t e = room((const void*)kern, smem_for<T, LG>((row_threads<T, LG>())), row_blocks<T, LG>());
     if (e != cudaSuccess) return e;
     const int th = threads_for<T, LG>(rows * 6), R = th / RowFft<T, LG>::TT;
     kern<<<(unsigned)((rows + R - 1) / R * 6), th, smem_for<T, LG>(th), s>>>(spec, p, (unsigned)rows, n2, n3, RowFft<T, LG>::table(t), t.twN, t.S, t.cj1, t.cj,
@@ -446,7 +450,7 @@ static cudaError_t update_lg(cplx<T>* spec, const RowPtrsW& EB, const RowPtrs& J
     const unsigned nfl = faraday ? 3u : 6u;
     const size_t full = smem_for<T, LG>(most);
     const auto any = (const void*)k_ampere_reg<T, LG, true, true, false>;                        // the launch bounds of all
-    cudaError_t e = room(any, full);
+    cudaError_t e = room(any, full, upd_blocks<T, LG>());
     if (e != cudaSuccess) return e;
     const unsigned resident = (unsigned)resident_grid(any, most, full) / 6u * 6u;
     const bool tm = resident && (rows * TT + most - 1) / most * nfl >= (int64_t)kTmRounds * resident;
@@ -459,7 +463,7 @@ static cudaError_t update_lg(cplx<T>* spec, const RowPtrsW& EB, const RowPtrs& J
         for (int c = 0; c < 3; c++) B.p[c] = EB.p[3 + c];
         const auto kern = d3 ? (tm ? k_faraday_reg<T, LG, true, true> : k_faraday_reg<T, LG, true, false>)
                              : (tm ? k_faraday_reg<T, LG, false, true> : k_faraday_reg<T, LG, false, false>);
-        e = room((const void*)kern, full);
+        e = room((const void*)kern, full, upd_blocks<T, LG>());
         if (e != cudaSuccess) return e;
         kern<<<blocks, th, smem, s>>>(spec, B, (unsigned)rows, n2, n3, tw, t.twN, t.S, a2, a3);
         e = cudaGetLastError();
@@ -469,7 +473,7 @@ static cudaError_t update_lg(cplx<T>* spec, const RowPtrsW& EB, const RowPtrs& J
                                : (tm ? k_ampere_reg<T, LG, true, false, true> : k_ampere_reg<T, LG, true, false, false>))
                          : (wb ? (tm ? k_ampere_reg<T, LG, false, true, true> : k_ampere_reg<T, LG, false, true, false>)
                                : (tm ? k_ampere_reg<T, LG, false, false, true> : k_ampere_reg<T, LG, false, false, false>));
-    e = room((const void*)kern, full);
+    e = room((const void*)kern, full, upd_blocks<T, LG>());
     if (e != cudaSuccess) return e;
     kern<<<blocks, th, smem, s>>>(spec, J, EB, (unsigned)rows, n2, n3, tw, t.twN, t.S, t.cj1, t.cj, a2, a3, nfl);
     return cudaGetLastError();

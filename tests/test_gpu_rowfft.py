@@ -1,6 +1,5 @@
 """The register-resident row transforms through the advance: every row length they take, 2D and 3D, row counts that
-fill no block, from two rows, both sides of the FP64 size rule, the three FP32 forms of a step (up to 2^20 cells, above,
-from 2^23), k1-resident and not, against the oracle (the
+fill no block, from two rows, both sides of the FP64 size rule, the three FP32 forms of a step (by row length and cells), k1-resident and not, against the oracle (the
 tolerances of the other parity tests)."""
 import numpy as np
 import pytest
@@ -19,7 +18,8 @@ pytestmark = pytest.mark.gpu
                                            (64, 256, 257, 1), (64, 128, 6, 3), (64, 512, 7, 1),
                                            (32, 1024, 5, 1), (32, 1024, 4, 3), (32, 128, 16411, 1), (32, 256, 111, 75), (32, 512, 4099, 1),
                                            (32, 1024, 2053, 1), (32, 1024, 29, 67), (32, 2048, 1031, 1), (32, 4096, 523, 1), (32, 8192, 311, 1),
-                                           (32, 128, 257, 257), (32, 1024, 8209, 1), (32, 4096, 67, 31)])
+                                           (32, 128, 257, 257), (32, 1024, 8209, 1), (32, 4096, 67, 31),
+                                           (32, 1024, 511, 1), (32, 1024, 513, 1), (32, 8192, 1031, 1)])
 def test_row_transforms_in_the_advance(prec, n1, n2, n3, resident, orc):
     need_gpu()
     hyb = hyb_module()
