@@ -103,23 +103,26 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
     {
         const int64_t i = blockIdx.x * (int64_t)kPushThreads + threadIdx.x;
         if (i < np) {
-            np_at = visit_at(perm, i);
-            ncc = reinterpret_cast<const int2*>(cell)[np_at];
-            noo = reinterpret_cast<const V2*>(off)[np_at];
+            const int64_t a = VISIT ? visit_at(perm, i) : i;
+            if (VISIT) np_at = a;
+            ncc = reinterpret_cast<const int2*>(cell)[a];
+            noo = reinterpret_cast<const V2*>(off)[a];
         }
     }
     for (int64_t base = blockIdx.x * (int64_t)kPushThreads; base < np; base += stride) {
-        const int64_t p = np_at;
+        const int64_t p = VISIT ? np_at : base + threadIdx.x;
         const bool live = base + threadIdx.x < np;
         const int2 cc = ncc;
         const V2 oo = noo;
         if (base + threadIdx.x + stride < np) {
-            np_at = visit_at(perm, base + threadIdx.x + stride);
-            ncc = reinterpret_cast<const int2*>(cell)[np_at];
-            noo = reinterpret_cast<const V2*>(off)[np_at];
+            const int64_t i = base + threadIdx.x + stride, a = VISIT ? visit_at(perm, i) : i;
+            if (VISIT) np_at = a;
+            ncc = reinterpret_cast<const int2*>(cell)[a];
+            noo = reinterpret_cast<const V2*>(off)[a];
         }
         // asked for before the tile is staged, used after it
-        T uu[3] = {(T)0, (T)0, (T)0}, qmp = (T)0;
+        T uu[3], qmp;
+        if (sizeof(T) == 4) uu[0] = uu[1] = uu[2] = qmp = (T)0;
         if (sizeof(T) == 4 && live) {        // (FP64 has no registers to hold them)
             uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2];
             qmp = qm[p];
@@ -157,10 +160,7 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
         }
         __syncthreads();
         if (ok) {
-            if (sizeof(T) == 8) {
-                uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2];
-                qmp = qm[p];
-            }
+            if (sizeof(T) == 8) { uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2]; }
             // weights for the integer (0) and half (1) positions along each axis
             T wx[2][L + 1], wy[2][L + 1];
             const int ix0 = pweights<L>(ox, wx[0]), ix1 = pweights<L>(ox - (T)0.5, wx[1]);
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
                 }
             }
             const T Ev[3] = {e1, e2, e3}, Bv[3] = {b1, b2, b3};
-            boris(uu, Ev, Bv, hdt * qmp);
+            boris(uu, Ev, Bv, hdt * (sizeof(T) == 4 ? qmp : qm[p]));
             const T gi = prsqrt((T)1 + uu[0] * uu[0] + uu[1] * uu[1] + uu[2] * uu[2]);
             reinterpret_cast<int2*>(cell)[p] = make_int2(cx, cy);
             V2 on;
