@@ -61,7 +61,7 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
                            int64_t np, int order) {
     hyb_grid* g = p->g;
     Visit visit;
-    if (order_reserve(p->order, g, np)) {
+    if (order_reserve(p->order, g, np, order)) {
         hyb_status st = order_particles<T>(p->order, g, cell, off, np, &visit);
         if (st != HYB_OK) return st;
     }

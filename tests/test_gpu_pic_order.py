@@ -121,3 +121,28 @@ def test_list_beside_the_scratch_and_beyond(n1, n2, n):
         g.close()
     for x, y in zip(*out):
         assert rel_err(x, y) < 1e-9                         # atomic sums in another order
+
+
+@pytest.mark.parametrize("prec,order,ppc", [(64, 2, 23), (32, 2, 23), (64, 3, 18), (32, 3, 18), (32, 1, 46)])
+def test_listed_particles_from_the_rule_on(prec, order, ppc, orc):
+    """Shuffled particles, just enough of them to be listed at each shape order, on one step against the oracle's composition."""
+    need_gpu()
+    hyb = hyb_module()
+    w, g, F, E, B = _setup(hyb, prec, False, ppc=ppc)
+    p = wl.pic_plasma_torch(w, "cuda")
+    assert p[4].numel() >= {1: 1 << 18, 2: 1 << 17, 3: 3 << 15}[order]
+    mix = torch.randperm(p[4].numel(), generator=torch.Generator().manual_seed(3)).cuda()
+    cell, off, u, qm, q = p = [t[mix].contiguous() for t in p]
+    a = [t.cpu().numpy() for t in p]
+    pic = hyb.Pic(g)
+    pic.step(cell, off, u, qm, q, torch.empty_like(off), torch.empty_like(qm), order=order, nsteps=1)
+    g.check()
+    go = orc.grid(n1=w.n1, n2=w.n2, dx1=w.dx1, dx2=w.dx2, dt=w.dt, filt_kc=w.filt_kc, filt_w=w.filt_w)
+    Eo, Bo, co, oo, uo = _oracle_pic(orc, go, F[0], F[1], a[0], a[1].astype(np.float64), *[x.astype(np.float64) for x in a[2:]], order, w.dt,
+                                     np.array([w.dx1, w.dx2]), 1)
+    tol = 1e-12 if prec == 64 else 1e-5
+    for x, y in zip(E + B, Eo + Bo):
+        assert rel_err(x.cpu().numpy(), y) < tol
+    assert np.array_equal(cell.cpu().numpy(), co)
+    pic.close()
+    g.close()
