@@ -293,7 +293,7 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
                     atomicOr(flag, 1);
                     continue;
                 }
-                const float c1 = c1s * qp, c2 = c2s * qp, c3 = c3s * qp * vp;
+                const float c1 = c1s * qp, c2 = c2s * qp, c3 = v3 ? c3s * qp * vp : 0.f;    // (no v3: no j3, also of an infinite charge)
                 const float lx = o0.x < o1.x ? o0.x : o1.x, ly = o0.y < o1.y ? o0.y : o1.y;
                 // the first of the particle's own WN points, from the window's first
                 const int ox = (int)floorf(lx - 0.5f * (float)(ORDER + 1)) + 1 - B0, oy = (int)floorf(ly - 0.5f * (float)(ORDER + 1)) + 1 - B0;
