@@ -33,7 +33,7 @@ struct hyb_pic {
     cudaStream_t cs = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaGraphExec_t exec = nullptr;
-    const void* key[12] = {};
+    const void* key[16] = {};
     int64_t key_np = -1;
     int key_order = 0, key_path = 0;
     bool key_res = false;
@@ -191,9 +191,10 @@ hyb_status hyb_pic_step(hyb_pic* p, int32_t* cell, void* off, void* u, const voi
     }
     hyb_status st = step();
     if (st != HYB_OK) return st;
-    const void* key[12] = {cell, off, u, qm, q, off_new, v3, g->E[0], g->E[1], g->E[2], g->B[0], g->J[0]};
+    // every array that the captured launches hold
+    const void* key[16] = {cell, off, u, qm, q, off_new, v3, g->E[0], g->E[1], g->E[2], g->B[0], g->B[1], g->B[2], g->J[0], g->J[1], g->J[2]};
     bool same = p->exec && np == p->key_np && shape_order == p->key_order && g->path == p->key_path && g->resident == p->key_res;
-    for (int i = 0; i < 12 && same; i++) same = key[i] == p->key[i];
+    for (int i = 0; i < 16 && same; i++) same = key[i] == p->key[i];
     if (!p->cs) {
         HYB_CUDA_TRY(cudaStreamCreateWithFlags(&p->cs, cudaStreamNonBlocking));
         HYB_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
@@ -225,7 +226,7 @@ hyb_status hyb_pic_step(hyb_pic* p, int32_t* cell, void* off, void* u, const voi
             }
             return HYB_OK;
         }
-        for (int i = 0; i < 12; i++) p->key[i] = key[i];
+        for (int i = 0; i < 16; i++) p->key[i] = key[i];
         p->key_np = np;
         p->key_order = shape_order;
         p->key_path = g->path;
