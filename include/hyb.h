@@ -183,7 +183,8 @@ HYB_API hyb_status hyb_pic_create(hyb_grid* g, hyb_pic** out);
  * [np][dims], off [np][dims] (x^n on entry, x^{n+nsteps} on exit, in [-1, 2)
  * of its cell), u [np][3], qm [np] (q/m), q [np] (macro-particle charge),
  * off_new [np][dims] (scratch, ends equal to off), v3 [np] (scratch; required
- * in 2D).  Errors of the push and deposit are flagged as for them (hyb_check).
+ * in 2D).  2D: cell, off and off_new aligned to one particle's pair, else
+ * HYB_EALIGN.  Errors of the push and deposit are flagged as for them (hyb_check).
  * With nsteps >= 4 (and unless g's fused kernel exchanges halo rows inside
  * the launch, as at n1 = 4096, or the grid's stream is being captured by the
  * caller) the first step runs as plain

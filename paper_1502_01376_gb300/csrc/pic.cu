@@ -169,6 +169,11 @@ hyb_status hyb_pic_step(hyb_pic* p, int32_t* cell, void* off, void* u, const voi
     }
     if (!p->g->bound) { set_error("hyb_pic_step: fields not bound"); return HYB_ESTATE; }
     hyb_grid* g = p->g;
+    const size_t pair = g->d.precision == 32 ? 8 : 16;               // as in hyb_push, whose kernel reads pairs at once
+    if (np > 0 && g->d.dims == 2 && ((uintptr_t)cell % 8 || (uintptr_t)off % pair || (uintptr_t)off_new % pair)) {
+        set_error("hyb_pic_step: 2D cell (8 bytes) and off, off_new (2 reals) must be aligned to one particle's pair");
+        return HYB_EALIGN;
+    }
     auto step = [&]() {
         return g->d.precision == 32
             ? pic_step<float>(p, cell, (float*)off, (float*)u, (const float*)qm, (const float*)q, (float*)off_new, (float*)v3, np, shape_order)

@@ -53,3 +53,34 @@ def test_replayed_step_follows_a_rebind(path, swap):
     b, _ = _run(hyb, path, swap, True)
     for x, y in zip(a, b):
         assert rel_err(x, y) < 1e-4                          # FP32, atomic sums in another order, twelve steps
+
+
+@pytest.mark.parametrize("prec", [32, 64])
+@pytest.mark.parametrize("which", ["cell", "off", "off_new"])
+@pytest.mark.parametrize("nsteps", [1, 6])
+def test_particle_pairs_must_be_aligned(prec, which, nsteps):
+    """2D arrays that start in the middle of a particle's pair are refused on the host, as hyb_push refuses them,
+    and nothing is touched."""
+    need_gpu()
+    hyb = hyb_module()
+    dt = torch.float64 if prec == 64 else torch.float32
+    n = 100
+    g = hyb.Grid(hyb.make_desc(dims=2, n1=32, n2=16, dx1=0.2, dx2=0.2, dt=0.08, precision=prec, filt_kc=0.0, filt_w=0.0))
+    F = [[torch.zeros((16, 32), device="cuda", dtype=dt) for _ in range(3)] for _ in range(3)]
+    g.bind(*F)
+    pic = hyb.Pic(g)
+
+    def pairs(name, fill, t):
+        flat = torch.full((2 * n + 1,), fill, device="cuda", dtype=t)
+        return (flat[1:] if name == which else flat[:-1]).view(n, 2)
+    cell, off, new = pairs("cell", 3, torch.int32), pairs("off", 0.25, dt), pairs("off_new", 9.0, dt)
+    u = torch.ones((n, 3), device="cuda", dtype=dt)
+    one, v3 = torch.ones(n, device="cuda", dtype=dt), torch.empty(n, device="cuda", dtype=dt)
+    with pytest.raises(hyb.HybError) as e:
+        pic.step(cell, off, u, one, one, new, v3, order=2, nsteps=nsteps)
+    assert e.value.status == hyb.HYB_EALIGN
+    torch.cuda.synchronize()
+    assert bool((cell == 3).all() and (off == 0.25).all() and (new == 9.0).all() and (u == 1).all())
+    assert all(bool((t == 0).all()) for f in F for t in f)
+    pic.close()
+    g.close()
