@@ -277,8 +277,9 @@ HYB_API hyb_status hyb_check(hyb_grid* g);
  * single-launch batched step (a role of two CTAs, one of which never arrives).
  * The limit is `seconds` at the device's clock rate.  Returns HYB_ETIMEOUT
  * when the wait gave up as designed (the expected result), HYB_OK if the
- * condition was met, HYB_EINVAL for which not in {0, 1, 2} or seconds not in
- * (0, 10], HYB_ECUDA on a CUDA error.  Synchronous on `stream`; allocates and
+ * condition was met, HYB_ESTATE if the drain after the mbarrier wait (which =
+ * 1: of what is in flight when a wait gave up) missed its phase, HYB_EINVAL for
+ * which not in {0, 1, 2} or seconds not in (0, 10], HYB_ECUDA on a CUDA error.  Synchronous on `stream`; allocates and
  * frees three ints of device memory. */
 HYB_API hyb_status hyb_wait_selftest(int which, double seconds, void* stream);
 

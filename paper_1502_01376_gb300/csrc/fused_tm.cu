@@ -13,7 +13,8 @@ __global__ void __launch_bounds__(tmk::NT, 1) k_fused_tm(FusedBatch fb) {
 
 // ------------------------------------------------------------------ self-test of the bounded waits
 // which = 0: the release/acquire flag wait of the halo exchange, on a flag nothing sets;
-// which = 1: the mbarrier wait of the row staging, on a phase nothing completes.
+// which = 1: the mbarrier wait of the row staging, on a phase nothing completes; then the drain after it, on the same
+// phase, which is completed first (the drain must not take the phase before for it: bit 2 of *err).
 // Both must give up after `limit` cycles and report through *err.
 __global__ void k_wait_probe(const int* flag, int* err, long long limit, int which) {
     __shared__ uint64_t bar;
@@ -25,7 +26,12 @@ __global__ void k_wait_probe(const int* flag, int* err, long long limit, int whi
         mbar_init(smem_addr(&bar), 1);
         mbar_fence_init();
         abort_flag = 0;
-        mbar_wait(smem_addr(&bar), 0, err, &abort_flag, limit);
+        uint32_t ph = 0;
+        mbar_wait_next(smem_addr(&bar), ph, err, &abort_flag, limit);
+        if (mbar_try_wait(smem_addr(&bar), ph)) atomicOr(err, 4);        // nothing has completed yet
+        mbar_expect_tx(smem_addr(&bar), 0);                              // the late arrival
+        mbar_drain(smem_addr(&bar), ph);
+        if (!mbar_try_wait(smem_addr(&bar), ph)) atomicOr(err, 4);
     }
 }
 

@@ -464,6 +464,7 @@ hyb_status hyb_wait_selftest(int which, double seconds, void* stream) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFree(d);
     if (e != cudaSuccess) return cuda_fail(e, "hyb_wait_selftest");
+    if (h & 4) { set_error("the drain after a wait that gave up missed its phase"); return HYB_ESTATE; }
     if (h & 2) { set_error("a bounded device-side wait gave up"); return HYB_ETIMEOUT; }
     return HYB_OK;
 }

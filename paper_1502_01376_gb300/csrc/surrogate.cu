@@ -535,8 +535,7 @@ __global__ void __launch_bounds__(CT, 1) k_mlp_chain(__grid_constant__ const Cha
         }
     };
     auto wait_product = [&]() {
-        mbar_wait(mb, mph, g.err, &s_abort);
-        mph ^= 1;
+        mbar_wait_next(mb, mph, g.err, &s_abort);
         tm_fence_after();
     };
     auto abort_now = [&]() {                            // the same answer in every thread

@@ -86,19 +86,28 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // bounded wait for phase `parity` of an mbarrier; on time-out sets bit 1 of *err
-// and the CTA's abort flag (later waits then return at once)
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int* err, volatile int* abort_flag,
+// and the CTA's abort flag (later waits then return at once).  False if it gave up.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err, volatile int* abort_flag,
                                           long long limit = kWaitCycles) {
-    if (mbar_try_wait(bar, parity)) return;
+    if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
-        if (*abort_flag) return;
+        if (*abort_flag) return false;
         if (clock64() - t0 > limit) {
             if (err) atomicOr(err, 2);
             *abort_flag = 1;
-            return;
+            return false;
         }
     }
+    return true;
+}
+// the same for the phase that ph counts.  ph goes on to the next phase only after a wait that succeeded: after one
+// that gave up, mbar_drain(bar, ph) still waits for what is in flight
+__device__ __forceinline__ bool mbar_wait_next(uint32_t bar, uint32_t& ph, int* err, volatile int* abort_flag,
+                                               long long limit = kWaitCycles) {
+    const bool done = mbar_wait(bar, ph, err, abort_flag, limit);
+    if (done) ph ^= 1u;
+    return done;
 }
 
 // ------------------------------------------------------------------ tcgen05.mma (kind::f16, BF16 in, FP32 out)
