@@ -449,9 +449,15 @@ template <int ORDER>
 static cudaError_t launch_runs(hyb_grid* g, float* J1, float* J2, float* J3, const int32_t* cell, const float* off_old,
                                const float* off_new, const float* v3, const float* q, int64_t np, float c1, float c2, float c3, const Visit& visit) {
     const auto kern = visit.perm ? k_deposit2d_runs<ORDER, true> : k_deposit2d_runs<ORDER, false>;
-    // a contiguous range of particles per warp, four waves of resident blocks
-    const int64_t warps = (int64_t)resident_grid((const void*)kern, 32 * kRunWarps, 0) * kRunWarps * 4;
-    const int64_t per = std::max<int64_t>(32, ((np + warps - 1) / warps + 255) / 256 * 256);
+    // A contiguous range of particles per warp: 256 or a multiple of it, four waves of resident blocks.  A call that would leave
+    // resident warps idle that way (up to 160 particles for each of them) spreads over all of them, down to 32 particles a
+    // warp, but no further than to some 16 cells' worth, which still make runs.  8192 particles of a 256 x 256 grid, order 1, 2,
+    // 3: 12, 12, 12 us; 256 to a warp, one after another, 27, 41, 51 us; one thread per particle 19, 23, 25.  With 192 to a
+    // warp already (400000 particles) ranges of 256 are faster again, 35 against 37 us.
+    const int64_t warps = (int64_t)resident_grid((const void*)kern, 32 * kRunWarps, 0) * kRunWarps;
+    const int64_t even = (np + warps - 1) / warps;
+    int64_t per = ((np + 4 * warps - 1) / (4 * warps) + 255) / 256 * 256;
+    if (even <= 160) per = std::min<int64_t>(256, (std::max<int64_t>(even, 16 * np / g->cells) + 31) / 32 * 32);
     const unsigned blocks = (unsigned)((np + per * kRunWarps - 1) / (per * kRunWarps));
     kern<<<blocks, 32 * kRunWarps, 0, g->stream>>>(J1, J2, J3, g->d.n1, g->d.n2, reinterpret_cast<const int2*>(cell),
                                                    reinterpret_cast<const float2*>(off_old),
