@@ -212,20 +212,27 @@ __device__ __noinline__ void deposit_alone(float* J1, float* J2, float* J3, int 
 
 constexpr int kRunWarps = 4, kRunScan = 512;      // warps per block; particles looked at for 32 runs
 constexpr int kRunMax = 32;                       // a longer run is cut (at multiples of this many particles)
+// Particles taken one by one where there are no runs.  32 at a time, with 64 cells looked at before each, 2 M shuffled particles
+// (1024 x 512, order 2) took 388 us; 361 now, 335 with a thread per particle and no runs looked for.
+constexpr int kAlone = 256;
+
+// warps below `full` take `per` particles each, the others `fine`
+struct RunSplit { int64_t per, full, fine; };
 
 template <int ORDER, bool VISIT>
 __global__ void __launch_bounds__(32 * kRunWarps, ORDER == 3 ? 3 : 4)
 k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restrict__ J3, int n1, int n2,
                  const int2* __restrict__ cell, const float2* __restrict__ off0, const float2* __restrict__ off1,
-                 const float* __restrict__ v3, const float* __restrict__ q, int64_t np, int64_t per_warp, float c1s, float c2s,
+                 const float* __restrict__ v3, const float* __restrict__ q, int64_t np, const __grid_constant__ RunSplit split, float c1s, float c2s,
                  float c3s, int* __restrict__ flag, Visit visit) {
     constexpr int WN = ORDER + 2, N = ORDER + 3, B0 = ORDER == 3 ? -2 : -1;
     __shared__ int s_start[kRunWarps][64];       // at most 32 + 32 heads
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* const start = s_start[warp];
     const int* const perm = VISIT ? visit_perm(visit) : nullptr;
-    const int64_t first = ((int64_t)blockIdx.x * kRunWarps + warp) * per_warp;
-    const int64_t last = first + per_warp < np ? first + per_warp : np;
+    const int64_t w = (int64_t)blockIdx.x * kRunWarps + warp, mine = w < split.full ? split.per : split.fine;
+    const int64_t first = w < split.full ? w * split.per : split.full * split.per + (w - split.full) * split.fine;
+    const int64_t last = first + mine < np ? first + mine : np;
     int64_t base = first;
     while (base < last) {
         // ---- the next runs: places (from base) where the cell changes or a multiple of kRunMax begins
@@ -367,8 +374,10 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
                 }
             }
         } else {
-            // ---- scattered: a particle per lane
+            // ---- scattered: a particle per lane, kAlone of them before looking for runs again (asking for the next particle's
+            // data ahead was worth 2 % of this, and its registers cost the runs as much)
             if (end > 32) end &= ~31;                                // whole warps; the rest in the next round
+            end = max(end, (int)min((int64_t)kAlone, last - base));
             for (int i = lane; i < end; i += 32) {
                 const int64_t p = visit_at(perm, base + i);
                 const int2 pc = cell[p];
@@ -451,17 +460,30 @@ static cudaError_t launch_runs(hyb_grid* g, float* J1, float* J2, float* J3, con
     const auto kern = visit.perm ? k_deposit2d_runs<ORDER, true> : k_deposit2d_runs<ORDER, false>;
     // A contiguous range of particles per warp: 256 or a multiple of it, four waves of resident blocks.  A call that would leave
     // resident warps idle that way (up to 160 particles for each of them) spreads over all of them, down to 32 particles a
-    // warp, but no further than to some 16 cells' worth, which still make runs.  8192 particles of a 256 x 256 grid, order 1, 2,
-    // 3: 12, 12, 12 us; 256 to a warp, one after another, 27, 41, 51 us; one thread per particle 19, 23, 25.  With 192 to a
-    // warp already (400000 particles) ranges of 256 are faster again, 35 against 37 us.
+    // warp; over a quarter of them where that leaves a warp some 16 cells' worth, which still makes runs.  8192 particles of a
+    // 256 x 256 grid, order 1, 2, 3: 12, 12, 12 us; 256 to a warp, one after another, 27, 41, 51 us; one thread per particle 19,
+    // 23, 25.  With 192 to a warp already (400000 particles) ranges of 256 are faster again, 35 against 37 us.
     const int64_t warps = (int64_t)resident_grid((const void*)kern, 32 * kRunWarps, 0) * kRunWarps;
     const int64_t even = (np + warps - 1) / warps;
     int64_t per = ((np + 4 * warps - 1) / (4 * warps) + 255) / 256 * 256;
-    if (even <= 160) per = std::min<int64_t>(256, (std::max<int64_t>(even, 16 * np / g->cells) + 31) / 32 * 32);
-    const unsigned blocks = (unsigned)((np + per * kRunWarps - 1) / (per * kRunWarps));
+    if (even <= 160) per = std::min<int64_t>(256, (std::max(even, std::min<int64_t>(16 * np / g->cells, 4 * even)) + 31) / 32 * 32);
+    // Up to 1.4 waves of 256: one wave of longer ranges (the second would be nearly empty; order 3, 614400 particles of a 1024 x
+    // 300 grid, in cell order 74 -> 58 us, shuffled 222 -> 184).  Ranges longer than 256: half a wave's worth at the end in
+    // halves, so that the last wave ends evenly (2 M, 1024 x 512, order 3, in cell order 193 -> 172 us, shuffled 696 -> 555; 4 M,
+    // order 2, 216 -> 208 and 691 -> 685), as long as those hold 16 cells' worth: ranges of 256 in halves make too few runs of 16
+    // particles per cell (31 -> 39 us), ranges of 512 of 38 (256 x 256, order 2, 2.5 M, 101 -> 111).
+    else if (even > 256 && 10 * np <= 14 * 256 * warps) per = (even + 31) / 32 * 32;
+    RunSplit split{per, (np + per - 1) / per, per};
+    int64_t all = split.full;
+    if (per > 256 && 10 * np > 14 * 256 * warps) {
+        split.fine = std::min(per, std::max<int64_t>({256, per / 2, 16 * np / g->cells}));
+        split.full = (np - std::min(np / 2, warps * per / 2)) / per;
+        all = split.full + (np - split.full * per + split.fine - 1) / split.fine;
+    }
+    const unsigned blocks = (unsigned)((all + kRunWarps - 1) / kRunWarps);
     kern<<<blocks, 32 * kRunWarps, 0, g->stream>>>(J1, J2, J3, g->d.n1, g->d.n2, reinterpret_cast<const int2*>(cell),
                                                    reinterpret_cast<const float2*>(off_old),
-                                                   reinterpret_cast<const float2*>(off_new), v3, q, np, per, c1, c2, c3, g->dflag, visit);
+                                                   reinterpret_cast<const float2*>(off_new), v3, q, np, split, c1, c2, c3, g->dflag, visit);
     return cudaGetLastError();
 }
 
