@@ -99,12 +99,12 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
     int2 ncc = make_int2(0, 0);
     V2 noo;
     noo.x = noo.y = (T)0;
-    int64_t np_at = 0;
+    int np_at = 0;                            // (a list holds ints)
     {
         const int64_t i = blockIdx.x * (int64_t)kPushThreads + threadIdx.x;
         if (i < np) {
             const int64_t a = VISIT ? visit_at(perm, i) : i;
-            if (VISIT) np_at = a;
+            if (VISIT) np_at = (int)a;
             ncc = reinterpret_cast<const int2*>(cell)[a];
             noo = reinterpret_cast<const V2*>(off)[a];
         }
@@ -116,14 +116,17 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
         const V2 oo = noo;
         if (base + threadIdx.x + stride < np) {
             const int64_t i = base + threadIdx.x + stride, a = VISIT ? visit_at(perm, i) : i;
-            if (VISIT) np_at = a;
+            if (VISIT) np_at = (int)a;
             ncc = reinterpret_cast<const int2*>(cell)[a];
             noo = reinterpret_cast<const V2*>(off)[a];
         }
-        // asked for before the tile is staged, used after it
+        // asked for before the tile is staged, used after it, where there are registers to hold them: not in FP64, nor at
+        // order 3 (8192 particles 10.4 us with them, 8.6 without; 16 M in cell order 493 and 473; at orders 1 and 2 16 M
+        // take 363 and 378 us with them, 397 and 419 without)
+        constexpr bool kEarly = sizeof(T) == 4 && L < 3;
         T uu[3], qmp;
-        if (sizeof(T) == 4) uu[0] = uu[1] = uu[2] = qmp = (T)0;
-        if (sizeof(T) == 4 && live) {        // (FP64 has no registers to hold them)
+        if (kEarly) uu[0] = uu[1] = uu[2] = qmp = (T)0;
+        if (kEarly && live) {
             uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2];
             qmp = qm[p];
         }
@@ -160,7 +163,7 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
         }
         __syncthreads();
         if (ok) {
-            if (sizeof(T) == 8) { uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2]; }
+            if (!kEarly) { uu[0] = u[3 * p]; uu[1] = u[3 * p + 1]; uu[2] = u[3 * p + 2]; }
             // weights for the integer (0) and half (1) positions along each axis
             T wx[2][L + 1], wy[2][L + 1];
             const int ix0 = pweights<L>(ox, wx[0]), ix1 = pweights<L>(ox - (T)0.5, wx[1]);
@@ -206,7 +209,7 @@ __global__ void __launch_bounds__(kPushThreads, 3) k_push2d(PushFields F, int n1
                 }
             }
             const T Ev[3] = {e1, e2, e3}, Bv[3] = {b1, b2, b3};
-            boris(uu, Ev, Bv, hdt * (sizeof(T) == 4 ? qmp : qm[p]));
+            boris(uu, Ev, Bv, hdt * (kEarly ? qmp : qm[p]));
             const T gi = prsqrt((T)1 + uu[0] * uu[0] + uu[1] * uu[1] + uu[2] * uu[2]);
             reinterpret_cast<int2*>(cell)[p] = make_int2(cx, cy);
             V2 on;
