@@ -517,7 +517,7 @@ hyb_status deposit(hyb_grid* g, const int32_t* cell, const T* off_old, const T* 
         int threads = kDepThreads;
         while (threads > 32 && np < (int64_t)threads * dev_sms) threads >>= 1;
         const unsigned blocks = (unsigned)std::min<int64_t>((np + threads - 1) / threads, (int64_t)dev_sms * 32);
-#define HYB_DEP2(O) (visit.perm ? k_deposit2d<T, O, true> : k_deposit2d<T, O, false>)<<<blocks, threads, 0, g->stream>>>(J1, J2, J3, d.n1, d.n2, cell, off_old, off_new, v3, q, np, c1, c2, c3, g->dflag, visit)
+#define HYB_DEP2(O) (visit.perm ? k_deposit2d<T, O, sizeof(T) == 4> : k_deposit2d<T, O, false>)<<<blocks, threads, 0, g->stream>>>(J1, J2, J3, d.n1, d.n2, cell, off_old, off_new, v3, q, np, c1, c2, c3, g->dflag, visit)
         if (order == 1) HYB_DEP2(1); else if (order == 2) HYB_DEP2(2); else HYB_DEP2(3);
 #undef HYB_DEP2
     } else {

@@ -372,7 +372,7 @@ void order_place(Order& o, const hyb_grid* g, void* at);
 void order_free(Order& o);
 // room for np particles of g (false: none, e.g. while a stream is captured; the particles are then visited as stored)
 bool order_reserve(Order& o, const hyb_grid* g, int64_t np, int shape);
-template <typename T> hyb_status order_particles(Order& o, hyb_grid* g, const int32_t* cell, const T* off, int64_t np, Visit* v);
+hyb_status order_particles(Order& o, hyb_grid* g, const int32_t* cell, const float* off, int64_t np, Visit* v);
 
 // deposit (deposit.cu)
 template <typename T>

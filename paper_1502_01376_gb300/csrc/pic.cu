@@ -20,6 +20,8 @@
 // transformed back into scratch arrays, and step 4 transforms only j forward, so a
 // step takes 12 row transforms (3 for B^n, 3 for j, 6 for E, B).
 // Scattered particles (2D) are visited cell by cell in steps 2 and 3 (order.cu).
+#include <type_traits>
+
 #include "hyb_internal.cuh"
 
 struct hyb_pic {
@@ -61,9 +63,11 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
                            int64_t np, int order) {
     hyb_grid* g = p->g;
     Visit visit;
-    if (order_reserve(p->order, g, np, order)) {
-        hyb_status st = order_particles<T>(p->order, g, cell, off, np, &visit);
-        if (st != HYB_OK) return st;
+    if constexpr (std::is_same<T, float>::value) {
+        if (order_reserve(p->order, g, np, order)) {
+            hyb_status st = order_particles(p->order, g, cell, off, np, &visit);
+            if (st != HYB_OK) return st;
+        }
     }
     if (g->resident || !p->shadow) {
         void* Bh[3];

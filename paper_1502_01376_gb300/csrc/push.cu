@@ -308,7 +308,7 @@ hyb_status push_fields(hyb_grid* g, void* const E[3], void* const B[3], int32_t*
     const T hdt = (T)(0.5 * d.dt);
     const T s1 = (T)(d.dt / d.dx1), s2 = (T)(d.dt / d.dx2), s3 = (T)(d.dt / d.dx3);
     if (d.dims == 2) {
-#define HYB_PUSH2(O) (visit.perm ? k_push2d<T, O, true> : k_push2d<T, O, false>)<<<blocks, threads, 0, g->stream>>>(F, d.n1, d.n2, cell, off, u, qm, off_new, v3, np, hdt, s1, s2, g->dflag, visit)
+#define HYB_PUSH2(O) (visit.perm ? k_push2d<T, O, sizeof(T) == 4> : k_push2d<T, O, false>)<<<blocks, threads, 0, g->stream>>>(F, d.n1, d.n2, cell, off, u, qm, off_new, v3, np, hdt, s1, s2, g->dflag, visit)
         if (order == 1) HYB_PUSH2(1); else if (order == 2) HYB_PUSH2(2); else HYB_PUSH2(3);
 #undef HYB_PUSH2
     } else {

@@ -1,0 +1,62 @@
+"""When a PIC step lists its particles cell by cell: what that may cost a step, and the steps that do it."""
+import numpy as np
+import pytest
+
+from gpu_util import hyb_module, need_gpu, torch
+
+pytestmark = pytest.mark.gpu
+
+FROM = {1: 1 << 19, 2: 1 << 17, 3: 3 << 15}              # particles from which FP32 2D sets are listed, by shape order
+
+
+def _set(n, n1, n2, dt, ordered, seed=7, u_th=1e-4, drift=50.0):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    cell = torch.stack([torch.randint(0, k, (n,), generator=gen, device="cuda", dtype=torch.int32) for k in (n1, n2)], 1)
+    if ordered:
+        cell = cell[torch.argsort(cell[:, 1].long() * n1 + cell[:, 0], stable=True)]
+    off = torch.rand((n, 2), generator=gen, device="cuda", dtype=dt) * 0.999
+    u = torch.randn((n, 3), generator=gen, device="cuda", dtype=dt) * u_th
+    u[:, 0] += drift
+    q = torch.where(torch.arange(n, device="cuda") % 2 == 0, 1.0, -1.0).to(dt)
+    return cell.contiguous(), off, u, q.clone(), q * 1e-4
+
+
+def _grid(hyb, n1, n2, prec, resident=True):
+    dt = torch.float64 if prec == 64 else torch.float32
+    g = hyb.Grid(hyb.make_desc(dims=2, n1=n1, n2=n2, dx1=0.2, dx2=0.2, dt=0.08, precision=prec, filt_kc=0.5, filt_w=0.2))
+    F = [[torch.zeros((n2, n1), device="cuda", dtype=dt) for _ in range(3)] for _ in range(3)]
+    g.bind(*F)
+    if resident:
+        g.set_resident(True)
+    return g, F, dt
+
+
+def _step_us(hyb, n, prec, order, ordered, n1=256, n2=256):
+    g, _, dt = _grid(hyb, n1, n2, prec)
+    p = _set(n, n1, n2, dt, ordered)
+    new, v3 = torch.empty_like(p[1]), torch.empty_like(p[3])
+    pic = hyb.Pic(g)
+    pic.step(*p, new, v3, order=order, nsteps=8)
+    best = 1e9
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        pic.step(*p, new, v3, order=order, nsteps=16)
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / 16)
+    g.check()
+    pic.close()
+    g.close()
+    return best
+
+
+@pytest.mark.parametrize("order", [2, 3])
+def test_double_precision_steps_are_not_listed_at_a_loss(order):
+    """Shuffled FP64 particles: a step of 2 % more of them, past any number from which they might be listed, takes no
+    more than 2 % (and 3 % of noise) longer; listing them cost 5 to 10 %."""
+    need_gpu()
+    hyb = hyb_module()
+    n = {2: 130900, 3: 98200}[order]
+    a, b = (_step_us(hyb, k, 64, order, False, 512, 256) for k in (n, n * 102 // 100))
+    assert b < 1.05 * a, (a, b)
