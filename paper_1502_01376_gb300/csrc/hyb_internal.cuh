@@ -362,9 +362,13 @@ __device__ __forceinline__ bool renormalise(int& c, T& o, int n) {
 // cell order of scattered particles (order.cu): perm[0 .. np) lists the particles cell by cell
 struct Order {
     int* perm = nullptr;          // [cap]
-    int* count = nullptr;         // [cells]: particles of a cell, then its next place in the list
+    int* count = nullptr;         // [cells]: particles of a cell; zero between steps
+    int* next = nullptr;          // [cells]: a cell's next place in the list
     unsigned* ctl = nullptr;      // jumps, cursor
     int64_t cap = 0, cells = 0;
+    bool off = false;             // no list: count may not be zero
+    cudaStream_t side = nullptr;  // the list is made beside the grid's stream: from fork to join
+    cudaEvent_t fork = nullptr, join = nullptr;
     std::vector<void*> blocks;    // allocations, the current one last
 };
 size_t order_bytes(const hyb_grid* g);               // of a list that order_place puts into the caller's memory
@@ -372,7 +376,9 @@ void order_place(Order& o, const hyb_grid* g, void* at);
 void order_free(Order& o);
 // room for np particles of g (false: none, e.g. while a stream is captured; the particles are then visited as stored)
 bool order_reserve(Order& o, const hyb_grid* g, int64_t np, int shape);
+// starts the list of what is on g's stream; order_wait before the first kernel that visits by it, or changes cell or off
 hyb_status order_particles(Order& o, hyb_grid* g, const int32_t* cell, const float* off, int64_t np, Visit* v);
+hyb_status order_wait(const Order& o, hyb_grid* g, const Visit& v);
 
 // deposit (deposit.cu)
 template <typename T>

@@ -63,6 +63,15 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
                            int64_t np, int order) {
     hyb_grid* g = p->g;
     Visit visit;
+    // the grid's stream goes on after the list whatever happens to the step: its kernels read cell and off
+    struct Joined {
+        const Order& o;
+        hyb_grid* g;
+        const Visit& v;
+        bool pending = true;
+        hyb_status wait() { pending = false; return order_wait(o, g, v); }
+        ~Joined() { if (pending) order_wait(o, g, v); }
+    } list{p->order, g, visit};
     if constexpr (std::is_same<T, float>::value) {
         if (order_reserve(p->order, g, np, order)) {
             hyb_status st = order_particles(p->order, g, cell, off, np, &visit);
@@ -75,6 +84,7 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
         hyb_status st = HYB_OK;
         if (!g->resident || g->res_stale) st = generic_resident_import<T>(g);  // E^n, B^{n-1/2} spectra
         if (st == HYB_OK) st = generic_b_half<T>(g, Bh);                        // B^n
+        if (st == HYB_OK) st = list.wait();
         if (st == HYB_OK) st = push_fields<T>(g, g->E, Bh, cell, off, u, qm, off_new, v3, np, order, visit);
         if (st == HYB_OK) st = deposit<T>(g, cell, off, off_new, v3, q, np, order, visit);
         if (st == HYB_OK) st = g->resident ? hyb_advance(g, 1) : generic_advance<T>(g, 1, true);   // j forward only
@@ -103,6 +113,8 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
                                                         (const T*)g->B[1], (const T*)g->B[2], g->cells);
         HYB_CUDA_TRY(cudaGetLastError());
     }
+    st = list.wait();
+    if (st != HYB_OK) return st;
     st = push_fields<T>(g, g->E, Bs, cell, off, u, qm, off_new, v3, np, order, visit);   // u^{n+1/2}, x^{n+1}
     if (st != HYB_OK) return st;
     st = deposit<T>(g, cell, off, off_new, v3, q, np, order, visit);  // j^{n+1/2}
