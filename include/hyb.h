@@ -197,6 +197,12 @@ HYB_API hyb_status hyb_pic_create(hyb_grid* g, hyb_pic** out);
 HYB_API hyb_status hyb_pic_step(hyb_pic* p, int32_t* cell, void* off, void* u, const void* qm, const void* q,
                                 void* off_new, void* v3, int64_t np, int shape_order, int nsteps);
 
+/* How the last step visited its particles (instrumentation): *listed is 1 if cell
+ * by cell, 0 if as stored because they were found in order, -1 if as stored
+ * without a look (too few, not FP32, not 2D, no room for a list).  Waits for the
+ * grid's stream. */
+HYB_API hyb_status hyb_pic_listed(hyb_pic* p, int* listed);
+
 /* Frees the PIC step's second grid, scratch and list (not g). */
 HYB_API hyb_status hyb_pic_destroy(hyb_pic* p);
 

@@ -379,6 +379,7 @@ bool order_reserve(Order& o, const hyb_grid* g, int64_t np, int shape);
 // starts the list of what is on g's stream; order_wait before the first kernel that visits by it, or changes cell or off
 hyb_status order_particles(Order& o, hyb_grid* g, const int32_t* cell, const float* off, int64_t np, Visit* v);
 hyb_status order_wait(const Order& o, hyb_grid* g, const Visit& v);
+hyb_status order_listed(const Order& o, const hyb_grid* g, int* listed);   // what the last one on g's stream decided
 
 // deposit (deposit.cu)
 template <typename T>

@@ -176,6 +176,14 @@ hyb_status order_particles(Order& o, hyb_grid* g, const int32_t* cell, const flo
     return HYB_OK;
 }
 
+hyb_status order_listed(const Order& o, const hyb_grid* g, int* listed) {
+    unsigned jumps = 0;
+    HYB_CUDA_TRY(cudaMemcpyAsync(&jumps, o.ctl, sizeof(jumps), cudaMemcpyDeviceToHost, g->stream));
+    HYB_CUDA_TRY(cudaStreamSynchronize(g->stream));
+    *listed = jumps > (unsigned)kSamplePairs / 2;
+    return HYB_OK;
+}
+
 hyb_status order_wait(const Order& o, hyb_grid* g, const Visit& v) {
     if (v.perm) HYB_CUDA_TRY(cudaStreamWaitEvent(g->stream, o.join, 0));
     return HYB_OK;

@@ -30,6 +30,7 @@ struct hyb_pic {
     void* scratch = nullptr;      // with a shadow grid E'[3], B'[3], J'[3] = 0; else B'[3]
     size_t field_bytes = 0;
     hyb::Order order;             // cell order of scattered particles
+    bool looked = false;          // the last step asked whether its particles are scattered
     // one step captured as a CUDA graph, replayed for the later steps of a call (and of later calls
     // with the same arguments): its own stream, fork/join events, and the arguments it was taken with
     cudaStream_t cs = nullptr;
@@ -78,6 +79,7 @@ static hyb_status pic_step(hyb_pic* p, int32_t* cell, T* off, T* u, const T* qm,
             if (st != HYB_OK) return st;
         }
     }
+    p->looked = visit.perm != nullptr;
     if (g->resident || !p->shadow) {
         void* Bh[3];
         for (int c = 0; c < 3; c++) Bh[c] = (char*)p->scratch + (size_t)((p->shadow ? 3 : 0) + c) * p->field_bytes;
@@ -257,6 +259,12 @@ hyb_status hyb_pic_step(hyb_pic* p, int32_t* cell, void* off, void* u, const voi
     HYB_CUDA_TRY(cudaEventRecord(p->ev_join, p->cs));
     HYB_CUDA_TRY(cudaStreamWaitEvent(orig, p->ev_join, 0));
     return HYB_OK;
+}
+
+hyb_status hyb_pic_listed(hyb_pic* p, int* listed) {
+    if (!p || !listed) { set_error("hyb_pic_listed: null argument"); return HYB_EINVAL; }
+    *listed = -1;
+    return p->looked ? order_listed(p->order, p->g, listed) : HYB_OK;
 }
 
 hyb_status hyb_pic_destroy(hyb_pic* p) {

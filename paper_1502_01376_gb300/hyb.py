@@ -131,6 +131,8 @@ def lib():
             L.hyb_pic_create.restype = S
             L.hyb_pic_step.argtypes = [_V, _V, _V, _V, _V, _V, _V, _V, ctypes.c_int64, ctypes.c_int, ctypes.c_int]
             L.hyb_pic_step.restype = S
+            L.hyb_pic_listed.argtypes = [_V, ctypes.POINTER(ctypes.c_int)]
+            L.hyb_pic_listed.restype = S
             L.hyb_pic_destroy.argtypes = [_V]
             L.hyb_pic_destroy.restype = S
             L.hyb_mlp_create.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, _V, ctypes.POINTER(_V)]
@@ -500,6 +502,12 @@ class Pic:
     def step(self, cell, off, u, qm, q, off_new, v3, order=2, nsteps=1):
         _check(lib().hyb_pic_step(_V(self.h), _V(_ptr(cell)), _V(_ptr(off)), _V(_ptr(u)), _V(_ptr(qm)), _V(_ptr(q)),
                                   _V(_ptr(off_new)), _V(_ptr(v3)), qm.numel(), order, nsteps))
+
+    def listed(self) -> int:
+        """How the last step visited its particles (hyb_pic_listed): 1 cell by cell, 0 in order, -1 not looked at."""
+        r = ctypes.c_int()
+        _check(lib().hyb_pic_listed(_V(self.h), ctypes.byref(r)))
+        return r.value
 
     def close(self):
         if self.h:
