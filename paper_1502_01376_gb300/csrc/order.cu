@@ -123,10 +123,11 @@ static bool order_clear(Order& o) {
     return false;
 }
 // A first list beside the step's scratch: 32 particles per cell, at most 16 MB (an allocation inside the first step
-// cost it 50 us, half its time on a grid of this size); none for sets that stay as stored
+// cost it 50 us, half its time on a grid of this size); none where such sets stay as stored at every
+// shape order
 static int64_t order_first(const hyb_grid* g) {
     const int64_t n = std::min<int64_t>(32 * (int64_t)g->cells, 1 << 22);
-    return g->d.dims == 2 && g->d.precision == 32 && g->cells <= 1 << 20 && n >= order_min(2) ? n : 0;
+    return g->d.dims == 2 && g->d.precision == 32 && g->cells <= 1 << 20 && n >= order_min(3) ? n : 0;
 }
 size_t order_bytes(const hyb_grid* g) {
     const int64_t n = order_first(g);

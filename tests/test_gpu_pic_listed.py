@@ -171,3 +171,27 @@ def test_a_step_captured_by_the_caller():
     assert _same_places(out[0], out[1], 64, 80)
     for x, y in zip(out[0][2:], out[1][2:]):
         assert rel_err(x, y) < 1e-4
+
+
+@pytest.mark.parametrize("n1,n2", [(64, 56), (32, 96)])
+def test_a_captured_first_step_is_listed_on_small_grids(n1, n2):
+    """The list for up to 32 particles per cell comes with the Pic: a first step that the caller captures, when nothing
+    can be allocated, lists order-3 sets from 98304 particles on, on grids from 3072 cells on."""
+    need_gpu()
+    hyb = hyb_module()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        w, g, F, E, B = _setup(hyb, 32, False, n1=n1, n2=n2, ppc=1)
+        p = _random_set(98304, n1, n2, torch.Generator(device="cuda").manual_seed(4))
+        new, v3 = torch.empty_like(p[1]), torch.empty_like(p[3])
+        pic = hyb.Pic(g)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            pic.step(*p, new, v3, order=3, nsteps=1)
+        graph.replay()
+        assert pic.listed() == 1
+        g.check()
+        del graph
+        pic.close()
+        g.close()
