@@ -586,7 +586,10 @@ static hyb_status nci_launch(const double* samples, int64_t n, int order, int co
     if (n == 0) return HYB_OK;
     const int64_t total = n * n_alias;
     // 32 pairs per warp where that still gives every SM eight warps, fewer on small calls
-    const int64_t spread = total / (152 * 8);
+    int dev = 0, sms = 0;
+    HYB_CUDA_TRY(cudaGetDevice(&dev));
+    HYB_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int64_t spread = total / ((int64_t)sms * 8);
     const int group = spread >= 32 ? 32 : spread < 1 ? 1 : (int)spread;
     const int64_t per_block = (int64_t)group * (kNciThreads / 32);
     k_nci<<<(unsigned)((total + per_block - 1) / per_block), kNciThreads, 0, (cudaStream_t)stream>>>(
