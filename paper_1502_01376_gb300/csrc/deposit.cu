@@ -471,11 +471,12 @@ static cudaError_t launch_runs(hyb_grid* g, float* J1, float* J2, float* J3, con
     // 300 grid, in cell order 74 -> 58 us, shuffled 222 -> 184).  Ranges longer than 256: half a wave's worth at the end in
     // halves, so that the last wave ends evenly (2 M, 1024 x 512, order 3, in cell order 193 -> 172 us, shuffled 696 -> 555; 4 M,
     // order 2, 216 -> 208 and 691 -> 685), as long as those hold 16 cells' worth: ranges of 256 in halves make too few runs of 16
-    // particles per cell (31 -> 39 us), ranges of 512 of 38 (256 x 256, order 2, 2.5 M, 101 -> 111).
+    // particles per cell (31 -> 39 us), ranges of 512 of 38 (256 x 256, order 2, 2.5 M, 101 -> 111).  Beyond 4096 the last wave
+    // is short against the rest (67 M: 1543 us whole, 1550 with halves).
     else if (even > 256 && 10 * np <= 14 * 256 * warps) per = (even + 31) / 32 * 32;
     RunSplit split{per, (np + per - 1) / per, per};
     int64_t all = split.full;
-    if (per > 256 && 10 * np > 14 * 256 * warps) {
+    if (per > 256 && per <= 4096 && 10 * np > 14 * 256 * warps) {
         split.fine = std::min(per, std::max<int64_t>({256, per / 2, 16 * np / g->cells}));
         split.full = (np - std::min(np / 2, warps * per / 2)) / per;
         all = split.full + (np - split.full * per + split.fine - 1) / split.fine;
