@@ -164,14 +164,15 @@ HYB_API hyb_status hyb_push(hyb_grid* g, int32_t* cell, void* off, void* u, cons
  *   hyb_advance (E^{n+1}, B^{n+1/2});  off <- off_new.
  * hyb_pic_create borrows g (which must stay bound to the same arrays) and
  * allocates 3 scratch fields on the three-pass path (path 1), a second grid of
- * the same description and 9 scratch fields on the others.  FP32 2D steps of at least
- * 98304 particles (shape order 3; 131072 at order 2, 524288 at order 1) list
- * scattered particles cell by cell (on a private stream ordered after and
- * before the grid's stream) and visit them in that order.  The list (an
- * int per particle and two per cell) for up to 32 particles per
- * cell and 4 M particles of grids of at most 2^20 cells comes with the scratch;
- * a larger one is allocated by the first step that needs it (not while the
- * grid's stream is being captured: the particles are then visited as stored).
+ * the same description and 9 scratch fields on the others.  FP32 2D steps of
+ * 131072 to 6 M particles (shape order 2; from 98304 on at order 3; 524288 to
+ * 2 M, at least three per cell, at order 1; M = 2^20) list scattered particles
+ * cell by cell (on a private stream ordered after and before the grid's stream)
+ * and visit them in that order.  The list (an int per particle and two per cell)
+ * for up to 32 particles per cell and 4 M particles of grids of at most 2^20
+ * cells comes with the scratch; a larger one is allocated by the first step that
+ * needs it (not while the grid's stream is being captured: the particles are
+ * then visited as stored).
  * hyb_pic_destroy frees all of it.
  * On the three-pass path, and on any path when g is k1-resident
  * (hyb_set_resident), the step takes B^n from the spectra of E^n and B^{n-1/2}

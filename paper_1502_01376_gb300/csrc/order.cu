@@ -24,6 +24,15 @@ constexpr int kOrderThreads = 512;
 //   order 3: shuffled 100 K 86 and 64, 270 K 189 and 102, 1 M 584 and 226; in order 100 K 43 and 52.
 // (At orders 2 and 3 shuffled sets of 60 K gain a little already, those in order lose a fifth.)
 static int64_t order_min(int shape) { return shape == 1 ? 1 << 19 : shape == 2 ? 1 << 17 : 3 << 15; }
+// and up to which.  Sets beyond the L2 (some 3 M particles) come from memory a sector at a time when listed, 0.3 ns a
+// particle and step whatever the order; as stored they take 0.16, 0.32 and 0.5 ns at orders 1, 2 and 3.  Shuffled, 256 x 256, us as
+// stored and listed: order 1 2 M 350 and 337, 4 M 671 and 896, 8 M 1303 and 2430; order 2 6 M 2065 and 1792, 16 M 5126 and 5790;
+// order 3 16 M 8800 and 5944.  At order 1 fewer than three particles per cell do not pay either (1024 x 1000: 1 M 290 and 301, 2 M
+// 449 and 480).
+static int64_t order_max(int shape) { return shape == 1 ? 1 << 21 : shape == 2 ? 6 << 20 : INT32_MAX; }
+static bool order_pays(const hyb_grid* g, int64_t np, int shape) {
+    return np >= order_min(shape) && np <= order_max(shape) && (shape > 1 || np >= 3 * g->cells);
+}
 constexpr int kSamplePairs = kOrderThreads;         // a pair per thread
 constexpr int kScanCells = 4;                       // cells per thread of k_ranges
 
@@ -140,7 +149,7 @@ void order_place(Order& o, const hyb_grid* g, void* at) {
 
 bool order_reserve(Order& o, const hyb_grid* g, int64_t np, int shape) {
     // 2D, FP32; small sets stay as stored (their kernels are bound by launches and latency); places are ints
-    if (o.off || g->d.dims != 2 || g->d.precision != 32 || np < order_min(shape) || np > INT32_MAX || g->cells > INT32_MAX) return false;
+    if (o.off || g->d.dims != 2 || g->d.precision != 32 || !order_pays(g, np, shape) || g->cells > INT32_MAX) return false;
     if (np <= o.cap && g->cells == o.cells) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(g->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) { cudaGetLastError(); return false; }

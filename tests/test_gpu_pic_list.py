@@ -73,3 +73,36 @@ def test_particles_in_order_pay_little_for_the_decision(order):
     hyb = hyb_module()
     a, b = (_step_us(hyb, n, 32, order, True, nsteps=1) for n in (FROM[order] - 256, FROM[order]))
     assert b - a < 15.5, (a, b)
+
+
+def test_sets_beyond_the_cache_are_not_listed_at_a_loss():
+    """Order 1, shuffled: twice the particles take at most 2.3 times as long, whether their arrays fit the L2 or not
+    (listed beyond it, 2.7 times)."""
+    need_gpu()
+    hyb = hyb_module()
+    a, b = (_step_us(hyb, n, 32, 1, False) for n in ((1 << 21) - 8, 1 << 22))
+    assert b < 2.3 * a, (a, b)
+
+
+@pytest.mark.parametrize("order,n,n1,n2,listed", [(1, 1 << 21, 256, 256, 1), (1, (1 << 21) + 1, 256, 256, -1), (2, 6 << 20, 256, 256, 1),
+                                                  (2, (6 << 20) + 1, 256, 256, -1), (3, (6 << 20) + 1, 256, 256, 1),
+                                                  (1, 3 << 18, 512, 512, 1), (1, (3 << 18) - 1, 512, 512, -1), (2, 3 << 17, 512, 512, 1)])
+def test_which_sets_are_listed(order, n, n1, n2, listed):
+    """The rule at its edges, on shuffled particles; the total current is that of the particles either way."""
+    need_gpu()
+    hyb = hyb_module()
+    g, F, dt = _grid(hyb, n1, n2, 32, resident=False)
+    p = _set(n, n1, n2, dt, False, u_th=0.5, drift=0.0)
+    new, v3 = torch.empty_like(p[1]), torch.empty_like(p[3])
+    pic = hyb.Pic(g)
+    x0 = p[0].double() + p[1].double()
+    pic.step(*p, new, v3, order=order, nsteps=1)
+    assert pic.listed() == listed
+    g.check()
+    dx = (p[0].double() + p[1].double() - x0 + 128) % 256 - 128 if n1 == 256 else (p[0].double() + p[1].double() - x0 + 256) % 512 - 256
+    want = (p[4].double()[:, None] * dx).sum(0) / 0.08 * 0.2 / 0.04                # sum of q v over the cell area
+    scale = (p[4].double().abs()[:, None] * dx.abs()).sum(0) / 0.08 * 0.2 / 0.04
+    for c in range(2):
+        assert abs(float(F[2][c].double().sum() - want[c])) < 1e-4 * float(scale[c]), (c, float(F[2][c].double().sum()), float(want[c]))
+    pic.close()
+    g.close()
