@@ -300,14 +300,14 @@ k_deposit2d_runs(float* __restrict__ J1, float* __restrict__ J2, float* __restri
                     atomicOr(flag, 1);
                     continue;
                 }
-                const float c1 = c1s * qp, c2 = c2s * qp, c3 = v3 ? c3s * qp * vp : 0.f;    // (no v3: no j3, also of an infinite charge)
+                const float c1 = c1s * qp, c2 = c2s * qp, c3 = c3s * qp * vp;
                 const float lx = o0.x < o1.x ? o0.x : o1.x, ly = o0.y < o1.y ? o0.y : o1.y;
                 // the first of the particle's own WN points, from the window's first
                 const int ox = (int)floorf(lx - 0.5f * (float)(ORDER + 1)) + 1 - B0, oy = (int)floorf(ly - 0.5f * (float)(ORDER + 1)) + 1 - B0;
                 // an order-2 particle that moves back by more than half a cell leaves the window, and 0 times a
-                // non-finite charge would spread over it: such a particle on its own
+                // non-finite charge would spread over it: such a particle on its own (without v3 it has no j3, infinite or not)
                 if (ox < 0 || oy < 0 || !(isfinite(c1) && isfinite(c2) && isfinite(c3))) {
-                    deposit_alone<ORDER>(J1, J2, J3, n1, n2, cc, o0, o1, c1, c2, c3);
+                    deposit_alone<ORDER>(J1, J2, J3, n1, n2, cc, o0, o1, c1, c2, v3 ? c3 : 0.f);
                     continue;
                 }
                 float Sx0[N], Sx1[N], Sy0[N], Sy1[N], p1[N], sx[N];
