@@ -373,14 +373,19 @@ __global__ void __launch_bounds__((row_threads<T, LG>()), (upd_blocks<T, LG>()))
 // two on it is not slower (step of 8192 x 32 22.7 and 22.6 us, 128 x 4000 26.7 and 26.4, 256 x 4000 40 and 37, 128 x
 // 30000 163 and 137); a single round would fill it for one row
 constexpr int kTmRounds = 2;
-// threads of a block: the largest, fewer while that leaves under about four blocks per SM
+// threads of a block: the largest, fewer while that leaves under `blocks` of them: about four per SM
+constexpr int kRowBlocks = 600;
 template <typename T, int LG>
-static int threads_for(int64_t total_rows) {
+static int threads_for(int64_t total_rows, int blocks = kRowBlocks) {
     constexpr int TT = RowFft<T, LG>::TT;
     int th = row_threads<T, LG>();
-    while (th > std::max(TT, 32) && total_rows < (int64_t)(th / TT) * 600) th >>= 1;
+    while (th > std::max(TT, 32) && total_rows < (int64_t)(th / TT) * blocks) th >>= 1;
     return th;
 }
+// of a step's forward transforms and Ampere with E's inverse (rows of all their fields): two per SM for FP32 rows of 1024
+// points (steps of 1024 x 128 12.3 us instead of 14.4, 1024 x 260 14.4 instead of 16.4), four for others (two: 512 x 1100 22.5 us
+// instead of 20.6, FP64 128 x 400 26.7 instead of 24.8)
+template <typename T, int LG> constexpr int row_step_blocks() { return sizeof(T) == 4 && LG == 9 ? kRowBlocks / 2 : kRowBlocks; }
 template <typename T, int LG>
 static size_t smem_for(int threads) { return sizeof(cplx<T>) * 2 * RowFft<T, LG>::M * (size_t)(threads / RowFft<T, LG>::TT); }
 // shared memory for the kernel's largest block, and a carveout that holds `blocks` of them and leaves the rest to L1: rows
@@ -411,7 +416,7 @@ static cudaError_t rfft_lg(const RowPtrs& p, int nf, cplx<T>* out, int64_t rows,
         }
     }
     const auto kern = k_rfft_reg<T, LG, false>;
-    const int th = threads_for<T, LG>(total), R = th / RowFft<T, LG>::TT;
+    const int th = threads_for<T, LG>(total, row_step_blocks<T, LG>()), R = th / RowFft<T, LG>::TT;
     const size_t smem = smem_for<T, LG>(th);
     const int64_t blocks = std::min<int64_t>((total + R - 1) / R, resident_grid((const void*)kern, th, smem));
     kern<<<(unsigned)blocks, th, smem, s>>>(p, out, (unsigned)rows, (unsigned)total, RowFft<T, LG>::table(t), t.twN);
@@ -435,7 +440,7 @@ static cudaError_t ampere_lg(cplx<T>* spec, const RowPtrsW& p, int64_t rows, int
                          : (wb ? k_ampere_irfft_reg<T, LG, false, true> : k_ampere_irfft_reg<T, LG, false, false>);
     cudaError_t e = room((const void*)kern, smem_for<T, LG>((row_threads<T, LG>())), row_blocks<T, LG>());
     if (e != cudaSuccess) return e;
-    const int th = threads_for<T, LG>(rows * 6), R = th / RowFft<T, LG>::TT;
+    const int th = threads_for<T, LG>(rows * 6, row_step_blocks<T, LG>()), R = th / RowFft<T, LG>::TT;
     kern<<<(unsigned)((rows + R - 1) / R * 6), th, smem_for<T, LG>(th), s>>>(spec, p, (unsigned)rows, n2, n3, RowFft<T, LG>::table(t), t.twN, t.S, t.cj1, t.cj,
                                                                             a2, a3);
     return cudaGetLastError();
