@@ -48,15 +48,15 @@ static hyb_status noalloc_address(void** out) {
 
 // The tables of one call, written on the device into the head of the static array (no
 // host copies): corr[nk] (Eq. currentcorrection, from the same mode_k the grid tables use),
-// twS[M] (stockham_twiddles), twN[M] = W_n1^j and twM[M] = W_M^j: every table the row
-// transforms may read; FP64, rounded once.
+// twS[M] (stockham_twiddles), twN[M] = W_n1^j and, where twM is given, twM[M] = W_M^j: every table
+// the row transforms may read; FP64, rounded once.
 template <typename T>
 __global__ void k_noalloc_tables(T* __restrict__ corr, cplx<T>* __restrict__ twS, cplx<T>* __restrict__ twN,
                                  cplx<T>* __restrict__ twM, int n1, double dx1, int yee_mode, double kmod_l,
                                  double kmod_u, double kmod_max) {
     using C = cplx<T>;
     const int M = n1 / 2, nk = M + 1;
-    const int total = nk + 3 * M;
+    const int total = nk + (twM ? 3 : 2) * M;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         if (i < nk) {
             corr[i] = (T)mode_corr(i, mode_k(i, n1, dx1, yee_mode, kmod_l, kmod_u, kmod_max));
@@ -86,9 +86,12 @@ static hyb_status run(const hyb_grid_desc& d, T* j1, cudaStream_t s) {
     using C = cplx<T>;
     const int n1 = d.n1, M = n1 / 2, nk = M + 1;
     const int64_t rows = (int64_t)d.n2 * (d.dims == 3 ? d.n3 : 1);
-    // tables in the head of the array: corr[nk], twS[M], twN[M], twM[M]; then row blocks
+    // tables in the head of the array: corr[nk], twS[M], twN[M] and, for the short FP64 rows whose transform
+    // reads it (rowfft.cuh), twM[M]; then row blocks.  (Room for it at any n1 cost 8192-point FP64 rows one of 125 rows
+    // per block: 500 rows in five blocks, 512 -> 636 us.)
+    const bool with_twM = sizeof(T) == 8 && n1 <= 256;
     auto up256 = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t tab_bytes = up256(sizeof(T) * nk) + up256(sizeof(C) * M) * 3;
+    const size_t tab_bytes = up256(sizeof(T) * nk) + up256(sizeof(C) * M) * (with_twM ? 3 : 2);
     const size_t row_bytes = sizeof(C) * (size_t)nk;
     if (tab_bytes + row_bytes > kNoallocBytes) {
         set_error("hyb_correct_current_noalloc: n1 = %d needs %zu bytes of working memory, more than the %zu available",
@@ -102,14 +105,14 @@ static hyb_status run(const hyb_grid_desc& d, T* j1, cudaStream_t s) {
     T* corr = (T*)p;
     C* twS = (C*)(p + up256(sizeof(T) * nk));
     C* twN = (C*)(p + up256(sizeof(T) * nk) + up256(sizeof(C) * M));
-    C* twM = (C*)(p + up256(sizeof(T) * nk) + 2 * up256(sizeof(C) * M));
+    C* twM = with_twM ? (C*)(p + up256(sizeof(T) * nk) + 2 * up256(sizeof(C) * M)) : nullptr;
     C* spec = (C*)(p + tab_bytes);
     const int64_t rows_per_block = (int64_t)((kNoallocBytes - tab_bytes) / row_bytes);
 
     // every table entry is rewritten, so an earlier call's tables (other n1, dx1 or mode
     // switches) leave nothing behind; stream-ordered before the transforms that read them
     {
-        const int total = nk + 3 * M;
+        const int total = nk + (with_twM ? 3 : 2) * M;
         k_noalloc_tables<T><<<(total + 255) / 256, 256, 0, s>>>(corr, twS, twN, twM, n1, d.dx1, d.yee_mode, d.kmod_l,
                                                                d.kmod_u, d.kmod_max);
         HYB_CUDA_TRY(cudaGetLastError());
